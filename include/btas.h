@@ -282,12 +282,21 @@ btas_status btas_mul(int semiring, int dtype, int64_t n, const void *x, const vo
  * D : n x n int32 output; D == W (in place) is allowed, any other overlap is
  *     not.
  * btas_apsp checks the domain on the device (one synchronisation of
- * `stream`; BTAS_ERR_ARG if violated), enables the early exit, and picks the
- * exact representation per squaring as btas_apsp_ex does without FORCE
- * flags.
+ * `stream`; BTAS_ERR_ARG if violated).  It asks for the distances alone, and so
+ * does btas_apsp_ex with flags == BTAS_APSP_EARLY_EXIT and no out-parameter: from
+ * n = 49 up to 14400 such a call relaxes W's edges, sorted by weight, until
+ * nothing changes, 8 targets per block (every block works on its own, so no
+ * squaring is computed); blocks that run far longer than random graphs take
+ * (paths of very many edges) give up.  The same D then comes from the squarings
+ * below n = 2048 and from blocked Floyd-Warshall from there on, which also takes
+ * n > 14400.  Scratch for the relaxation: about 8 n min(n, 512) bytes, and n * n
+ * words more in place (D == W).  Other calls, and all of them while the
+ * environment sets any BTAS_APSP_* or BTAS_MID_* switch (BTAS_APSP_NO_RELAX=1 does
+ * nothing else), run the squarings, with the early exit and the exact
+ * representation per squaring as btas_apsp_ex describes.
  *
- * Execution by size (same results and the same squarings count in every
- * regime; FORCE_U16 / FORCE_CARRIER always take the tiled path):
+ * Execution of the squarings by size (same results and the same squarings
+ * count in every regime; FORCE_U16 / FORCE_CARRIER always take the tiled path):
  *   n <= 64         one thread block holds D in shared memory and runs the
  *                   domain check and every squaring (int32): one launch, one
  *                   read-back;
@@ -314,7 +323,7 @@ btas_status btas_mul(int semiring, int dtype, int64_t n, const void *x, const vo
  * BTAS_APSP_SMALL_MAX_N=m (0 .. 128) and BTAS_APSP_MID_MAX_N=m (0 .. 4096) in
  * the environment move the two boundaries (the latter as a plain size
  * limit); BTAS_APSP_NO_SMALL=1 / BTAS_APSP_NO_MID=1 send the first two
- * regimes to the tiled path.  The cooperative regime keeps, per calling host
+ * regimes to the tiled path.  The cooperative regime and the relaxation keep, per calling host
  * thread, 64 bytes of mapped host memory for its status words and (for
  * workspaces up to 32 MiB, on the first device the thread uses) a 32 MiB
  * device workspace, both released when the thread exits; other workspace

@@ -13,6 +13,7 @@
 #include <vector>
 
 #include <nvtx3/nvToolsExt.h>
+#include <unistd.h>
 
 #include "common.cuh"
 #include "kernels.h"
@@ -748,6 +749,15 @@ struct MidThreadState {
 };
 constexpr size_t kMidCachedWs = size_t(32) << 20;
 
+// Whether the environment names a regime of the squarings (any BTAS_APSP_* or
+// BTAS_MID_* switch, BTAS_APSP_NO_RELAX=1 among them): btas_apsp then keeps to
+// them.
+static bool apsp_regime_pinned() {
+    for (char **e = environ; e && *e; ++e)
+        if (!strncmp(*e, "BTAS_APSP_", 10) || !strncmp(*e, "BTAS_MID_", 9)) return true;
+    return false;
+}
+
 static MidThreadState &thread_state() {
     thread_local MidThreadState ts;
     if (!ts.mbox_tried) {
@@ -763,28 +773,76 @@ static MidThreadState &thread_state() {
     return ts;
 }
 
+// The thread's cached workspace (up to kMidCachedWs, on the first device
+// used), else one from the pool in `ws`.
+static cudaError_t thread_workspace(MidThreadState &ts, size_t need, Workspace &ws, void **out) {
+    int dev = 0;
+    cudaError_t e = cudaGetDevice(&dev);
+    if (e != cudaSuccess) return e;
+    if (need > kMidCachedWs || (ts.ws_dev >= 0 && ts.ws_dev != dev)) {
+        e = ws.alloc(need);
+        *out = ws.p;
+        return e;
+    }
+    if (ts.ws_bytes < need) {
+        if ((e = cudaMalloc(&ts.ws, kMidCachedWs)) != cudaSuccess) return e;
+        ts.ws_bytes = kMidCachedWs;
+        ts.ws_dev = dev;
+    }
+    *out = ts.ws;
+    return cudaSuccess;
+}
+
+// Relaxation over sorted edge lists (relax.cu).  In place (D == W) it reads a
+// copy of W, left in copy_ws.  Returns a btas_status, or
+// kRelaxGaveUpFallback: D may then hold some columns already, and the caller
+// solves W (the copy, if there is one) another way.
+constexpr int kRelaxGaveUpFallback = -1;
+constexpr int64_t kRelaxMinN = 48;  // up to it the one-block kernel is as fast (n = 48: 34-38 us per call both)
+
+static int apsp_relax_solve(int64_t n, const int32_t *W, int32_t *D, Workspace &copy_ws, cudaStream_t st) {
+    MidThreadState &ts = thread_state();
+    if (!ts.mbox) return kRelaxGaveUpFallback;
+    Workspace ws(st);
+    void *wsp = nullptr;
+    BTAS_CUDA(thread_workspace(ts, relax_workspace(n), ws, &wsp), "workspace alloc");
+    if (W == D) {
+        const size_t bytes = (size_t)n * (size_t)n * 4;
+        BTAS_CUDA(copy_ws.alloc(bytes), "workspace alloc");
+        BTAS_CUDA(cudaMemcpyAsync(copy_ws.p, W, bytes, cudaMemcpyDeviceToDevice, st), "copy");
+        W = static_cast<const int32_t *>(copy_ws.p);
+    }
+    volatile int *out = ts.mbox;
+    out[0] = 0;  // written by the last block as the solve ends
+    BTAS_CUDA(launch_relax(W, n, (int)n, D, n, wsp, ts.mbox, st), "relaxation");
+    BTAS_CUDA(cudaStreamSynchronize(st), "relaxation");
+    const int outcome = out[0], bad = out[1], deg = out[2], wide = out[3];
+    if (outcome == kRelaxBad)
+        return fail(BTAS_ERR_ARG,
+                    "btas_apsp: %d entries outside the domain (negative weight, weight > 2^28, or non-zero "
+                    "diagonal)",
+                    bad);
+    if (outcome != kRelaxDone && outcome != kRelaxGaveUp)
+        return fail((btas_status)BTAS_ERR_INTERNAL, "btas_apsp: the relaxation left no outcome");
+    // the log names the size regime of the squarings that this replaces
+    const bool dense = n > apsp_mid_max_n() && n <= kMidSparseMaxN && deg > apsp_mid_list_cap(n);
+    if (dense)
+        log_event("apsp n=%lld: too dense for the cooperative kernel's edge lists (%d edges in a row)", (long long)n,
+                  deg);
+    log_event("apsp n=%lld: %s range, relaxation over sorted edge lists in %s bits%s", (long long)n,
+              n <= apsp_small_limit() ? "one-block kernel"
+              : !dense && n <= kMidSparseMaxN ? "cooperative kernel" : "tiled kernels",
+              wide ? "32" : "16", outcome == kRelaxDone ? "" : ", given up");
+    return outcome == kRelaxDone ? BTAS_OK : kRelaxGaveUpFallback;
+}
+
 static int apsp_mid_solve(int64_t n, const int32_t *W, int32_t *D, int S, bool early, bool packed_ok,
                           int *squarings_done, int64_t *bound_out, int *path_out, cudaStream_t st) {
     MidThreadState &ts = thread_state();
-    int dev = 0;
-    BTAS_CUDA(cudaGetDevice(&dev), "device");
     const size_t need = apsp_mid_workspace(n, S);
     Workspace ws(st);
     void *wsp = nullptr;
-    if (need <= kMidCachedWs && (ts.ws_dev < 0 || ts.ws_dev == dev)) {
-        if (ts.ws_bytes < need) {
-            if (ts.ws) cudaFree(ts.ws);
-            ts.ws = nullptr;
-            ts.ws_bytes = 0;
-            BTAS_CUDA(cudaMalloc(&ts.ws, kMidCachedWs), "workspace alloc");
-            ts.ws_bytes = kMidCachedWs;
-            ts.ws_dev = dev;
-        }
-        wsp = ts.ws;
-    } else {
-        BTAS_CUDA(ws.alloc(need), "workspace alloc");
-        wsp = ws.p;
-    }
+    BTAS_CUDA(thread_workspace(ts, need, ws, &wsp), "workspace alloc");
     // the status words inside the workspace: zeroed by the launch
     int *info = apsp_mid_info(wsp, n);
     if (ts.mbox) ts.mbox[3] = -1;  // overwritten by the kernel as it ends
@@ -845,6 +903,29 @@ static btas_status apsp_impl(int64_t n, const int32_t *W, int32_t *D, int flags,
     const int S = btas_apsp_squarings(n);
     const bool early = (flags & BTAS_APSP_EARLY_EXIT) != 0;
     const size_t nn = (size_t)n * (size_t)n;
+
+    // A call that asks for the distances alone: relaxation over sorted edge
+    // lists, and blocked Floyd-Warshall where that is given up or does not
+    // reach (from n = 2048; below it the squarings are as fast, 1.4-2.2 ms
+    // against 1.6-2.2 ms).  Calls that ask for facts of the squaring
+    // sequence (its length, its representations) run it.
+    Workspace copy_ws(st);
+    if (!squarings_done && !bound_out && !path_out && flags == BTAS_APSP_EARLY_EXIT && n > kRelaxMinN &&
+        !apsp_regime_pinned()) {
+        if (n <= relax_max_n()) {
+            const int r = apsp_relax_solve(n, W, D, copy_ws, st);
+            if (r != kRelaxGaveUpFallback) return static_cast<btas_status>(r);
+            if (copy_ws.p) W = static_cast<const int32_t *>(copy_ws.p);
+        }
+        if (n >= 2048) {
+            const btas_status r = btas_apsp_fw(n, W, D, st);
+            if (r != BTAS_OK) return r;
+            // Floyd-Warshall clamps in its third phase only
+            BTAS_CUDA(launch_clamp(D, nn, st), "clamp");
+            log_event("apsp n=%lld: tiled kernels range, blocked Floyd-Warshall", (long long)n);
+            return BTAS_OK;
+        }
+    }
 
     // small graphs: the whole solve in one thread block (one launch, one
     // read-back) on the int32 arithmetic; BTAS_APSP_NO_SMALL=1 disables it

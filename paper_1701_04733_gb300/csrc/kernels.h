@@ -171,6 +171,23 @@ cudaError_t launch_apsp_mid(const int *W, long long ldw, int n, int S, bool earl
                             long long ldd, void *ws, size_t ws_bytes, int *info, cudaStream_t st,
                             int *mailbox = nullptr, bool bail_dense = false);
 
+// ---- APSP by relaxation over sorted edge lists (relax.cu), n <=
+// relax_max_n().  Two launches, on `st`; D must not overlap W.  ws:
+// relax_workspace(n) bytes, not initialised.  out: 4 host-mapped words, written
+// as the solve ends: [0] a RelaxOutcome, [1] entries of W outside the domain (D
+// is then not written), [2] most edges of a row, [3] whether 32 bits were
+// needed.  kRelaxGaveUp: some block ran longer than the budget that such
+// graphs are worth (paths of very many edges, or long rows of equal weights);
+// some columns of D may be written.  BTAS_RELAX_BUDGET=cycles overrides the
+// budget (tests).
+enum RelaxOutcome { kRelaxDone = 1, kRelaxBad = 2, kRelaxGaveUp = 3 };
+size_t relax_workspace(long long n);
+int relax_max_n();
+cudaError_t launch_relax(const int *W, long long ldw, int n, int *D, long long ldd, void *ws, int *out,
+                         cudaStream_t st);
+// Entries from INF - 2^28 on become INF, as the squarings leave them.
+cudaError_t launch_clamp(int *D, size_t count, cudaStream_t st);
+
 // ---- blocked Floyd-Warshall (fw.cu): phases 1 and 2 of pivot block kb
 // pmax (optional): atomicMax of the largest finite value the phases store
 // (the pivot row and column panels).

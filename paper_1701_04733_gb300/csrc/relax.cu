@@ -1,0 +1,242 @@
+// APSP by relaxation over sorted edge lists, many targets at a time: what
+// btas_apsp runs when the caller wants the distances alone.
+//
+// Squaring (Sec. III) computes n^3 terms several times over, and nearly all of
+// them are sums of two long paths that a third one undercuts.  Bellman-Ford
+// over W's edges computes far fewer, and every block can solve a few targets by
+// itself, without a grid barrier: 16 bytes per vertex hold the distances to 8
+// targets in 16 bits (or 4 in 32), which fits shared memory up to n = 14400.
+// One edge is then one 16-byte load and 4 DPX add-mins for 8 terms.
+//
+// What makes it short is the order of the edges.  Each row's list is sorted by
+// weight, and an edge of weight w cannot start a better path of two or more
+// edges unless w plus the lightest weight of all stays below the largest of the
+// vertex's current distances; so a sweep reads a row's list up to that bound
+// only, about 3 chunks of 4 edges on random graphs, whatever their density.
+// The same bound makes a list of the lightest edges enough on dense graphs; the
+// rare row that needs more is read from W.  The first two sweeps also leave
+// edges of 4 or more times the row's lightest weight for later (n = 8192, p =
+// 0.01: 3.93 -> 3.32 ms; the same at p = 1).
+//
+// Sums of non-negative weights reach one fixpoint in any order, so the result is
+// that of the squarings bit for bit; only the number of squarings is not known.
+//
+// Measured (GB300, us per call with its synchronisation, before -> after):
+//   n = 128 (complete), 256 (p = 0.1):              60 -> 41, 60 -> 48
+//   n = 512, 1024 (p = 0.1, w <= 100):              98 -> 65, 288 -> 100
+//   n = 2048 (p = 0.1 / complete, w <= 10^6):       1416 -> 193 / 3279 -> 280
+//   n = 2999 (p = 0.5, w <= 10^6):                  10400 -> 555
+//   n = 4096 (p = 0.05, w <= 7 / p = 0.01, w <= 10^6): 6260 -> 610 / 16700 -> 1610
+//   n = 8192 (p = 0.01, w <= 1000 / complete, w <= 100): 93600 -> 3320 / 47000 -> 4020
+// The sweeps are bound by shared memory: ncu at n = 4096 (p = 0.01) has the
+// L1/shared pipe 92 % busy while SMs are active, 43 % of its cycles bank
+// conflicts of the random 16-byte rows (8 lanes on 8 bank groups).  Wider rows
+// conflict less but do not fit; ordering a chunk's 4 edges by bank gains 5 %.
+// The last wave costs 15-30 % where n / 8 blocks are few per SM.
+#include <algorithm>
+#include <cstdlib>
+#include <type_traits>
+
+#include "common.cuh"
+#include "kernels.h"
+#include "relax.cuh"
+
+namespace btas {
+namespace {
+
+using relax::Lists;
+using relax::RowStats;
+
+constexpr int kListWarps = 8;               // rows of a block of the list kernel
+constexpr int kSolveSmem = 225 * 1024;       // most dynamic shared memory of the solve kernel
+enum Ctl { kAbort = 0, kWide = 1, kDone = 2 };  // control words, cleared by the list kernel
+
+struct RelaxArgs {
+    const int *W;
+    long long ldw;
+    int n;
+    Lists lists;
+    RowStats *stats;  // one per block of the list kernel
+    int *ctl;
+    int *D;
+    long long ldd;
+    int *out;  // host-mapped words (see kernels.h)
+    int halves;  // 2: a second block per 8 targets takes 4 of them where 32 bits are needed from the start
+};
+
+__global__ void __launch_bounds__(kListWarps * 32) relax_lists_kernel(const RelaxArgs a) {
+    __shared__ unsigned long long buf[kListWarps][relax::kCap];
+    __shared__ int hist[kListWarps][256];
+    __shared__ RowStats s_st[kListWarps];
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int row = blockIdx.x * kListWarps + warp;
+    if (blockIdx.x == 0 && threadIdx.x < 3) a.ctl[threadIdx.x] = 0;
+    RowStats st{0, 0, kInfI32, 0, 0, 0.0f};
+    if (row < a.n) st = relax::build_row(a.W, a.ldw, a.n, row, a.lists, buf[warp], hist[warp], lane);
+    if (lane == 0) s_st[warp] = st;
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        for (int i = 1; i < kListWarps; ++i) {
+            const RowStats &o = s_st[i];
+            st.bad += o.bad;
+            st.maxw = max(st.maxw, o.maxw);
+            st.minw = min(st.minw, o.minw);
+            st.deg = max(st.deg, o.deg);
+            st.far |= o.far;
+            st.light += o.light;
+        }
+        a.stats[blockIdx.x] = st;
+    }
+}
+
+template <int G, int MAXT>
+__global__ void __launch_bounds__(MAXT) relax_solve_kernel(const RelaxArgs a) {
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    uint4 *Y = reinterpret_cast<uint4 *>(smem_raw);
+    __shared__ int s_abort, s_wide;
+    __shared__ RowStats s_st;
+    const long long t0 = clock64();
+    const int n = a.n, tid = threadIdx.x;
+    const int groups = (n + 7) / 8, part = blockIdx.x >= groups ? 1 : 0;  // the second parts on SMs of their own
+    const int j0 = (blockIdx.x - part * groups) * 8;
+    if (tid == 0) s_st = RowStats{0, 0, kInfI32, 0, 0, 0.0f};
+    if (part == 0) relax::load_columns<true>(a.W, a.ldw, n, Y, j0);  // needs no lists
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+    __syncthreads();
+    const int nst = (n + kListWarps - 1) / kListWarps;
+    RowStats st{0, 0, kInfI32, 0, 0, 0.0f};
+    for (int i = tid; i < nst; i += blockDim.x) {
+        const RowStats o = a.stats[i];
+        st.bad += o.bad;
+        st.maxw = max(st.maxw, o.maxw);
+        st.minw = min(st.minw, o.minw);
+        st.deg = max(st.deg, o.deg);
+        st.far |= o.far;
+        st.light += o.light;
+    }
+    if (tid < nst) {
+        if (st.bad) atomicAdd(&s_st.bad, st.bad);
+        atomicMax(&s_st.maxw, st.maxw);
+        atomicMin(&s_st.minw, st.minw);
+        atomicMax(&s_st.deg, st.deg);
+        if (st.far) atomicOr(&s_st.far, 1);
+        atomicAdd(&s_st.light, st.light);
+    }
+    if (tid == 0) {
+        s_abort = *(volatile int *)(a.ctl + kAbort);
+        s_wide = *(volatile int *)(a.ctl + kWide);
+    }
+    __syncthreads();
+    st = s_st;
+    const bool wide_first = st.far != 0 || relax::expects_wide(n, st.light);  // the same in every block
+    if (st.bad == 0 && s_abort == 0) {
+        bool wide = wide_first || s_wide != 0;
+        auto give_up = [&]() {
+            if (*(volatile int *)(a.ctl + kAbort) != 0) return true;
+            if (clock64() - t0 <= (wide ? 2 : 1) * a.lists.budget) return false;
+            a.ctl[kAbort] = 1;
+            return true;
+        };
+        if (part == 0 && !wide && relax::solve<true, G>(a.W, a.ldw, n, a.lists, Y, st.minw, give_up)) {
+            wide = !relax::fits16(Y, n, st.maxw);
+            if (!wide) relax::store_columns<true>(a.D, a.ldd, n, Y, j0);
+            else if (tid == 0) a.ctl[kWide] = 1;
+        }
+        // in 32 bits, 4 targets at a time
+        const bool split = wide_first && a.halves == 2;
+        if (wide && (part == 0 || split)) {
+            for (int h = 4 * part; h < (split ? 4 * part + 4 : 8) && j0 + h < n; h += 4) {
+                __syncthreads();
+                relax::load_columns<false>(a.W, a.ldw, n, Y, j0 + h);
+                __syncthreads();
+                if (!relax::solve<false, G>(a.W, a.ldw, n, a.lists, Y, st.minw, give_up)) break;
+                relax::store_columns<false>(a.D, a.ldd, n, Y, j0 + h);
+            }
+        }
+    }
+    __syncthreads();
+    if (tid == 0) {
+        __threadfence();
+        if (atomicAdd(a.ctl + kDone, 1) == (int)gridDim.x - 1) {  // the last block tells the host
+            __threadfence();
+            a.out[1] = st.bad;
+            a.out[2] = st.deg;
+            a.out[3] = *(volatile int *)(a.ctl + kWide) | st.far;
+            a.out[0] = st.bad ? kRelaxBad : *(volatile int *)(a.ctl + kAbort) ? kRelaxGaveUp : kRelaxDone;
+            __threadfence_system();
+        }
+    }
+}
+
+__global__ void clamp_kernel(int *D, size_t count) {
+    for (size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x; i < count; i += (size_t)gridDim.x * blockDim.x)
+        if (D[i] >= kClampI32) D[i] = kInfI32;
+}
+
+size_t align256(size_t v) { return (v + 255) & ~size_t(255); }
+}  // namespace
+
+cudaError_t launch_clamp(int *D, size_t count, cudaStream_t st) {
+    clamp_kernel<<<(unsigned)std::min<size_t>((count + 255) / 256, 152 * 8), 256, 0, st>>>(D, count);
+    note_launch();
+    return cudaGetLastError();
+}
+
+int relax_max_n() { return kSolveSmem / 16; }
+
+size_t relax_workspace(long long n) {
+    const size_t rows = (size_t)((n + 31) & ~31LL);
+    return 256 + align256((size_t)((n + kListWarps - 1) / kListWarps) * sizeof(RowStats)) + align256(rows * 4) +
+           relax::list_words(n) * 8;
+}
+
+cudaError_t launch_relax(const int *W, long long ldw, int n, int *D, long long ldd, void *ws, int *out,
+                         cudaStream_t st) {
+    const size_t rows = (size_t)((n + 31) & ~31);
+    const int blocks = (n + kListWarps - 1) / kListWarps;
+    char *p = static_cast<char *>(ws);
+    RelaxArgs a{};
+    a.W = W;
+    a.ldw = ldw;
+    a.n = n;
+    a.D = D;
+    a.ldd = ldd;
+    a.out = out;
+    const char *bud = getenv("BTAS_RELAX_BUDGET");
+    a.lists.budget = bud && *bud ? atoll(bud) : relax::budget_cycles(n);
+    a.ctl = reinterpret_cast<int *>(p);
+    a.stats = reinterpret_cast<RowStats *>(p += 256);
+    a.lists.next = reinterpret_cast<int *>(p += align256(blocks * sizeof(RowStats)));
+    a.lists.edges = reinterpret_cast<uint4 *>(p += align256(rows * 4));
+    a.lists.wide = reinterpret_cast<int4 *>(p + relax::list_words(n) * 4);
+    a.lists.chunks = relax::list_chunks(n);
+    // Two blocks share 8 targets in 32 bits while one wave holds them all (n =
+    // 1024, w <= 10^6, p = 0.5: 283 -> 158 us per call).
+    a.halves = n <= 1216 ? 2 : 1;
+    relax_lists_kernel<<<blocks, kListWarps * 32, 0, st>>>(a);
+    note_launch();
+    // Two lanes per vertex where one would leave warps idle (n <= 256); 512
+    // threads while two blocks fit an SM (n = 4096, p = 0.01: 1118 us with 1024
+    // threads, 1060 with 512), 1024 beyond (n = 8192: 3662 us against 3779).
+    const int G = n <= 256 ? 2 : 1, maxt = n > 7000 ? 1024 : 512;
+    void (*kern)(const RelaxArgs) = G == 2 ? relax_solve_kernel<2, 512>
+                                    : maxt == 512 ? relax_solve_kernel<1, 512> : relax_solve_kernel<1, 1024>;
+    cudaError_t e = set_smem_once(reinterpret_cast<const void *>(kern), kSolveSmem);
+    if (e != cudaSuccess) return e;
+    cudaLaunchConfig_t cfg{};
+    cfg.gridDim = dim3((n + 7) / 8 * a.halves);
+    cfg.blockDim = dim3(std::min(maxt, (n * G + 31) / 32 * 32));
+    cfg.dynamicSmemBytes = (size_t)n * 16;
+    cfg.stream = st;
+    cudaLaunchAttribute at{};
+    at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at.val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = &at;
+    cfg.numAttrs = 1;
+    e = cudaLaunchKernelEx(&cfg, kern, a);
+    if (e == cudaSuccess) note_launch();
+    return e;
+}
+
+}  // namespace btas

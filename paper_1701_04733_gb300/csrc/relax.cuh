@@ -1,0 +1,565 @@
+// Shortest paths to a few targets at a time, by relaxation over edge lists
+// sorted by weight (relax.cu describes the method; the batched launch uses the
+// same pieces).
+//
+// Lists.  Row v's list holds its edges (v, k), lightest first, 4 to a 16-byte
+// chunk, each edge as (w << 16) | k with w saturated at 0x7FFF, and the same
+// edges' full weights in a second array.  Chunk c of rows 32 r .. 32 r + 31 is
+// contiguous, so a warp that reads chunk c of 32 rows reads 512 bytes.  A list
+// shorter than the capacity ends with chunks of pads (w = 0x7FFF, INF).  A row
+// with more edges than the capacity keeps its lightest ones; next[v] is then a
+// lower bound of the weights left out (INF: none).
+#pragma once
+
+#include <type_traits>
+
+#include "common.cuh"
+
+namespace btas {
+namespace relax {
+
+constexpr int kCap = 512;          // most edges a list holds
+__host__ __device__ constexpr int list_chunks(long long n) { return (int)((n < kCap ? n : kCap) + 3) / 4; }
+__host__ __device__ constexpr size_t list_words(long long n) {  // of Lists::edges, and of Lists::wide
+    return (size_t)((n + 31) / 32) * 32 * list_chunks(n) * 4;
+}
+constexpr int kTruncTarget = 256;  // a longer row keeps at most about this many
+constexpr int kPadChunks = 2;      // chunks of pads after a list: one per lane that reads it (solve's G)
+constexpr int kEarlySweeps = 2, kEarlyChunks = 2;  // solve's first sweeps
+constexpr int kSample = 1024;      // entries the first guess of a long row's cutoff is taken from
+
+struct Lists {
+    uint4 *edges;  // [ceil(n / 32)][chunks][32]
+    int4 *wide;    // the weights in 32 bits, same places
+    int *next;     // n words
+    int chunks;    // capacity / 4
+    long long budget;  // clock cycles after which a block gives up
+};
+
+// What building the lists of some rows finds out.
+struct RowStats {
+    int bad;    // entries outside the domain
+    int maxw;   // largest weight
+    int minw;   // smallest off-diagonal weight (INF: no edge)
+    int deg;    // most edges of a row
+    int far;    // 1: some row's lightest edge does not fit 16 bits
+    float light;  // sum of the rows' lightest weights
+};
+
+// Clock cycles a block of 8 targets is worth: about twice what the slowest
+// random graphs take (n = 256 ... 8192, edge probability 0.01 ... 1).
+__host__ __device__ constexpr long long budget_cycles(long long n) {
+    return 30000 + 200 * n + (n / 8 < 300 ? n / 8 : 300) * n;
+}
+
+// Whether 16 bits are likely to be too few: the largest distance of a random
+// graph is about 3 ln n times the mean of its rows' lightest weights.
+__device__ __forceinline__ bool expects_wide(int n, float light) {
+    return 3.0f * __logf((float)n) * light >= (float)n * BTAS_INF_U16;
+}
+
+__device__ __forceinline__ size_t chunk_at(const Lists &l, int row, int c) {
+    return ((size_t)(row >> 5) * l.chunks + c) * 32 + (row & 31);
+}
+
+// --------------------------------------------------------------- sorting
+template <class Key>
+__device__ __forceinline__ void order(Key &a, Key &b, bool up) {
+    const Key lo = min(a, b), hi = max(a, b);
+    a = up ? lo : hi;
+    b = up ? hi : lo;
+}
+
+// The stages of a bitonic merge inside one lane's E consecutive elements.
+template <class Key, int E>
+__device__ __forceinline__ void merge_lane(Key (&key)[E], int first, bool up) {
+#pragma unroll
+    for (int j = E / 2; j > 0; j >>= 1)
+        if (j <= first) {
+#pragma unroll
+            for (int e = 0; e < E; ++e)
+                if ((e & j) == 0) order(key[e], key[e | j], up);
+        }
+}
+
+// Ascending bitonic sort of 32 E keys, element lane * E + e in key[e]: the
+// short exchanges stay in registers, the others are one shuffle per key.
+template <class Key, int E>
+__device__ __forceinline__ void sort_warp(Key (&key)[E], int lane) {
+#pragma unroll
+    for (int k = 2; k < E; k <<= 1)  // runs of k inside the lane, alternating directions
+#pragma unroll
+        for (int j = k >> 1; j > 0; j >>= 1)
+#pragma unroll
+            for (int e = 0; e < E; ++e)
+                if ((e & j) == 0) order(key[e], key[e | j], (e & k) == 0);
+    for (int k = E; k <= 32 * E; k <<= 1) {
+        const bool up = ((lane * E) & k) == 0;
+        for (int j = k >> 1; j >= E; j >>= 1) {
+            const int d = j / E;
+            const bool low = ((lane & d) == 0) == up;
+#pragma unroll
+            for (int e = 0; e < E; ++e) {
+                const Key o = __shfl_xor_sync(0xffffffffu, key[e], d);
+                key[e] = low ? min(key[e], o) : max(key[e], o);
+            }
+        }
+        merge_lane<Key, E>(key, k >> 1, up);
+    }
+}
+
+// cnt <= 32 E keys (w << 32 | k) in `buf` -> the row's chunks, lightest first.
+// Key32: (w - base) << 16 | k, where the weights span less than 2^16 - 1.
+template <bool Key32, int E>
+__device__ __forceinline__ void sort_and_store(const unsigned long long *buf, int cnt, int row, int base,
+                                               const Lists &l, int lane) {
+    using Key = typename std::conditional<Key32, unsigned, unsigned long long>::type;
+    Key key[E];
+#pragma unroll
+    for (int e = 0; e < E; ++e) {
+        const int i = lane * E + e;
+        if (Key32) {
+            const unsigned long long b = i < cnt ? buf[i] : 0;
+            key[e] = i < cnt ? (Key)((((unsigned)(b >> 32) - (unsigned)base) << 16) | (unsigned)b) : ~(Key)0;
+        } else {
+            key[e] = i < cnt ? (Key)buf[i] : ~(Key)0;
+        }
+    }
+    sort_warp<Key, E>(key, lane);
+    // the list's chunks and its pads; a full list has none
+    const int chunks = min(l.chunks, (cnt + 3) / 4 + kPadChunks);
+#pragma unroll
+    for (int q = 0; q < E / 4; ++q) {
+        const int c = lane * (E / 4) + q;
+        if (c >= chunks) continue;
+        unsigned p[4];
+        int w[4];
+#pragma unroll
+        for (int e = 0; e < 4; ++e) {
+            const Key kk = key[4 * q + e];
+            const bool edge = 4 * c + e < cnt;
+            w[e] = !edge ? kInfI32 : Key32 ? (int)((unsigned)kk >> 16) + base : (int)((unsigned long long)kk >> 32);
+            p[e] = ((unsigned)min(w[e], BTAS_INF_U16) << 16) | (edge ? (unsigned)kk & 0xFFFFu : (unsigned)row);
+        }
+        l.edges[chunk_at(l, row, c)] = make_uint4(p[0], p[1], p[2], p[3]);
+        l.wide[chunk_at(l, row, c)] = make_int4(w[0], w[1], w[2], w[3]);
+    }
+    // pads beyond the sorted block (cnt close to 32 E)
+    const int c = 8 * E + lane;
+    if (c < chunks) {
+        const unsigned p = ((unsigned)BTAS_INF_U16 << 16) | (unsigned)row;
+        l.edges[chunk_at(l, row, c)] = make_uint4(p, p, p, p);
+        l.wide[chunk_at(l, row, c)] = make_int4(kInfI32, kInfI32, kInfI32, kInfI32);
+    }
+}
+
+// A weight such that about `target` of the edges among the row's first m
+// entries are lighter (at most `target`; at least half of it unless weights
+// repeat too often: then ties is set and the edges at the cutoff weight
+// itself fill up the list).  Histograms of 256 equal bins of [lo, hi], refined
+// around the bin that does not fit.  `hist`: 256 words of the warp's own.
+__device__ __forceinline__ int select_cut(const int *wr, int row, int m, int target, int lo, int hi, int *hist,
+                                          int lane, bool &ties) {
+    int below = 0;  // edges lighter than lo
+    ties = false;
+    for (;;) {
+        const int sh = max(0, 24 - __clz(max(hi - lo, 1)));  // (hi - lo) >> sh <= 255
+        for (int b = lane; b < 256; b += 32) hist[b] = 0;
+        __syncwarp();
+        for (int j0 = 0; j0 < m; j0 += 128) {
+            int v[4];
+#pragma unroll
+            for (int u = 0; u < 4; ++u) {
+                const int j = j0 + 32 * u + lane;
+                v[u] = j < m && j != row ? __ldg(wr + j) : kInfI32;
+            }
+#pragma unroll
+            for (int u = 0; u < 4; ++u)
+                if (v[u] >= lo && v[u] <= hi) atomicAdd(hist + ((v[u] - lo) >> sh), 1);
+        }
+        __syncwarp();
+        int h[8], tot = 0;
+#pragma unroll
+        for (int b = 0; b < 8; ++b) {
+            h[b] = hist[lane * 8 + b];
+            tot += h[b];
+        }
+        int pre = tot;
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+            const int x = __shfl_up_sync(0xffffffffu, pre, o);
+            if (lane >= o) pre += x;
+        }
+        pre -= tot;  // edges in the bins of the lanes before this one
+        int fit = 0, kept = 0;  // bins, from the first, that fit together
+#pragma unroll
+        for (int b = 0; b < 8; ++b) {
+            pre += h[b];
+            if (below + pre <= target) {
+                ++fit;
+                kept = pre;
+            }
+        }
+        fit = __reduce_add_sync(0xffffffffu, fit);
+        kept = __reduce_max_sync(0xffffffffu, kept);
+        __syncwarp();
+        below += kept;
+        if (fit == 256) return hi + 1;
+        const int cut = lo + (fit << sh);
+        if (2 * below >= target) return cut;
+        if (sh == 0) {
+            ties = true;
+            return cut;
+        }
+        lo = cut;
+        hi = min(hi, cut + (1 << sh) - 1);
+    }
+}
+
+// One pass over row `row` of W by one warp: the domain check, the statistics,
+// and the edges lighter than `cut` (or as light, with ties) to buf, kCap of
+// them at most.  Returns how many there are; deg: all of the row's edges.
+__device__ __forceinline__ int scan_row(const int *wr, int n, int row, int cut, bool ties, unsigned long long *buf,
+                                        int lane, RowStats &st, int &mn, int &mx, int &deg) {
+    constexpr int U = 8;
+    const unsigned lt = (1u << lane) - 1u;
+    int cnt = 0;
+    deg = 0;
+    mn = kInfI32;
+    mx = 0;
+    int bad = 0;
+    for (int c0 = 0; c0 < n; c0 += 32 * U) {
+        int v[U];
+#pragma unroll
+        for (int u = 0; u < U; ++u) {
+            const int j = c0 + 32 * u + lane;
+            v[u] = j < n ? __ldg(wr + j) : kInfI32;
+        }
+#pragma unroll
+        for (int u = 0; u < U; ++u) {
+            const int j = c0 + 32 * u + lane;
+            const bool fin = (unsigned)v[u] <= (unsigned)BTAS_I32_FINITE_MAX;
+            bad += (!fin && v[u] != kInfI32) || (j == row && v[u] != 0);
+            const bool edge = fin && j != row;
+            deg += edge;
+            mx = max(mx, edge ? v[u] : 0);
+            mn = min(mn, edge ? v[u] : kInfI32);
+            const bool keep = edge && (v[u] < cut || (ties && v[u] == cut));
+            const unsigned m = __ballot_sync(0xffffffffu, keep);
+            const int q = cnt + __popc(m & lt);
+            if (keep && q < kCap) buf[q] = ((unsigned long long)(unsigned)v[u] << 32) | (unsigned)j;
+            cnt += __popc(m);
+        }
+    }
+    st.bad = __reduce_add_sync(0xffffffffu, bad);
+    deg = __reduce_add_sync(0xffffffffu, deg);
+    mx = __reduce_max_sync(0xffffffffu, mx);
+    mn = __reduce_min_sync(0xffffffffu, mn);
+    __syncwarp();
+    return cnt;
+}
+
+// Row `row`'s list, by one warp.  buf: kCap keys, hist: 256 words, both the
+// warp's own shared memory.
+__device__ __forceinline__ RowStats build_row(const int *W, long long ldw, int n, int row, const Lists &l,
+                                              unsigned long long *buf, int *hist, int lane) {
+    const int *wr = W + (long long)row * ldw;
+    const int cap = min(kCap, 4 * l.chunks);
+    RowStats st{};
+    int cut = kInfI32;
+    bool ties = false;
+    // A long row is read once: its first entries say whether it will overflow
+    // and, if so, about where to cut.
+    if (n >= 2 * kSample) {
+        int d = 0, mn = kInfI32, mx = 0;
+#pragma unroll 8
+        for (int j = lane; j < kSample; j += 32) {
+            const int v = __ldg(wr + j);
+            if ((unsigned)v <= (unsigned)BTAS_I32_FINITE_MAX && j != row) {
+                ++d;
+                mn = min(mn, v);
+                mx = max(mx, v);
+            }
+        }
+        d = __reduce_add_sync(0xffffffffu, d);
+        mn = __reduce_min_sync(0xffffffffu, mn);
+        mx = __reduce_max_sync(0xffffffffu, mx);
+        if ((long long)d * n > (long long)cap * kSample * 9 / 10)
+            cut = select_cut(wr, row, kSample, max(4, (int)((long long)kTruncTarget * kSample / n)), mn, mx, hist,
+                             lane, ties);
+        if (ties) cut = kInfI32, ties = false;
+    }
+    int mn, mx, deg;
+    int cnt = scan_row(wr, n, row, cut, ties, buf, lane, st, mn, mx, deg);
+    if (cnt > cap || (cnt < deg && cnt < 64)) {
+        cut = select_cut(wr, row, n, kTruncTarget, mn, mx, hist, lane, ties);
+        cnt = min(cap, scan_row(wr, n, row, cut, ties, buf, lane, st, mn, mx, deg));
+    }
+    if (lane == 0) l.next[row] = cnt < deg ? cut : kInfI32;
+    const bool k32 = (cnt < deg ? cut : mx) - mn < 0xFFFF;
+    if (cnt <= 128) {
+        if (k32) sort_and_store<true, 4>(buf, cnt, row, mn, l, lane);
+        else sort_and_store<false, 4>(buf, cnt, row, mn, l, lane);
+    } else {
+        if (k32) sort_and_store<true, 16>(buf, cnt, row, mn, l, lane);
+        else sort_and_store<false, 16>(buf, cnt, row, mn, l, lane);
+    }
+    st.maxw = mx;
+    st.minw = mn;
+    st.deg = deg;
+    st.far = deg > 0 && mn >= BTAS_INF_U16;
+    st.light = deg > 0 ? (float)mn : 0.0f;
+    return st;
+}
+
+// -------------------------------------------------------------- relaxing
+// Y[v] in shared memory: 16 bytes, the distances from v to 8 targets in 16
+// bits (0x7FFF: none known) or to 4 targets in 32.  Only the lanes of v's own
+// group write Y[v], and a stale read costs a further sweep and no more, so the
+// accesses of a sweep are relaxed ones.
+__device__ __forceinline__ uint4 lds_relaxed(const uint4 *p) {
+    uint4 v;
+    asm volatile("ld.relaxed.cta.shared.v4.b32 {%0, %1, %2, %3}, [%4];"
+                 : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w)
+                 : "r"(smem_u32(p))
+                 : "memory");
+    return v;
+}
+__device__ __forceinline__ void sts_relaxed(uint4 *p, uint4 v) {
+    asm volatile("st.relaxed.cta.shared.v4.b32 [%0], {%1, %2, %3, %4};" ::"r"(smem_u32(p)), "r"(v.x), "r"(v.y),
+                 "r"(v.z), "r"(v.w)
+                 : "memory");
+}
+template <bool U16>
+__device__ __forceinline__ int top(const uint4 &y) {
+    if (U16) {
+        const unsigned m = __vmaxu2(__vmaxu2(y.x, y.y), __vmaxu2(y.z, y.w));
+        return (int)max(m >> 16, m & 0xFFFFu);
+    }
+    return max(max((int)y.x, (int)y.y), max((int)y.z, (int)y.w));
+}
+// acc = min(acc, y + w); w: the weight in both halves with U16
+template <bool U16>
+__device__ __forceinline__ void relax4(uint4 &acc, const uint4 &y, unsigned w) {
+    if (U16) {
+        acc.x = u16x2_addmin(y.x, w, acc.x);
+        acc.y = u16x2_addmin(y.y, w, acc.y);
+        acc.z = u16x2_addmin(y.z, w, acc.z);
+        acc.w = u16x2_addmin(y.w, w, acc.w);
+    } else {
+        acc.x = (unsigned)__viaddmin_s32((int)y.x, (int)w, (int)acc.x);
+        acc.y = (unsigned)__viaddmin_s32((int)y.y, (int)w, (int)acc.y);
+        acc.z = (unsigned)__viaddmin_s32((int)y.z, (int)w, (int)acc.z);
+        acc.w = (unsigned)__viaddmin_s32((int)y.w, (int)w, (int)acc.w);
+    }
+}
+template <bool U16>
+__device__ __forceinline__ uint4 min4(const uint4 &a, const uint4 &b) {
+    if (U16) return make_uint4(__vminu2(a.x, b.x), __vminu2(a.y, b.y), __vminu2(a.z, b.z), __vminu2(a.w, b.w));
+    return make_uint4((unsigned)min((int)a.x, (int)b.x), (unsigned)min((int)a.y, (int)b.y),
+                      (unsigned)min((int)a.z, (int)b.z), (unsigned)min((int)a.w, (int)b.w));
+}
+__device__ __forceinline__ uint4 shfl_xor4(const uint4 &a, int o) {
+    return make_uint4(__shfl_xor_sync(0xffffffffu, a.x, o), __shfl_xor_sync(0xffffffffu, a.y, o),
+                      __shfl_xor_sync(0xffffffffu, a.z, o), __shfl_xor_sync(0xffffffffu, a.w, o));
+}
+__device__ __forceinline__ uint4 clamp4(const uint4 &v) {
+    return make_uint4((unsigned)clamp_i32<kMin>((int)v.x), (unsigned)clamp_i32<kMin>((int)v.y),
+                      (unsigned)clamp_i32<kMin>((int)v.z), (unsigned)clamp_i32<kMin>((int)v.w));
+}
+__device__ __forceinline__ bool differ(const uint4 &a, const uint4 &b) {
+    return ((a.x ^ b.x) | (a.y ^ b.y) | (a.z ^ b.z) | (a.w ^ b.w)) != 0;
+}
+
+template <bool U16>
+constexpr int targets() { return U16 ? 8 : 4; }
+
+// Columns [j0, j0 + targets) of W -> Y: the paths of one edge.
+template <bool U16>
+__device__ __forceinline__ void load_columns(const int *W, long long ldw, int n, uint4 *Y, int j0) {
+    constexpr int S = targets<U16>();
+    const bool vec = (ldw & 3) == 0 && (reinterpret_cast<uintptr_t>(W) & 15) == 0 && j0 + S <= n;
+    for (int v = threadIdx.x; v < n; v += blockDim.x) {
+        int x[S];
+        const int *p = W + (long long)v * ldw + j0;
+        if (vec) {
+#pragma unroll
+            for (int s = 0; s < S; s += 4) {
+                const int4 q = __ldg(reinterpret_cast<const int4 *>(p + s));
+                x[s] = q.x, x[s + 1] = q.y, x[s + 2] = q.z, x[s + 3] = q.w;
+            }
+        } else {
+#pragma unroll
+            for (int s = 0; s < S; ++s) x[s] = j0 + s < n ? __ldg(p + s) : 0;  // an absent target: nothing to lower
+        }
+        if constexpr (U16) {
+#pragma unroll
+            for (int s = 0; s < S; ++s) x[s] = min(x[s], BTAS_INF_U16);
+            Y[v] = make_uint4(x[0] | x[1] << 16, x[2] | x[3] << 16, x[4] | x[5] << 16, x[6] | x[7] << 16);
+        } else {
+            Y[v] = make_uint4(x[0], x[1], x[2], x[3]);
+        }
+    }
+}
+
+// Y -> columns [j0, j0 + targets) of D.
+template <bool U16>
+__device__ __forceinline__ void store_columns(int *D, long long ldd, int n, const uint4 *Y, int j0) {
+    constexpr int S = targets<U16>();
+    const bool vec = (ldd & 3) == 0 && (reinterpret_cast<uintptr_t>(D) & 15) == 0 && j0 + S <= n;
+    for (int v = threadIdx.x; v < n; v += blockDim.x) {
+        const uint4 y = Y[v];
+        const unsigned ws[4] = {y.x, y.y, y.z, y.w};
+        int x[S];
+#pragma unroll
+        for (int s = 0; s < S; ++s) {
+            if (U16) {
+                x[s] = (int)((ws[s >> 1] >> (16 * (s & 1))) & 0xFFFFu);
+                if (x[s] == BTAS_INF_U16) x[s] = kInfI32;
+            } else {
+                x[s] = (int)ws[s & 3];
+            }
+        }
+        int *p = D + (long long)v * ldd + j0;
+        if (vec) {
+#pragma unroll
+            for (int s = 0; s < S; s += 4)
+                *reinterpret_cast<int4 *>(p + s) = make_int4(x[s], x[s + 1], x[s + 2], x[s + 3]);
+        } else {
+#pragma unroll
+            for (int s = 0; s < S; ++s)
+                if (j0 + s < n) p[s] = x[s];
+        }
+    }
+}
+
+// Sweeps over all vertices until Y is the closure's columns.  A sweep lowers
+// every Y[v] through v's edges, G lanes to a vertex (lane g takes chunks g, g +
+// G, ...).  A path of two or more edges that improves Y[v] starts with an edge
+// of weight w and goes on for at least minw, so w + minw < max(Y[v]): the list
+// is sorted, and the first chunk with w >= max(Y[v]) - minw ends it.
+// A row whose list was cut short of that bound at the fixpoint is then relaxed
+// from W itself, and the sweeps go on if that lowered anything.  In the end
+// every edge that could lower an entry has been tried against final values.
+//
+// One thread asks give_up() from time to time; returns false if it said so.
+// Called by the whole block.
+template <bool U16, int G, class GiveUp>
+__device__ __forceinline__ bool solve(const int *W, long long ldw, int n, const Lists &l, uint4 *Y, int minw,
+                                      GiveUp give_up) {
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, nwarps = blockDim.x >> 5;
+    constexpr int VW = 32 / G;  // vertices of a warp
+    int sweeps = 0;
+    for (;;) {
+        for (;;) {
+            bool ch = false, cut = false;
+            ++sweeps;
+            const int early_c = sweeps <= kEarlySweeps ? kEarlyChunks : l.chunks;
+            for (int v0 = warp * VW; v0 < n; v0 += nwarps * VW) {
+                const int v = v0 + lane / G, g = lane % G;
+                if (G == 1 && v >= n) break;
+                const int vc = G == 1 ? v : min(v, n - 1);
+                const uint4 old = lds_relaxed(Y + vc);
+                uint4 acc = old;
+                int lim = top<U16>(acc) - minw;
+                const uint4 *pe = l.edges + chunk_at(l, vc, g);
+                const int4 *pw = l.wide + chunk_at(l, vc, g);
+                uint4 e = *pe;
+                int4 w = make_int4(0, 0, 0, 0);
+                if (!U16) w = *pw;
+                const int heavy = 4 * (U16 ? (int)(e.x >> 16) : w.x);
+                for (int c = g;;) {
+                    if ((U16 ? (int)(e.x >> 16) : w.x) >= lim) break;
+                    const uint4 y0 = lds_relaxed(Y + (e.x & 0xFFFFu)), y1 = lds_relaxed(Y + (e.y & 0xFFFFu));
+                    const uint4 y2 = lds_relaxed(Y + (e.z & 0xFFFFu)), y3 = lds_relaxed(Y + (e.w & 0xFFFFu));
+                    const unsigned w0 = U16 ? __byte_perm(e.x, 0, 0x3232) : (unsigned)w.x;
+                    const unsigned w1 = U16 ? __byte_perm(e.y, 0, 0x3232) : (unsigned)w.y;
+                    const unsigned w2 = U16 ? __byte_perm(e.z, 0, 0x3232) : (unsigned)w.z;
+                    const unsigned w3 = U16 ? __byte_perm(e.w, 0, 0x3232) : (unsigned)w.w;
+                    c += G;
+                    const bool more = c < l.chunks;
+                    if (more) {  // the next chunk, while this one is relaxed
+                        pe += 32 * G;
+                        e = *pe;
+                        if (!U16) {
+                            pw += 32 * G;
+                            w = *pw;
+                        }
+                    }
+                    relax4<U16>(acc, y0, w0);
+                    relax4<U16>(acc, y1, w1);
+                    relax4<U16>(acc, y2, w2);
+                    relax4<U16>(acc, y3, w3);
+                    if (!more) break;
+                    lim = top<U16>(acc) - minw;
+                    // an early sweep leaves the heavier edges for later
+                    if (c >= early_c && (U16 ? (int)(e.x >> 16) : w.x) >= heavy) {
+                        cut = true;
+                        break;
+                    }
+                }
+                if (G > 1) {
+                    __syncwarp();
+#pragma unroll
+                    for (int o = G / 2; o > 0; o >>= 1) acc = min4<U16>(acc, shfl_xor4(acc, o));
+                }
+                if (!U16) acc = clamp4(acc);
+                if (differ(acc, old) && (G == 1 || (g == 0 && v < n))) {
+                    sts_relaxed(Y + v, acc);
+                    ch = true;
+                }
+            }
+            if (!__syncthreads_or(ch || cut)) break;
+            if ((sweeps & 7) == 0 && __syncthreads_or(tid == 0 && give_up())) return 0;
+        }
+        bool ch = false;
+        for (int v0 = warp * 32; v0 < n; v0 += nwarps * 32) {
+            const int vv = min(v0 + lane, n - 1);
+            const bool need = v0 + lane < n && l.next[vv] < top<U16>(lds_relaxed(Y + vv)) - minw;
+            for (unsigned m = __ballot_sync(0xffffffffu, need); m; m &= m - 1) {
+                const int v = v0 + __ffs(m) - 1;
+                const uint4 old = lds_relaxed(Y + v);
+                uint4 acc = old;
+                const int *wr = W + (long long)v * ldw;
+                for (int k = lane; k < n; k += 32) {
+                    const int w = __ldg(wr + k);
+                    if (w < (U16 ? BTAS_INF_U16 : kInfI32))
+                        relax4<U16>(acc, lds_relaxed(Y + k), U16 ? (unsigned)w * 0x10001u : (unsigned)w);
+                }
+                __syncwarp();
+#pragma unroll
+                for (int o = 16; o > 0; o >>= 1) acc = min4<U16>(acc, shfl_xor4(acc, o));
+                if (!U16) acc = clamp4(acc);
+                if (differ(acc, old)) {
+                    if (lane == 0) sts_relaxed(Y + v, acc);
+                    ch = true;
+                }
+            }
+        }
+        if (!__syncthreads_or(ch)) return true;
+        if (__syncthreads_or(tid == 0 && give_up())) return false;
+    }
+}
+
+// Whether 16 bits were enough.  Saturating sums commute with the minimum, so
+// Y = min(distance, 0x7FFF); an entry at 0x7FFF is a missing path when no
+// finite distance plus one edge, and no path of n - 1 edges, reaches 0x7FFF.
+__device__ __forceinline__ bool fits16(const uint4 *Y, int n, int maxw) {
+    int inf = 0, fin = 0;
+    for (int v = threadIdx.x; v < n; v += blockDim.x) {
+        const uint4 y = Y[v];
+        const unsigned ws[4] = {y.x, y.y, y.z, y.w};
+#pragma unroll
+        for (int s = 0; s < 8; ++s) {
+            const int x = (int)((ws[s >> 1] >> (16 * (s & 1))) & 0xFFFFu);
+            if (x == BTAS_INF_U16) inf = 1;
+            else fin = max(fin, x);
+        }
+    }
+    const bool some_inf = __syncthreads_or(inf) != 0;
+    const bool some_far = __syncthreads_or((long long)fin + maxw >= BTAS_INF_U16) != 0;
+    return !some_inf || !some_far || (long long)(n - 1) * maxw < BTAS_INF_U16;
+}
+
+}  // namespace relax
+}  // namespace btas
