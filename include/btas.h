@@ -586,8 +586,14 @@ int btas_tune_entries(void);
  *                      BTAS_BATCH_NO_GRAPH launches the kernel directly
  *                      instead of replaying a captured graph.
  * btas_batch_add_apsp: APSP by repeated squaring of W into D (device, n x n
- *                      int32, leading dimension n), as btas_apsp with int32
- *                      kernels and the early exit.  D must not overlap W.
+ *                      int32, leading dimension n); D as btas_apsp's.  D must
+ *                      not overlap W.  Up to n = 4096 the solve is a relaxation
+ *                      over sorted edge lists as in btas_apsp, with the
+ *                      squarings planned behind it for when it is given up;
+ *                      the squarings alone in a batch created with
+ *                      BTAS_BATCH_PROFILE (which traces them) or planned with
+ *                      one of BTAS_BATCH_TILE, _NO_U16, _NO_CERT, _CERT_MIN_N or
+ *                      _NO_RELAX in the environment.
  *                      The domain (zero diagonal, weights in [0, 2^28] or
  *                      INF) is assumed, not checked.
  * btas_batch_add_gemm: C = A (x) B as btas_gemm (int32 or fp32, min-plus or

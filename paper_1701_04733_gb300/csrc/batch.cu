@@ -17,7 +17,15 @@
 // memory), so the next squaring finds its B operand ready.  Early exit: the
 // first squaring whose predecessor changed nothing copies that fixpoint into
 // D, and the squarings after it do nothing (the result is unchanged).
-// Closure certificate (graphs of n >= 256): level 0 also builds W's edge
+// Relaxation.  An APSP instance of n <= 4096 starts as a relaxation instead
+// (relax.cuh): level 0 builds W's sorted edge lists, level 1 solves 8 columns of
+// D per task in the CTA's shared memory.  Its squarings are planned too, after
+// all other tasks; they run only if the relaxation was given up (the tasks from
+// fallback_start on first wait for every relaxation).  512 graphs of n = 32 ...
+// 1024 (p = 0.1) and as many products: 37.9 -> 17.0 ms per launch; relaxation is
+// bound by shared memory and shares the SMs with the products, bound by the
+// ALUs.
+// Closure certificate (squarings of graphs of n >= 256): level 0 also builds W's edge
 // lists, and after squarings 2 .. S-1 certificate tasks, placed after all of
 // their level's tiles, check X_s (x) W >= X_s at the entries squaring s
 // lowered; when every block passes, squaring s + 1 copies X_s forward
@@ -74,6 +82,7 @@ __host__ __device__ __forceinline__ bool has_cert(const BInst &I, int level) {
 // lists), level s >= 1 the output tiles (and, after an APSP squaring s <
 // levels, the certificate tasks).
 __device__ __forceinline__ int tasks_at(const BInst &I, int level) {
+    if (I.kind == kInstRelax) return (I.n + kRelaxTaskRows - 1) / kRelaxTaskRows;  // level 0: the only one waited for
     if (level == 0)
         return (I.t0_rows > 0 ? ((I.t0_rows + kBT - 1) / kBT) * ((I.t0_cols + kBT - 1) / kBT) : 0) +
                (I.cert ? list_tasks(I) : 0);
@@ -229,6 +238,86 @@ __device__ __forceinline__ bool cert_task(const BInst &I, int s, int t, int *sme
     return viol;
 }
 
+// (Both relaxation tasks stay out of line: their registers are not the product
+// tiles'.)
+//
+// Relaxation, level 0: the lists of rows 32 t .. 32 t + 31, four rows per warp,
+// and what they say about the weights.
+__device__ __noinline__ void relax_lists_task(const BInst &I, int t, unsigned char *smem, int tid) {
+    const int lane = tid & 31, warp = tid >> 5;
+    constexpr int kWarps = BCfg::kThreads / 32;
+    auto *buf = reinterpret_cast<unsigned long long *>(smem) + warp * relax::kCap;
+    int *hist = reinterpret_cast<int *>(smem + kWarps * relax::kCap * 8) + warp * 256;
+    static_assert(kWarps * (relax::kCap * 8 + 256 * 4) <= batch_smem_words() * 4, "list buffers");
+    relax::RowStats all{0, 0, kInfI32, 0, 0, 0.0f};
+    for (int q = 0; q < kRelaxTaskRows / kWarps; ++q) {
+        const int row = t * kRelaxTaskRows + q * kWarps + warp;
+        if (row >= I.n) break;
+        const relax::RowStats st =
+            relax::build_row(static_cast<const int *>(I.A), I.lda, I.n, row, I.rl, buf, hist, lane);
+        all.bad += st.bad;
+        all.maxw = max(all.maxw, st.maxw);
+        all.minw = min(all.minw, st.minw);
+        all.far |= st.far;
+        all.light += st.light;
+        __syncwarp();
+    }
+    if (lane == 0) {
+        if (all.bad) atomicAdd(I.rstat + kRelaxBadEntries, all.bad);
+        atomicMax(I.rstat + kRelaxMaxW, all.maxw);
+        atomicMax(I.rstat + kRelaxMinW, kInfI32 - all.minw);
+        if (all.far) atomicOr(I.rstat + kRelaxWide, 1);
+        atomicAdd(reinterpret_cast<float *>(I.rstat + kRelaxLight), all.light);
+    }
+}
+
+// Relaxation, level 1: columns 8 R t .. 8 R t + 8 R - 1 of D.  A task that runs too long
+// (about four times what a random graph takes on an SM shared with product
+// tiles) gives the whole solve up.
+template <int R>
+__device__ __noinline__ void relax_task(const BInst &I, int t, unsigned char *smem, int tid, int *done) {
+    constexpr int T = relax::targets<true, R>();
+    const int n = I.n, j0 = T * t;
+    uint4 *Y = reinterpret_cast<uint4 *>(smem);
+    const int *W = static_cast<const int *>(I.A);
+    int *D = static_cast<int *>(I.C);
+    const int maxw = ld_acquire(I.rstat + kRelaxMaxW), minw = kInfI32 - ld_acquire(I.rstat + kRelaxMinW);
+    const float light = __int_as_float(ld_acquire(I.rstat + kRelaxLight));
+    // the same in every thread: two words that other tasks may set meanwhile
+    __shared__ int s_word[2];
+    if (tid == 0) {
+        s_word[0] = ld_acquire(I.rstat + kRelaxWide);
+        s_word[1] = ld_acquire(I.rstat + kRelaxGaveUpWord) | (I.checked ? ld_acquire(I.rstat + kRelaxBadEntries) : 0);
+    }
+    __syncthreads();
+    bool wide = s_word[0] != 0 || relax::expects_wide(n, light);
+    if (s_word[1] != 0) return;
+    const long long t0 = clock64(), budget = I.rl.budget;
+    auto give_up = [&]() {
+        if (ld_acquire(I.rstat + kRelaxGaveUpWord) != 0) return true;
+        if (clock64() - t0 <= (wide ? 2 : 1) * budget) return false;
+        if (atomicExch(I.rstat + kRelaxGaveUpWord, 1) == 0) atomicAdd(done + 1, 1);
+        return true;
+    };
+    if (!wide) {
+        relax::load_columns<true, R>(W, I.lda, n, Y, j0);
+        __syncthreads();
+        if (!relax::solve<true, 1, R>(W, I.lda, n, I.rl, Y, minw, give_up)) return;
+        wide = !relax::fits16<R>(Y, n, maxw);
+        if (!wide) relax::store_columns<true, R>(D, I.ldc, n, Y, j0);
+        else if (tid == 0) atomicOr(I.rstat + kRelaxWide, 1);
+    }
+    if (wide) {
+        for (int h = 0; h < T && j0 + h < n; h += T / 2) {
+            __syncthreads();
+            relax::load_columns<false, R>(W, I.lda, n, Y, j0 + h);
+            __syncthreads();
+            if (!relax::solve<false, 1, R>(W, I.lda, n, I.rl, Y, minw, give_up)) return;
+            relax::store_columns<false, R>(D, I.ldc, n, Y, j0 + h);
+        }
+    }
+}
+
 // 128 x 128 transpose of a 4-byte matrix through shared memory.  With Cd /
 // Cu it also stores the tile's packed 16-bit forms (row-major, not
 // transposed) and reports the largest finite int32 entry to *maxfin.
@@ -323,6 +412,21 @@ __global__ void __launch_bounds__(BCfg::kThreads, BCfg::MINB) batch_kernel(const
             s_closed = 0;
             s_m = 0x7FFFFFFF;
             s_wait = 0;
+            if (w.x >= 0 && t >= p.fallback_start) {
+                // every relaxation first; then only the solves they gave up
+                const long long t0 = clock64();
+                while (ld_acquire(p.relax_done) < p.relax_tasks) {
+                    if (ld_acquire(p.status) != 0) break;
+                    if (clock64() - t0 > p.timeout_cycles) {
+                        atomicCAS(p.status, 0, BTAS_ERR_TIMEOUT);
+                        break;
+                    }
+                    __nanosleep(500);
+                }
+                if (ld_acquire(p.status) != 0 || ld_acquire(p.relax_done + 1) == 0) w.x = -1;
+                else if (ld_acquire(p.insts[p.insts[w.y].relax_of].rstat + kRelaxGaveUpWord) == 0) w.x = -2;
+                s_task[0] = w.x;
+            }
             if (w.x >= 0 && w.z > 0) {
                 // wait until every task of the previous level of this instance
                 // is done; a certificate task waits for the output tiles of its
@@ -366,6 +470,7 @@ __global__ void __launch_bounds__(BCfg::kThreads, BCfg::MINB) batch_kernel(const
         const int prev_closed = s_closed;
         const int prev_max = s_m;
         __syncthreads();
+        if (type == -2) continue;  // squarings of a solve that the relaxation finished
         if (type < 0) break;
         const long long t_task = clock64();
         int slot = BTAS_BATCH_SLOT_COPY;
@@ -396,6 +501,13 @@ __global__ void __launch_bounds__(BCfg::kThreads, BCfg::MINB) batch_kernel(const
                                                                   p.certfail + I.flag_base + level);
                 if (fail && tid == 0) atomicOr(p.certfail + I.flag_base + level, 1);
             }
+        } else if (type == kTaskRelaxLists) {
+            relax_lists_task(p.insts[inst], tile, smem_raw, tid);
+        } else if (type == kTaskRelax) {
+            const BInst &RI = p.insts[inst];
+            if (I.relax_rows == 4) relax_task<4>(RI, tile, smem_raw, tid, p.relax_done);
+            else if (I.relax_rows == 2) relax_task<2>(RI, tile, smem_raw, tid, p.relax_done);
+            else relax_task<1>(RI, tile, smem_raw, tid, p.relax_done);
         } else if (type == kTaskCopy) {
             // n <= 2: D = W
             const int bm = (tile / I.tiles_n) * TT, bn = (tile % I.tiles_n) * TT;
@@ -527,6 +639,7 @@ __global__ void __launch_bounds__(BCfg::kThreads, BCfg::MINB) batch_kernel(const
         __syncthreads();
         if (tid == 0) {
             atomicAdd(p.done + I.done_base + level, 1);
+            if (type == kTaskRelax) atomicAdd(p.relax_done, 1);
             if (p.prof != nullptr) {
                 atomicAdd(p.prof + 2 * slot, (unsigned long long)(clock64() - t_task));
                 atomicAdd(p.prof + 2 * slot + 1, 1ULL);
@@ -554,6 +667,19 @@ cudaError_t launch_batch_kernel(const BatchParams &p, int grid, cudaStream_t st)
     batch_kernel<<<grid, BCfg::kThreads, batch_kernel_smem(), st>>>(p);
     note_launch();
     return cudaGetLastError();
+}
+
+size_t relax_inst_bytes(long long n) {
+    return relax::list_words(n) * 8 + (((size_t)n * 4 + 255) & ~size_t(255));
+}
+
+void relax_inst_place(BInst &I, char *mem) {
+    I.rl.chunks = relax::list_chunks(I.n);
+    I.rl.edges = reinterpret_cast<uint4 *>(mem);
+    I.rl.wide = reinterpret_cast<int4 *>(mem + relax::list_words(I.n) * 4);
+    I.rl.next = reinterpret_cast<int *>(mem + relax::list_words(I.n) * 8);
+    const char *e = getenv("BTAS_RELAX_BUDGET");
+    I.rl.budget = e && *e ? atoll(e) : 4 * relax::budget_cycles(I.n);
 }
 
 long long batch_timeout_cycles(int device) {
@@ -624,6 +750,7 @@ struct btas_batch_t {
     cudaGraphExec_t exec = nullptr;
     cudaStream_t cap = nullptr;
     long long workspace_bytes = 0;
+    bool squarings = false;  // the tuner: APSP by squarings only
     int force_tile = 0;  // the tuner's timing batches: this output tile for every instance
 };
 
@@ -680,17 +807,75 @@ btas_status bfail(btas_status s, const char *msg) {
     return s;
 }
 
+// Whether the batch's APSP solves start as relaxations.  A profiled batch
+// traces the squarings' tasks, the tile tuner times them, and BTAS_BATCH_TILE,
+// BTAS_BATCH_NO_U16, BTAS_BATCH_NO_CERT and BTAS_BATCH_CERT_MIN_N name how they
+// run: those keep to them, as BTAS_BATCH_NO_RELAX=1 does.
+bool relax_allowed(const btas_batch_t *b) {
+    if (b->squarings || (b->flags & BTAS_BATCH_PROFILE)) return false;
+    for (const char *name : {"BTAS_BATCH_TILE", "BTAS_BATCH_NO_U16", "BTAS_BATCH_NO_CERT", "BTAS_BATCH_CERT_MIN_N",
+                             "BTAS_BATCH_NO_RELAX"}) {
+        const char *e = getenv(name);
+        if (e && *e) return false;
+    }
+    return true;
+}
+
+// Vectors of 8 targets a relaxation task solves at once.  Rows of 32 and 64
+// bytes conflict less in shared memory (2.1 and 1.5 cycles for 8 lanes' random
+// rows where 16-byte rows take 2.6 to move as much), but make fewer and longer tasks: as
+// wide as shared memory holds while two tasks per CTA remain.  The 512 graphs of
+// the mixed batch alone: 9.11 ms with 16-byte rows, 7.14 ms with 64-byte ones.
+int relax_rows_for(long long n, long long vectors, long long ctas) {
+    int rows = 1;
+    while (rows < 4 && 16 * n * 2 * rows <= batch_smem_words() * 4 && vectors >= 2 * ctas * 2 * rows) rows *= 2;
+    return rows;
+}
+
 btas_status build_plan(btas_batch_t *b) {
     release_plan(b);
     int dev = 0;
     if (cudaGetDevice(&dev) != cudaSuccess) return bfail(BTAS_ERR_CUDA, "btas_batch: cudaGetDevice failed");
     b->device = dev;
-    const size_t ninst = b->reqs.size();
+    // An APSP solve that may start as a relaxation is two instances: the
+    // relaxation in its place, and its squarings after all others.
+    std::vector<BInst> all;
+    std::vector<long long> work;
+    for (const auto &r : b->reqs) {
+        all.push_back(r.inst);
+        work.push_back(r.work);
+    }
+    const size_t nreq = all.size();
+    int nrelax = 0;
+    if (relax_allowed(b)) {
+        for (size_t i = 0; i < nreq; ++i) {
+            if (all[i].kind != kInstApsp || all[i].levels == 0 || all[i].n > kRelaxBatchMaxN) continue;
+            BInst I = all[i];
+            I.fallback = 1;
+            I.relax_of = (int)i;
+            all.push_back(I);
+            work.push_back(work[i]);
+            all[i].kind = kInstRelax;
+            all[i].levels = 1;
+            all[i].t0_rows = all[i].t0_cols = 0;
+            work[i] = (long long)I.n * I.n * I.n;  // next to the product of its size, which it leaves the ALUs to
+            ++nrelax;
+        }
+    }
+    const size_t ninst = all.size();
     // order instances by work, largest first
-    std::vector<int> order(ninst);
-    for (size_t i = 0; i < ninst; ++i) order[i] = (int)i;
-    std::stable_sort(order.begin(), order.end(),
-                     [&](int x, int y) { return b->reqs[x].work > b->reqs[y].work; });
+    std::vector<int> order, fallbacks;
+    for (size_t i = 0; i < ninst; ++i) (all[i].fallback ? fallbacks : order).push_back((int)i);
+    for (auto *o : {&order, &fallbacks})
+        std::stable_sort(o->begin(), o->end(), [&](int x, int y) { return work[x] > work[y]; });
+    // resident CTAs of the persistent grid
+    int per_sm = 0, sms = 0;
+    if (batch_kernel_prepare(&per_sm) != cudaSuccess) return bfail(BTAS_ERR_CUDA, "btas_batch: kernel attributes");
+    cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+    const long long grid_ctas = (long long)per_sm * sms;
+    long long relax_vectors = 0;  // 16-byte vectors of 8 targets, over all relaxations
+    for (const BInst &I : all)
+        if (I.kind == kInstRelax) relax_vectors += (I.n + 7) / 8;
     // workspace per instance and counter bases
     std::vector<BInst> insts(ninst);
     size_t ws = 0;
@@ -706,7 +891,7 @@ btas_status build_plan(btas_batch_t *b) {
     const bool allow_cert = !(no_cert && *no_cert && atoi(no_cert) != 0);
     const long long cert_min_n = (cert_min && *cert_min) ? atoll(cert_min) : 256;
     for (size_t i = 0; i < ninst; ++i) {
-        BInst I = b->reqs[i].inst;
+        BInst I = all[i];
         I.tile = choose_tile(b, dev, I);
         I.tiles_m = (I.m + I.tile - 1) / I.tile;
         I.tiles_n = (I.n + I.tile - 1) / I.tile;
@@ -729,6 +914,9 @@ btas_status build_plan(btas_batch_t *b) {
                     ws += al256((size_t)I.n * I.cap * 8) + al256((size_t)I.n * 4);
                 }
             }
+        } else if (I.kind == kInstRelax) {
+            I.relax_rows = relax_rows_for(I.n, relax_vectors, grid_ctas);
+            ws += al256(relax_inst_bytes(I.n));
         } else if (!I.trans_b) {
             I.ldq = (I.k + 3) & ~3LL;
             ws += al256((size_t)I.n * I.ldq * 4);
@@ -741,40 +929,53 @@ btas_status build_plan(btas_batch_t *b) {
     }
     // tasks
     std::vector<int4> tasks;
-    for (int level = 0; level <= max_level; ++level) {
-        for (int oi : order) {
-            const BInst &I = insts[oi];
-            if (level == 0) {
-                if (I.t0_rows > 0) {
-                    const int nt = ((I.t0_rows + kBT - 1) / kBT) * ((I.t0_cols + kBT - 1) / kBT);
-                    for (int t = 0; t < nt; ++t) tasks.push_back(make_int4(kTaskTranspose, oi, 0, t));
+    auto emit = [&](const std::vector<int> &who) {
+        for (int level = 0; level <= max_level; ++level) {
+            for (int oi : who) {
+                const BInst &I = insts[oi];
+                if (level == 0) {
+                    if (I.kind == kInstRelax)
+                        for (int t = 0; t * kRelaxTaskRows < I.n; ++t)
+                            tasks.push_back(make_int4(kTaskRelaxLists, oi, 0, t));
+                    if (I.t0_rows > 0) {
+                        const int nt = ((I.t0_rows + kBT - 1) / kBT) * ((I.t0_cols + kBT - 1) / kBT);
+                        for (int t = 0; t < nt; ++t) tasks.push_back(make_int4(kTaskTranspose, oi, 0, t));
+                    }
+                    if (I.cert)
+                        for (int t = 0; t < list_tasks(I); ++t) tasks.push_back(make_int4(kTaskLists, oi, 0, t));
+                    continue;
                 }
-                if (I.cert)
-                    for (int t = 0; t < list_tasks(I); ++t) tasks.push_back(make_int4(kTaskLists, oi, 0, t));
-                continue;
+                const int nt = I.tiles_m * I.tiles_n;
+                if (I.kind == kInstRelax) {
+                    if (level == 1)
+                        for (int t = 0; 8 * I.relax_rows * t < I.n; ++t) tasks.push_back(make_int4(kTaskRelax, oi, 1, t));
+                } else if (I.kind == kInstApsp && I.levels == 0) {
+                    if (level == 1)
+                        for (int t = 0; t < nt; ++t) tasks.push_back(make_int4(kTaskCopy, oi, 1, t));
+                } else if (I.kind == kInstApsp && level <= I.levels) {
+                    for (int t = 0; t < nt; ++t) tasks.push_back(make_int4(kTaskApsp, oi, level, t));
+                } else if (I.kind == kInstGemm && level == 1) {
+                    for (int t = 0; t < nt; ++t) tasks.push_back(make_int4(kTaskGemm, oi, 1, t));
+                }
             }
-            const int nt = I.tiles_m * I.tiles_n;
-            if (I.kind == kInstApsp && I.levels == 0) {
-                if (level == 1)
-                    for (int t = 0; t < nt; ++t) tasks.push_back(make_int4(kTaskCopy, oi, 1, t));
-            } else if (I.kind == kInstApsp && level <= I.levels) {
-                for (int t = 0; t < nt; ++t) tasks.push_back(make_int4(kTaskApsp, oi, level, t));
-            } else if (I.kind == kInstGemm && level == 1) {
-                for (int t = 0; t < nt; ++t) tasks.push_back(make_int4(kTaskGemm, oi, 1, t));
+            // the certificates of this level after every instance's tiles of it:
+            // each waits only for tasks claimed before it
+            for (int oi : who) {
+                const BInst &I = insts[oi];
+                if (I.kind == kInstApsp && has_cert(I, level))
+                    for (int t = 0; t < cert_tasks(I); ++t) tasks.push_back(make_int4(kTaskCert, oi, level, t));
             }
         }
-        // the certificates of this level after every instance's tiles of it:
-        // each waits only for tasks claimed before it
-        for (int oi : order) {
-            const BInst &I = insts[oi];
-            if (I.kind == kInstApsp && has_cert(I, level))
-                for (int t = 0; t < cert_tasks(I); ++t) tasks.push_back(make_int4(kTaskCert, oi, level, t));
-        }
-    }
+    };
+    emit(order);
+    const int fallback_start = (int)tasks.size();
+    const int relax_tasks =
+        (int)std::count_if(tasks.begin(), tasks.end(), [](const int4 &t) { return t.x == kTaskRelax; });
+    emit(fallbacks);
     b->total = (int)tasks.size();
     const size_t task_bytes = al256(tasks.size() * sizeof(int4));
     const size_t inst_bytes = al256(ninst * sizeof(BInst));
-    b->counter_bytes = al256((size_t)(2 + 4 * counters) * 4);
+    b->counter_bytes = al256((size_t)(2 + 4 * counters + 2 + kRelaxWords * nrelax) * 4);
     b->workspace_bytes = (long long)ws;
     const size_t prof_bytes = (b->flags & BTAS_BATCH_PROFILE) ? al256(2 * BTAS_BATCH_PROFILE_SLOTS * 8) : 0;
     b->dev_bytes = task_bytes + inst_bytes + b->counter_bytes + prof_bytes + ws;
@@ -789,9 +990,15 @@ btas_status build_plan(btas_batch_t *b) {
     if (b->d_prof && cudaMemset(b->d_prof, 0, prof_bytes) != cudaSuccess)
         return bfail(BTAS_ERR_CUDA, "btas_batch: profile reset");
     char *d_ws = base + task_bytes + inst_bytes + b->counter_bytes + prof_bytes;
+    int *relax_words = b->d_counters + 2 + 4 * counters;  // [0, 2) tasks done and solves given up, then rstat
+    int relax_next = 0;
     for (size_t i = 0; i < ninst; ++i) {
         BInst &I = insts[i];
         char *w = d_ws + ws_off[i];
+        if (I.kind == kInstRelax) {
+            relax_inst_place(I, w);
+            I.rstat = relax_words + 2 + kRelaxWords * relax_next++;
+        }
         if (I.kind == kInstApsp && I.levels > 0) {
             const size_t blk = al256((size_t)I.n * I.ldq * 4);
             I.X0 = w;
@@ -824,6 +1031,9 @@ btas_status build_plan(btas_batch_t *b) {
     p.maxfin = b->d_counters + 2 + 2 * counters;
     p.certfail = b->d_counters + 2 + 3 * counters;
     p.insts = d_insts;
+    p.fallback_start = fallback_start;
+    p.relax_tasks = relax_tasks;
+    p.relax_done = relax_words;
     p.timeout_cycles = batch_timeout_cycles(dev);
     p.prof = b->d_prof;
     // Fault injection (tests only): BTAS_BATCH_WITHHOLD=i makes the host
@@ -833,10 +1043,7 @@ btas_status build_plan(btas_batch_t *b) {
     p.withhold_inst = (wh && *wh) ? atoi(wh) : -1;
     // grid: resident CTAs
     b->smem = batch_kernel_smem();
-    int per_sm = 0, sms = 0;
-    if (batch_kernel_prepare(&per_sm) != cudaSuccess) return bfail(BTAS_ERR_CUDA, "btas_batch: kernel attributes");
-    cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-    b->grid = std::max(1, std::min(per_sm * sms, std::max(1, b->total)));
+    b->grid = (int)std::max(1LL, std::min(grid_ctas, std::max(1LL, (long long)b->total)));
     // capture: counter reset + persistent kernel
     if (!(b->flags & BTAS_BATCH_NO_GRAPH)) {
         if (!b->cap && cudaStreamCreateWithFlags(&b->cap, cudaStreamNonBlocking) != cudaSuccess)
@@ -1128,6 +1335,7 @@ btas_status batch_tune_impl(int64_t n_max, cudaStream_t st, double *ms_out, int 
                 btas_batch_t *b = nullptr;
                 btas_batch_create(&b, 0);
                 b->force_tile = ti == 0 ? kBT : kBTSmall;
+                b->squarings = true;
                 for (auto &m : mats) {
                     const long long n = m.first;
                     const size_t mb = al256((size_t)n * n * 4);

@@ -5,6 +5,8 @@
 #include <cstdint>
 #include <cuda_runtime.h>
 
+#include "relax.cuh"
+
 namespace btas {
 
 constexpr int kBT = 128;  // task tile edge (level-0 transposes, and the default output tile)
@@ -17,15 +19,30 @@ enum TaskType : int {
     kTaskCopy = 3,
     kTaskSquare = 4,
     kTaskLists = 5,  // APSP level 0: the edge lists of 32 rows of W
-    kTaskCert = 6    // APSP after squaring s (its level): the closure certificate over a block of rows
+    kTaskCert = 6,   // APSP after squaring s (its level): the closure certificate over a block of rows
+    kTaskRelaxLists = 7,  // relaxation, level 0: the sorted edge lists of 32 rows of W
+    kTaskRelax = 8        // relaxation, level 1: 8 relax_rows columns of D
 };
-enum InstKind : int { kInstApsp = 0, kInstGemm = 1, kInstSquare = 2 };
+enum InstKind : int { kInstApsp = 0, kInstGemm = 1, kInstSquare = 2, kInstRelax = 3 };
+// Words of BInst::rstat, zero before the launch.
+enum RelaxWord : int {
+    kRelaxBadEntries = 0,  // entries of W outside the domain
+    kRelaxMaxW = 1,        // largest weight
+    kRelaxMinW = 2,        // INF - the smallest off-diagonal weight
+    kRelaxWide = 3,        // set: 32-bit distances
+    kRelaxGaveUpWord = 4,  // set: left to the squarings
+    kRelaxLight = 5,       // float: the sum of the rows' lightest weights
+    kRelaxWords = 8
+};
+constexpr int kRelaxTaskRows = 32;     // rows of a list task
+constexpr int kRelaxBatchMaxN = 4096;  // 16 n bytes of the kernel's shared memory
 
 // One problem of a launch.  kInstApsp: a whole APSP solve (levels = S
 // squarings); kInstGemm: one product; kInstSquare: ONE squaring
 // C = A (x) A with prev = A, B operand A^T in Q0 (level 0 transposes A into
 // Q0 when t0_rows > 0), optional transposed output into Q1 and a change flag
-// at changed_ptr.
+// at changed_ptr.  kInstRelax: a whole APSP solve by relaxation over sorted
+// edge lists (relax.cuh), which either fills C or sets rstat's gave-up word.
 struct BInst {
     int kind, sr, dtype;
     int tile;             // output tile edge of the level >= 1 tasks: kBT or kBTSmall (0 = kBT)
@@ -70,6 +87,15 @@ struct BInst {
     int cert_rows;
     int2 *lists;
     int *deg;
+    // relaxation: its lists, its words, and whether W's domain is checked (C
+    // is then not written where it is violated)
+    relax::Lists rl;
+    int *rstat;
+    int checked;
+    int relax_rows;  // vectors of 8 targets per task: 1, 2 or 4
+    // APSP squarings that only run when the relaxation of instance relax_of
+    // (>= 0) gave up
+    int fallback, relax_of;
 };
 
 struct BatchParams {
@@ -84,6 +110,11 @@ struct BatchParams {
     int *status;
     const BInst *insts;
     long long timeout_cycles;
+    // tasks from fallback_start on are the squarings of solves whose relaxation
+    // may give up; they wait until all relax_tasks relaxation tasks are done
+    int fallback_start;
+    int relax_tasks;
+    int *relax_done;    // [0] relaxation tasks done, [1] solves given up
     int withhold_inst;  // fault injection for tests: this instance's level-1+ tasks never become ready
     unsigned long long *prof;  // optional: (cycles, count) per BTAS_BATCH_SLOT_*
 };
@@ -94,5 +125,9 @@ int batch_kernel_threads();
 cudaError_t batch_kernel_prepare(int *ctas_per_sm);
 cudaError_t launch_batch_kernel(const BatchParams &p, int grid, cudaStream_t st);
 long long batch_timeout_cycles(int device);
+// Sets up a kInstRelax instance: lists for n vertices at `mem`
+// (relax_inst_bytes(n) bytes, not initialised).
+size_t relax_inst_bytes(long long n);
+void relax_inst_place(BInst &I, char *mem);
 
 }  // namespace btas

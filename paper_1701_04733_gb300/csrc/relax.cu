@@ -98,10 +98,11 @@ __global__ void __launch_bounds__(MAXT) relax_solve_kernel(const RelaxArgs a) {
     __shared__ RowStats s_st;
     const long long t0 = clock64();
     const int n = a.n, tid = threadIdx.x;
-    const int groups = (n + 7) / 8, part = blockIdx.x >= groups ? 1 : 0;  // the second parts on SMs of their own
-    const int j0 = (blockIdx.x - part * groups) * 8;
+    constexpr int R = 1, T = relax::targets<true, R>();  // targets of a block, in 16 bits
+    const int groups = (n + T - 1) / T, part = blockIdx.x >= groups ? 1 : 0;  // the second parts on SMs of their own
+    const int j0 = (blockIdx.x - part * groups) * T;
     if (tid == 0) s_st = RowStats{0, 0, kInfI32, 0, 0, 0.0f};
-    if (part == 0) relax::load_columns<true>(a.W, a.ldw, n, Y, j0);  // needs no lists
+    if (part == 0) relax::load_columns<true, R>(a.W, a.ldw, n, Y, j0);  // needs no lists
     asm volatile("griddepcontrol.wait;" ::: "memory");
     __syncthreads();
     const int nst = (n + kListWarps - 1) / kListWarps;
@@ -138,20 +139,20 @@ __global__ void __launch_bounds__(MAXT) relax_solve_kernel(const RelaxArgs a) {
             a.ctl[kAbort] = 1;
             return true;
         };
-        if (part == 0 && !wide && relax::solve<true, G>(a.W, a.ldw, n, a.lists, Y, st.minw, give_up)) {
-            wide = !relax::fits16(Y, n, st.maxw);
-            if (!wide) relax::store_columns<true>(a.D, a.ldd, n, Y, j0);
+        if (part == 0 && !wide && relax::solve<true, G, R>(a.W, a.ldw, n, a.lists, Y, st.minw, give_up)) {
+            wide = !relax::fits16<R>(Y, n, st.maxw);
+            if (!wide) relax::store_columns<true, R>(a.D, a.ldd, n, Y, j0);
             else if (tid == 0) a.ctl[kWide] = 1;
         }
-        // in 32 bits, 4 targets at a time
+        // in 32 bits, half of the targets at a time
         const bool split = wide_first && a.halves == 2;
         if (wide && (part == 0 || split)) {
-            for (int h = 4 * part; h < (split ? 4 * part + 4 : 8) && j0 + h < n; h += 4) {
+            for (int h = part * T / 2; h < (split ? (part + 1) * T / 2 : T) && j0 + h < n; h += T / 2) {
                 __syncthreads();
-                relax::load_columns<false>(a.W, a.ldw, n, Y, j0 + h);
+                relax::load_columns<false, R>(a.W, a.ldw, n, Y, j0 + h);
                 __syncthreads();
-                if (!relax::solve<false, G>(a.W, a.ldw, n, a.lists, Y, st.minw, give_up)) break;
-                relax::store_columns<false>(a.D, a.ldd, n, Y, j0 + h);
+                if (!relax::solve<false, G, R>(a.W, a.ldw, n, a.lists, Y, st.minw, give_up)) break;
+                relax::store_columns<false, R>(a.D, a.ldd, n, Y, j0 + h);
             }
         }
     }
@@ -216,10 +217,14 @@ cudaError_t launch_relax(const int *W, long long ldw, int n, int *D, long long l
     a.halves = n <= 1216 ? 2 : 1;
     relax_lists_kernel<<<blocks, kListWarps * 32, 0, st>>>(a);
     note_launch();
-    // Two lanes per vertex where one would leave warps idle (n <= 256); 512
-    // threads while two blocks fit an SM (n = 4096, p = 0.01: 1118 us with 1024
-    // threads, 1060 with 512), 1024 beyond (n = 8192: 3662 us against 3779).
-    const int G = n <= 256 ? 2 : 1, maxt = n > 7000 ? 1024 : 512;
+    // Two lanes per vertex where one would leave warps idle (n <= 256).  1024
+    // threads where one block per SM holds all targets (n = 1024, p = 0.1: 93 us
+    // per call, 112 with 512 threads) or fills shared memory (n = 8192: 3662 us
+    // against 3779), 512 and two blocks per SM between (n = 4096, p = 0.01: 1060
+    // us against 1118).  Rows of 16 or 32 targets, which pay in the batched
+    // launch, lose more to their fewer blocks than they gain (n = 2048: 265 and
+    // 377 us against 249).
+    const int G = n <= 256 ? 2 : 1, maxt = (n > 608 && n <= 1216) || n > 7000 ? 1024 : 512;
     void (*kern)(const RelaxArgs) = G == 2 ? relax_solve_kernel<2, 512>
                                     : maxt == 512 ? relax_solve_kernel<1, 512> : relax_solve_kernel<1, 1024>;
     cudaError_t e = set_smem_once(reinterpret_cast<const void *>(kern), kSolveSmem);

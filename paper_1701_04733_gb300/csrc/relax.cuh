@@ -313,9 +313,9 @@ __device__ __forceinline__ RowStats build_row(const int *W, long long ldw, int n
 }
 
 // -------------------------------------------------------------- relaxing
-// Y[v] in shared memory: 16 bytes, the distances from v to 8 targets in 16
-// bits (0x7FFF: none known) or to 4 targets in 32.  Only the lanes of v's own
-// group write Y[v], and a stale read costs a further sweep and no more, so the
+// Y in shared memory: a row of 16 R bytes per vertex v, the distances from v to
+// 8 R targets in 16 bits (0x7FFF: none known) or to 4 R in 32.  Only v's own
+// lanes write its row, and a stale read costs a further sweep and no more, so the
 // accesses of a sweep are relaxed ones.
 __device__ __forceinline__ uint4 lds_relaxed(const uint4 *p) {
     uint4 v;
@@ -371,18 +371,21 @@ __device__ __forceinline__ bool differ(const uint4 &a, const uint4 &b) {
     return ((a.x ^ b.x) | (a.y ^ b.y) | (a.z ^ b.z) | (a.w ^ b.w)) != 0;
 }
 
-template <bool U16>
-constexpr int targets() { return U16 ? 8 : 4; }
+// A vertex's row is R vectors of 16 bytes, each with its own lane: 8 R targets
+// in 16 bits, 4 R in 32.
+template <bool U16, int R>
+constexpr int targets() { return (U16 ? 8 : 4) * R; }
 
 // Columns [j0, j0 + targets) of W -> Y: the paths of one edge.
-template <bool U16>
+template <bool U16, int R>
 __device__ __forceinline__ void load_columns(const int *W, long long ldw, int n, uint4 *Y, int j0) {
-    constexpr int S = targets<U16>();
-    const bool vec = (ldw & 3) == 0 && (reinterpret_cast<uintptr_t>(W) & 15) == 0 && j0 + S <= n;
-    for (int v = threadIdx.x; v < n; v += blockDim.x) {
+    constexpr int S = targets<U16, 1>();
+    const bool vec = (ldw & 3) == 0 && (reinterpret_cast<uintptr_t>(W) & 15) == 0;
+    for (int i = threadIdx.x; i < n * R; i += blockDim.x) {
+        const int j = j0 + (i % R) * S;
         int x[S];
-        const int *p = W + (long long)v * ldw + j0;
-        if (vec) {
+        const int *p = W + (long long)(i / R) * ldw + j;
+        if (vec && j + S <= n) {
 #pragma unroll
             for (int s = 0; s < S; s += 4) {
                 const int4 q = __ldg(reinterpret_cast<const int4 *>(p + s));
@@ -390,65 +393,69 @@ __device__ __forceinline__ void load_columns(const int *W, long long ldw, int n,
             }
         } else {
 #pragma unroll
-            for (int s = 0; s < S; ++s) x[s] = j0 + s < n ? __ldg(p + s) : 0;  // an absent target: nothing to lower
+            for (int s = 0; s < S; ++s) x[s] = j + s < n ? __ldg(p + s) : 0;  // an absent target: nothing to lower
         }
         if constexpr (U16) {
 #pragma unroll
             for (int s = 0; s < S; ++s) x[s] = min(x[s], BTAS_INF_U16);
-            Y[v] = make_uint4(x[0] | x[1] << 16, x[2] | x[3] << 16, x[4] | x[5] << 16, x[6] | x[7] << 16);
+            Y[i] = make_uint4(x[0] | x[1] << 16, x[2] | x[3] << 16, x[4] | x[5] << 16, x[6] | x[7] << 16);
         } else {
-            Y[v] = make_uint4(x[0], x[1], x[2], x[3]);
+            Y[i] = make_uint4(x[0], x[1], x[2], x[3]);
         }
     }
 }
 
 // Y -> columns [j0, j0 + targets) of D.
-template <bool U16>
+template <bool U16, int R>
 __device__ __forceinline__ void store_columns(int *D, long long ldd, int n, const uint4 *Y, int j0) {
-    constexpr int S = targets<U16>();
-    const bool vec = (ldd & 3) == 0 && (reinterpret_cast<uintptr_t>(D) & 15) == 0 && j0 + S <= n;
-    for (int v = threadIdx.x; v < n; v += blockDim.x) {
-        const uint4 y = Y[v];
+    constexpr int S = targets<U16, 1>();
+    const bool vec = (ldd & 3) == 0 && (reinterpret_cast<uintptr_t>(D) & 15) == 0;
+    for (int i = threadIdx.x; i < n * R; i += blockDim.x) {
+        const int j = j0 + (i % R) * S;
+        const uint4 y = Y[i];
         const unsigned ws[4] = {y.x, y.y, y.z, y.w};
         int x[S];
 #pragma unroll
         for (int s = 0; s < S; ++s) {
             if (U16) {
-                x[s] = (int)((ws[s >> 1] >> (16 * (s & 1))) & 0xFFFFu);
+                x[s] = (int)((ws[(s >> 1) & 3] >> (16 * (s & 1))) & 0xFFFFu);
                 if (x[s] == BTAS_INF_U16) x[s] = kInfI32;
             } else {
                 x[s] = (int)ws[s & 3];
             }
         }
-        int *p = D + (long long)v * ldd + j0;
-        if (vec) {
+        int *p = D + (long long)(i / R) * ldd + j;
+        if (vec && j + S <= n) {
 #pragma unroll
             for (int s = 0; s < S; s += 4)
                 *reinterpret_cast<int4 *>(p + s) = make_int4(x[s], x[s + 1], x[s + 2], x[s + 3]);
         } else {
 #pragma unroll
             for (int s = 0; s < S; ++s)
-                if (j0 + s < n) p[s] = x[s];
+                if (j + s < n) p[s] = x[s];
         }
     }
 }
 
 // Sweeps over all vertices until Y is the closure's columns.  A sweep lowers
-// every Y[v] through v's edges, G lanes to a vertex (lane g takes chunks g, g +
-// G, ...).  A path of two or more edges that improves Y[v] starts with an edge
-// of weight w and goes on for at least minw, so w + minw < max(Y[v]): the list
-// is sorted, and the first chunk with w >= max(Y[v]) - minw ends it.
+// every Y[v] through v's edges, R lanes to a vertex's row and G sets of them to
+// a vertex (set g takes chunks g, g + G, ...).  A path of two or more edges that
+// improves Y[v] starts with an edge of weight w and goes on for at least minw,
+// so w + minw < max(Y[v]): the list is sorted, and the first chunk with w >=
+// max(Y[v]) - minw ends it, for each lane by its own targets.
 // A row whose list was cut short of that bound at the fixpoint is then relaxed
 // from W itself, and the sweeps go on if that lowered anything.  In the end
 // every edge that could lower an entry has been tried against final values.
 //
 // One thread asks give_up() from time to time; returns false if it said so.
 // Called by the whole block.
-template <bool U16, int G, class GiveUp>
+template <bool U16, int G, int R, class GiveUp>
 __device__ __forceinline__ bool solve(const int *W, long long ldw, int n, const Lists &l, uint4 *Y, int minw,
                                       GiveUp give_up) {
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, nwarps = blockDim.x >> 5;
-    constexpr int VW = 32 / G;  // vertices of a warp
+    constexpr int VW = 32 / (G * R);  // vertices of a warp
+    const int sub = lane % R, g = (lane / R) % G;
+    const uint4 *Ys = Y + sub;  // Ys[v * R]: this lane's part of v's row
     int sweeps = 0;
     for (;;) {
         for (;;) {
@@ -456,10 +463,10 @@ __device__ __forceinline__ bool solve(const int *W, long long ldw, int n, const 
             ++sweeps;
             const int early_c = sweeps <= kEarlySweeps ? kEarlyChunks : l.chunks;
             for (int v0 = warp * VW; v0 < n; v0 += nwarps * VW) {
-                const int v = v0 + lane / G, g = lane % G;
+                const int v = v0 + lane / (G * R);
                 if (G == 1 && v >= n) break;
                 const int vc = G == 1 ? v : min(v, n - 1);
-                const uint4 old = lds_relaxed(Y + vc);
+                const uint4 old = lds_relaxed(Ys + vc * R);
                 uint4 acc = old;
                 int lim = top<U16>(acc) - minw;
                 const uint4 *pe = l.edges + chunk_at(l, vc, g);
@@ -470,8 +477,8 @@ __device__ __forceinline__ bool solve(const int *W, long long ldw, int n, const 
                 const int heavy = 4 * (U16 ? (int)(e.x >> 16) : w.x);
                 for (int c = g;;) {
                     if ((U16 ? (int)(e.x >> 16) : w.x) >= lim) break;
-                    const uint4 y0 = lds_relaxed(Y + (e.x & 0xFFFFu)), y1 = lds_relaxed(Y + (e.y & 0xFFFFu));
-                    const uint4 y2 = lds_relaxed(Y + (e.z & 0xFFFFu)), y3 = lds_relaxed(Y + (e.w & 0xFFFFu));
+                    const uint4 y0 = lds_relaxed(Ys + (e.x & 0xFFFFu) * R), y1 = lds_relaxed(Ys + (e.y & 0xFFFFu) * R);
+                    const uint4 y2 = lds_relaxed(Ys + (e.z & 0xFFFFu) * R), y3 = lds_relaxed(Ys + (e.w & 0xFFFFu) * R);
                     const unsigned w0 = U16 ? __byte_perm(e.x, 0, 0x3232) : (unsigned)w.x;
                     const unsigned w1 = U16 ? __byte_perm(e.y, 0, 0x3232) : (unsigned)w.y;
                     const unsigned w2 = U16 ? __byte_perm(e.z, 0, 0x3232) : (unsigned)w.z;
@@ -501,37 +508,39 @@ __device__ __forceinline__ bool solve(const int *W, long long ldw, int n, const 
                 if (G > 1) {
                     __syncwarp();
 #pragma unroll
-                    for (int o = G / 2; o > 0; o >>= 1) acc = min4<U16>(acc, shfl_xor4(acc, o));
+                    for (int o = G * R / 2; o >= R; o >>= 1) acc = min4<U16>(acc, shfl_xor4(acc, o));
                 }
                 if (!U16) acc = clamp4(acc);
                 if (differ(acc, old) && (G == 1 || (g == 0 && v < n))) {
-                    sts_relaxed(Y + v, acc);
+                    sts_relaxed(Y + v * R + sub, acc);
                     ch = true;
                 }
             }
             if (!__syncthreads_or(ch || cut)) break;
-            if ((sweeps & 7) == 0 && __syncthreads_or(tid == 0 && give_up())) return 0;
+            if ((sweeps & 7) == 0 && __syncthreads_or(tid == 0 && give_up())) return false;
         }
         bool ch = false;
-        for (int v0 = warp * 32; v0 < n; v0 += nwarps * 32) {
-            const int vv = min(v0 + lane, n - 1);
-            const bool need = v0 + lane < n && l.next[vv] < top<U16>(lds_relaxed(Y + vv)) - minw;
-            for (unsigned m = __ballot_sync(0xffffffffu, need); m; m &= m - 1) {
-                const int v = v0 + __ffs(m) - 1;
-                const uint4 old = lds_relaxed(Y + v);
+        for (int v0 = warp * VW; v0 < n; v0 += nwarps * VW) {
+            const int vv = min(v0 + lane / (G * R), n - 1);
+            const bool need = l.next[vv] < top<U16>(lds_relaxed(Ys + vv * R)) - minw;
+            for (unsigned m = __ballot_sync(0xffffffffu, need); m;) {
+                const int first = (__ffs(m) - 1) / (G * R);  // the row's number in the warp
+                m &= ~(((1u << (G * R)) - 1u) << (first * G * R));
+                const int v = min(v0 + first, n - 1);
+                const uint4 old = lds_relaxed(Ys + v * R);
                 uint4 acc = old;
                 const int *wr = W + (long long)v * ldw;
-                for (int k = lane; k < n; k += 32) {
+                for (int k = lane / R; k < n; k += 32 / R) {
                     const int w = __ldg(wr + k);
                     if (w < (U16 ? BTAS_INF_U16 : kInfI32))
-                        relax4<U16>(acc, lds_relaxed(Y + k), U16 ? (unsigned)w * 0x10001u : (unsigned)w);
+                        relax4<U16>(acc, lds_relaxed(Ys + k * R), U16 ? (unsigned)w * 0x10001u : (unsigned)w);
                 }
                 __syncwarp();
 #pragma unroll
-                for (int o = 16; o > 0; o >>= 1) acc = min4<U16>(acc, shfl_xor4(acc, o));
+                for (int o = 16; o >= R; o >>= 1) acc = min4<U16>(acc, shfl_xor4(acc, o));
                 if (!U16) acc = clamp4(acc);
                 if (differ(acc, old)) {
-                    if (lane == 0) sts_relaxed(Y + v, acc);
+                    if (lane < R) sts_relaxed(Y + v * R + sub, acc);
                     ch = true;
                 }
             }
@@ -544,10 +553,11 @@ __device__ __forceinline__ bool solve(const int *W, long long ldw, int n, const 
 // Whether 16 bits were enough.  Saturating sums commute with the minimum, so
 // Y = min(distance, 0x7FFF); an entry at 0x7FFF is a missing path when no
 // finite distance plus one edge, and no path of n - 1 edges, reaches 0x7FFF.
+template <int R>
 __device__ __forceinline__ bool fits16(const uint4 *Y, int n, int maxw) {
     int inf = 0, fin = 0;
-    for (int v = threadIdx.x; v < n; v += blockDim.x) {
-        const uint4 y = Y[v];
+    for (int i = threadIdx.x; i < n * R; i += blockDim.x) {
+        const uint4 y = Y[i];
         const unsigned ws[4] = {y.x, y.y, y.z, y.w};
 #pragma unroll
         for (int s = 0; s < 8; ++s) {

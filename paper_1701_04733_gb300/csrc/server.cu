@@ -419,6 +419,7 @@ int launch_step(btas_server_t *sv, std::vector<Req *> &units) {
     p.total = (int)tasks.size();
     p.timeout_cycles = sv->timeout_cycles;
     p.withhold_inst = -1;
+    p.fallback_start = p.total;
     const int grid = std::max(1, std::min(sv->grid, p.total));
     if (launch_batch_kernel(p, grid, sv->compute) != cudaSuccess) return -1;
     // change flags and largest finite entries of this step's squarings ->

@@ -157,3 +157,44 @@ def test_domain_violation_leaves_the_result_untouched(btas, value):
         btas.apsp(dev(W), out=out)
     assert ei.value.status == 1
     assert (host(out) == 19).all()
+
+
+def solve_batch(btas, graphs, graph=True):
+    b = btas.Batch(graph=graph)
+    outs = [b.add_apsp(dev(W), dev(np.full_like(W, 5))) for W in graphs]
+    A = dev(gen.uniform_int(3, 9, (300, 200), 0, 1000))
+    C = b.add_gemm(A, A, dev(np.zeros((300, 300), np.int32)), trans_b=True)
+    results = []
+    for _ in range(2):  # the second launch replays the plan
+        b.launch()
+        b.wait()
+        results.append([host(o).copy() for o in outs + [C]])
+    b.close()
+    for x, y in zip(*results):
+        np.testing.assert_array_equal(x, y)
+    np.testing.assert_array_equal(results[0][-1], host(btas.gemm(A, A, trans_b=True)))
+    return results[0][:-1]
+
+
+@pytest.mark.parametrize("graph", [True, False])
+def test_batched_relaxation(btas, oracle_mod, graph):
+    """Every form of graph and the sizes around 2, a list task's rows and a list's capacity, beside a product."""
+    graphs = [GRAPHS[g](n) for g in sorted(GRAPHS) for n in (33, 150)]
+    graphs += [random(0.3, 100)(n) for n in (1, 2, 3, 7, 8, 9, 31, 32, 511, 512, 513, 700)]
+    graphs.append(hidden_heavy_edge(640))
+    for W, D in zip(graphs, solve_batch(btas, graphs, graph)):
+        ref = oracle_mod.floyd_warshall(W)
+        ref[ref >= INF - (1 << 28)] = INF
+        np.testing.assert_array_equal(D, ref)
+
+
+def test_batched_relaxation_given_up(btas, oracle_mod):
+    """Long paths with no time allowed: their squarings run, the other solves' do not have to."""
+    graphs = [path(100), random(0.2, 100)(60), path(300), random(0.05, 100)(300)]
+    os.environ["BTAS_RELAX_BUDGET"] = "0"
+    try:
+        outs = solve_batch(btas, graphs)
+    finally:
+        del os.environ["BTAS_RELAX_BUDGET"]
+    for W, D in zip(graphs, outs):
+        np.testing.assert_array_equal(D, oracle_mod.floyd_warshall(W))
