@@ -238,7 +238,9 @@ btas_status btas_gemv(int semiring, int dtype, int trans, int64_t m, int64_t n, 
  * domain check fails (BTAS_ERR_ARG).  iterations: HOST pointer or NULL,
  * receives the number of products that changed d.  All products run in one
  * cooperative launch with one bounded grid barrier each (BTAS_ERR_TIMEOUT if
- * a wait expires; the first product also checks the domain), and the call
+ * a wait expires; the first pass over W also checks the domain and builds
+ * edge lists, up to n n bytes of scratch; later products relax the vertices
+ * that the one before lowered), and the call
  * synchronises `stream` once.  Where a cooperative launch is refused (or
  * with BTAS_SSSP_NO_COOP=1 in the environment) it launches the products in
  * gated groups of 8 and synchronises once per group. */
