@@ -37,8 +37,14 @@ __device__ __forceinline__ uint32_t carrier_map(uint32_t bits, int mode) {
 }
 
 __global__ void transpose4_kernel(const uint32_t *__restrict__ src, long long lds, int rows, int cols,
-                                  uint32_t *__restrict__ dst, long long ldd, int mode, const int *skip) {
+                                  uint32_t *__restrict__ dst, long long ldd, int mode, const int *skip,
+                                  uint32_t *__restrict__ C, long long ldc, int m, uint32_t bits) {
     if (skip != nullptr && *skip == 0) return;
+    if (C != nullptr) {  // also fill C (m x cols): this block its 32 columns of every gridDim.y-th 8 rows
+        const int c = blockIdx.x * 32 + threadIdx.x;
+        for (int r = blockIdx.y * 8 + threadIdx.y; r < m; r += gridDim.y * 8)
+            if (c < cols) C[(long long)r * ldc + c] = bits;
+    }
     __shared__ uint32_t tile[32][33];
     const int c0 = blockIdx.x * 32, r0 = blockIdx.y * 32;
     const int tx = threadIdx.x, ty = threadIdx.y;  // 32 x 8
@@ -52,6 +58,21 @@ __global__ void transpose4_kernel(const uint32_t *__restrict__ src, long long ld
     for (int i = 0; i < 32; i += 8) {
         const int c = c0 + ty + i, r = r0 + tx;  // dst row c, dst col r
         if (r < rows && c < cols) dst[(long long)c * ldd + r] = tile[tx][ty + i];
+    }
+}
+
+// rows x cols words to another pitch: one row per blockIdx.y step, 4 columns per thread a warp's width apart.
+__global__ void pad4_kernel(const uint32_t *__restrict__ src, long long lds, int rows, int cols,
+                            uint32_t *__restrict__ dst, long long ldd) {
+    const int c0 = blockIdx.x * 1024 + threadIdx.x;
+    for (int r = blockIdx.y; r < rows; r += gridDim.y) {
+        uint32_t v[4];
+#pragma unroll
+        for (int q = 0; q < 4; ++q)
+            if (c0 + 256 * q < cols) v[q] = src[(long long)r * lds + c0 + 256 * q];
+#pragma unroll
+        for (int q = 0; q < 4; ++q)
+            if (c0 + 256 * q < cols) dst[(long long)r * ldd + c0 + 256 * q] = v[q];
     }
 }
 
@@ -179,7 +200,27 @@ cudaError_t launch_transpose4(const void *src, long long lds, int rows, int cols
     if (rows <= 0 || cols <= 0) return cudaSuccess;
     dim3 grid((cols + 31) / 32, (rows + 31) / 32), block(32, 8);
     transpose4_kernel<<<grid, block, 0, st>>>(static_cast<const uint32_t *>(src), lds, rows, cols,
-                                              static_cast<uint32_t *>(dst), ldd, mode, skip);
+                                              static_cast<uint32_t *>(dst), ldd, mode, skip, nullptr, 0, 0, 0);
+    note_launch();
+    return cudaGetLastError();
+}
+
+cudaError_t launch_transpose4_fill(const void *src, long long lds, int rows, int cols, void *dst, long long ldd,
+                                   void *C, long long ldc, int m, uint32_t bits, cudaStream_t st) {
+    if (rows <= 0 || cols <= 0) return cudaSuccess;
+    dim3 grid((cols + 31) / 32, (rows + 31) / 32), block(32, 8);
+    transpose4_kernel<<<grid, block, 0, st>>>(static_cast<const uint32_t *>(src), lds, rows, cols,
+                                              static_cast<uint32_t *>(dst), ldd, 0, nullptr,
+                                              static_cast<uint32_t *>(C), ldc, m, bits);
+    note_launch();
+    return cudaGetLastError();
+}
+
+cudaError_t launch_pad4(const void *src, long long lds, int rows, int cols, void *dst, long long ldd,
+                        cudaStream_t st) {
+    if (rows <= 0 || cols <= 0) return cudaSuccess;
+    pad4_kernel<<<dim3((cols + 1023) / 1024, rows < 16384 ? rows : 16384), 256, 0, st>>>(
+        static_cast<const uint32_t *>(src), lds, rows, cols, static_cast<uint32_t *>(dst), ldd);
     note_launch();
     return cudaGetLastError();
 }

@@ -2,6 +2,7 @@
 // selection, stream-ordered workspace, and the APSP squaring driver.
 #include <algorithm>
 #include <atomic>
+#include <cmath>
 #include <cstdarg>
 #include <cstdint>
 #include <cstdio>
@@ -217,53 +218,119 @@ int env_int(const char *name, int dflt) {
     return v && *v ? atoi(v) : dflt;
 }
 
+uint32_t ident_bits(int dtype, int sr) {
+    if (dtype == BTAS_I32) return static_cast<uint32_t>(sr == kMin ? kInfI32 : kNinfI32);
+    return sr == kMin ? 0x7f800000u : 0xff800000u;
+}
+
+// A product's kernel, raster group and k split.
+struct NtPlan {
+    const GemmKernel *kernel = nullptr;
+    int group_m = 8;
+    int splits = 1;
+};
+
+// Expected time (us) of an m x n x k product with a kernel's tiles, `splits` CTAs
+// to a tile: the busiest SM's CTAs (with many of them, the mean and a bit) at the
+// rate that so many resident CTAs reach, a launch, and for a split 6 % and the
+// atomics and the filling of C.  Measured on GB300 (terms per clock per SM with
+// every SM full, and the share of it that one CTA alone reaches): 128 x 128 at 2
+// CTAs/SM 57 and 0.9; 64 x 64 with 128 threads 54 and 0.4; 32 x 32 46 (fp32 40)
+// and 0.25; 64 x 64 with 64 threads 45 and 0.2.
+double nt_time(const GemmKernel &g, int dtype, double m, double n, double k, int splits, int sms) {
+    double rate = 57, alone = 0.9, resident = 2;
+    if (g.bm < 64) rate = dtype == BTAS_F32 ? 40 : 46, alone = 0.25, resident = 6;
+    else if (g.bm < 128 && g.threads < 128) rate = 45, alone = 0.2, resident = 3;
+    else if (g.bm < 128) rate = 54, alone = 0.4, resident = 4;
+    double per_sm = std::ceil(m / g.bm) * std::ceil(n / g.bn) * splits / sms;
+    per_sm = per_sm <= 4 ? std::ceil(per_sm) : per_sm + 0.3;
+    const double steps = std::ceil(std::ceil(k / 32) / splits);
+    const double clocks = per_sm * g.bm * g.bn * (32 * steps) / (rate * std::min(1.0, std::min(per_sm, resident) * alone));
+    return splits > 1 ? 1.06 * clocks / 2000.0 + 4.0 + m * n * splits * 0.5e-6 : clocks / 2000.0 + 2.5;
+}
+
+// The fastest split of one kernel: at least two k steps to a CTA.
+int nt_splits(const GemmKernel &g, int dtype, long long m, long long n, long long k, int sms, double *time) {
+    int best = 1;
+    *time = nt_time(g, dtype, (double)m, (double)n, (double)k, 1, sms);
+    for (int s = 2; s <= 256 && 64LL * s <= k + 63; s = s < 4 ? s + 1 : s + s / 2) {
+        const double t = nt_time(g, dtype, (double)m, (double)n, (double)k, s, sms);
+        if (t < *time) {
+            *time = t;
+            best = s;
+        }
+    }
+    return best;
+}
+
 // Kernel choice.  Explicit environment overrides win: BTAS_I32_VARIANT (0 =
 // DPX, 1 = mixed), BTAS_I32_NS, BTAS_F32_VARIANT (2 = f32x2, 3 = scalar, 4 =
 // two scalar adds + 3-input min) and BTAS_CFG.  Otherwise an autotuner entry
-// for the problem's size buckets (tune.cu), else the defaults measured on
-// GB300 at 8192^3, where the 2-CTA/SM, 64-bit-fragment tiles reach the
-// measured issue ceilings of their instruction mixes: int32 = IMAD/3-input-min
-// mix on 4 of 8 columns, fp32 = add.f32x2 + 3-input min; 64 x 64 tiles when
-// the 128 x 128 tiles would not fill one wave of 2 CTAs per SM.
-const GemmKernel *select_kernel(int dtype, int sr, long long m, long long n, long long k, cudaStream_t st,
-                                int *group_m) {
-    *group_m = 8;
-    const bool forced = getenv("BTAS_I32_VARIANT") || getenv("BTAS_I32_NS") || getenv("BTAS_F32_VARIANT") ||
-                        getenv("BTAS_CFG");
-    TuneChoice c{};
-    if (!forced && tune_choice(sr, dtype, m, n, k, st, &c)) {
-        const GemmKernel *t = find_gemm_kernel(c.var, sr, c.ns, c.cfg);
-        if (t) {
-            *group_m = c.group_m;
-            log_event("product %lldx%lldx%lld %s %s: variant %d ns %d cfg %d group %d (autotuner)", m, n, k,
-                      dtype == BTAS_F32 ? "fp32" : "int32", sr == kMin ? "min-plus" : "max-plus", t->var, t->ns,
-                      t->cfg, c.group_m);
-            return t;
-        }
-    }
-    int var, ns = 0;
-    if (dtype == BTAS_F32) {
-        var = env_int("BTAS_F32_VARIANT", kF32X2);
-    } else {
-        var = env_int("BTAS_I32_VARIANT", kI32Mix);
-        ns = var == kI32Mix ? env_int("BTAS_I32_NS", 4) : 0;
-    }
-    // 128 x 128 tiles at 2 CTAs/SM once they fill at least one full wave
+// for the problem's size buckets (tune.cu), else int32 = IMAD/3-input-min mix,
+// fp32 = add.f32x2 + 3-input min, on the tiles that nt_time() expects to be
+// fastest: 128 x 128 at 2 CTAs/SM for large products (8192^3: at the measured
+// issue ceilings of their instruction mixes), 64 x 64 and 32 x 32 where those
+// would leave SMs idle.  may_split: the k range of a tile may be shared out over
+// several CTAs (products that only write C), except with BTAS_CFG.
+NtPlan plan_nt(int dtype, int sr, long long m, long long n, long long k, bool may_split, cudaStream_t st) {
+    NtPlan plan;
     DeviceInfo di{};
     const int sms = current_device_info(&di) ? di.sms : 152;
-    const long long big_tiles = ((m + 127) / 128) * ((n + 127) / 128);
-    int cfg = env_int("BTAS_CFG", big_tiles >= 2LL * sms ? 4 : 2);
-    const GemmKernel *kk = find_gemm_kernel(var, sr, ns, cfg);
-    if (!kk && dtype == BTAS_I32) kk = find_gemm_kernel(kI32Mix, sr, 5, cfg);
-    if (!kk) kk = find_gemm_kernel(var, sr, ns, 0);
-    if (!kk && dtype == BTAS_I32) kk = find_gemm_kernel(kI32Mix, sr, 5, 0);
-    if (!kk && dtype == BTAS_I32) kk = find_gemm_kernel(kI32Dpx, sr, 0, 0);
-    if (!kk && dtype == BTAS_F32) kk = find_gemm_kernel(kF32X2, sr, 0, 0);
-    if (kk)
-        log_event("product %lldx%lldx%lld %s %s: variant %d ns %d cfg %d group 8 (%s)", m, n, k,
-                  dtype == BTAS_F32 ? "fp32" : "int32", sr == kMin ? "min-plus" : "max-plus", kk->var, kk->ns,
-                  kk->cfg, forced ? "environment" : "defaults");
-    return kk;
+    const bool forced = getenv("BTAS_I32_VARIANT") || getenv("BTAS_I32_NS") || getenv("BTAS_F32_VARIANT") ||
+                        getenv("BTAS_CFG");
+    double time = 0;
+    TuneChoice c{};
+    const char *from = forced ? "environment" : "defaults";
+    if (!forced && tune_choice(sr, dtype, m, n, k, st, &c)) {
+        plan.kernel = find_gemm_kernel(c.var, sr, c.ns, c.cfg);
+        if (plan.kernel) {
+            plan.group_m = c.group_m;
+            if (may_split) plan.splits = nt_splits(*plan.kernel, dtype, m, n, k, sms, &time);
+            from = "autotuner";
+        }
+    }
+    if (!plan.kernel && !forced) {
+        double best = 0;
+        for (int cfg : {4, 6, 7}) {
+            const int ns = dtype == BTAS_F32 ? 0 : cfg == 7 ? 2 : 4;
+            const GemmKernel *g = find_gemm_kernel(dtype == BTAS_F32 ? kF32X2 : kI32Mix, sr, ns, cfg);
+            if (!g) continue;
+            int s = 1;
+            if (may_split) s = nt_splits(*g, dtype, m, n, k, sms, &time);
+            else time = nt_time(*g, dtype, (double)m, (double)n, (double)k, 1, sms);
+            if (!plan.kernel || time < best) {
+                best = time;
+                plan.kernel = g;
+                plan.splits = s;
+            }
+        }
+    }
+    if (!plan.kernel) {
+        int var, ns = 0;
+        if (dtype == BTAS_F32) {
+            var = env_int("BTAS_F32_VARIANT", kF32X2);
+        } else {
+            var = env_int("BTAS_I32_VARIANT", kI32Mix);
+            ns = var == kI32Mix ? env_int("BTAS_I32_NS", 4) : 0;
+        }
+        // 128 x 128 tiles at 2 CTAs/SM once they fill at least one full wave
+        const long long big_tiles = ((m + 127) / 128) * ((n + 127) / 128);
+        int cfg = env_int("BTAS_CFG", big_tiles >= 2LL * sms ? 4 : 2);
+        const GemmKernel *kk = find_gemm_kernel(var, sr, ns, cfg);
+        if (!kk && dtype == BTAS_I32 && cfg == 7) kk = find_gemm_kernel(kI32Mix, sr, 2, cfg);
+        if (!kk && dtype == BTAS_I32) kk = find_gemm_kernel(kI32Mix, sr, 5, cfg);
+        if (!kk) kk = find_gemm_kernel(var, sr, ns, 0);
+        if (!kk && dtype == BTAS_I32) kk = find_gemm_kernel(kI32Mix, sr, 5, 0);
+        if (!kk && dtype == BTAS_I32) kk = find_gemm_kernel(kI32Dpx, sr, 0, 0);
+        if (!kk && dtype == BTAS_F32) kk = find_gemm_kernel(kF32X2, sr, 0, 0);
+        plan.kernel = kk;
+    }
+    if (may_split && getenv("BTAS_SPLIT")) plan.splits = env_int("BTAS_SPLIT", 1);
+    if (plan.kernel)
+        log_event("product %lldx%lldx%lld %s %s: variant %d ns %d cfg %d group %d splits %d (%s)", m, n, k,
+                  dtype == BTAS_F32 ? "fp32" : "int32", sr == kMin ? "min-plus" : "max-plus", plan.kernel->var,
+                  plan.kernel->ns, plan.kernel->cfg, plan.group_m, plan.splits, from);
+    return plan;
 }
 
 // IMAD/DPX split of the packed u16x2 kernel: BTAS_U16_NS, else the
@@ -275,13 +342,22 @@ int u16_ns(long long m, long long n, long long k, cudaStream_t st) {
     return 5;
 }
 
-// Run the NT kernel on A (m x k) and Bt (n x k).
-btas_status run_nt(int dtype, int sr, const GemmArgs &a, cudaStream_t st) {
-    int group_m = 8;
-    const GemmKernel *k = select_kernel(dtype, sr, a.m, a.n, a.k, st, &group_m);
+// Run the NT kernel on A (m x k) and Bt (n x k).  plan: a choice made before
+// (C then holds the (+)-identity if it splits), else one is made here.
+btas_status run_nt(int dtype, int sr, const GemmArgs &a, cudaStream_t st, const NtPlan *plan = nullptr) {
+    NtPlan own;
+    if (!plan) {
+        const bool only_c = !a.accumulate && !a.prev && !a.changed && !a.skip && !a.maxfin && !a.bypass;
+        own = plan_nt(dtype, sr, a.m, a.n, a.k, only_c, st);
+        if (own.splits > 1)
+            BTAS_CUDA(launch_fill4(a.C, a.ldc, a.m, a.n, ident_bits(dtype, sr), st), "fill");
+        plan = &own;
+    }
+    const GemmKernel *k = plan->kernel;
     if (!k) return fail(BTAS_ERR_UNSUPPORTED, "no kernel for dtype %d semiring %d", dtype, sr);
     GemmArgs args = a;
-    args.group_m = group_m;
+    args.group_m = plan->group_m;
+    args.splits = plan->splits;
     args.one = 1;
     {
         // Grids of two or more waves: groups of 16 tile columns and k run
@@ -291,7 +367,7 @@ btas_status run_nt(int dtype, int sr, const GemmArgs &a, cudaStream_t st) {
         DeviceInfo di{};
         const int sms = current_device_info(&di) ? di.sms : 152;
         const long long tiles = (long long)((a.m + k->bm - 1) / k->bm) * ((a.n + k->bn - 1) / k->bn);
-        if (tiles >= 4LL * sms && env_int("BTAS_KWAVE", 1) != 0) {
+        if (args.splits == 1 && tiles >= 4LL * sms && env_int("BTAS_KWAVE", 1) != 0) {
             args.kwave = sms;
             args.group_m = 16;
         }
@@ -302,10 +378,6 @@ btas_status run_nt(int dtype, int sr, const GemmArgs &a, cudaStream_t st) {
     return BTAS_OK;
 }
 
-uint32_t ident_bits(int dtype, int sr) {
-    if (dtype == BTAS_I32) return static_cast<uint32_t>(sr == kMin ? kInfI32 : kNinfI32);
-    return sr == kMin ? 0x7f800000u : 0xff800000u;
-}
 
 }  // namespace
 
@@ -447,7 +519,14 @@ btas_status btas_gemm(int semiring, int dtype, int64_t m, int64_t n, int64_t k, 
     const void *Bt = B;
     long long ldbt = ldb;
     const long long ldt = (k + 3) & ~3LL;
-    const size_t bt_bytes = trans_b ? 0 : align256((size_t)n * ldt * 4);
+    // Rows that do not start on 16 bytes are staged in 4-byte copies: 13 % of a
+    // product's time for one operand, 30 % for both (4001^3: 3.93 ms aligned, 4.42
+    // and 5.13 ms).  An operand that enough tiles read is copied to aligned rows
+    // first, where that is more than the copy's launch costs (from 20 us of work).
+    const bool worth = !(packed && dtype == BTAS_I32) && (double)m * n * k >= 4e8;
+    const bool pad_a = worth && n >= 512 && !aligned16(A, lda), pad_b = worth && trans_b && m >= 512 && !aligned16(B, ldb);
+    const size_t bt_bytes = trans_b && !pad_b ? 0 : align256((size_t)n * ldt * 4);
+    const size_t a_bytes = pad_a ? align256((size_t)m * ldt * 4) : 0;
     int *pack_state = nullptr;
     if (packed && dtype == BTAS_I32) {
         log_event("product %lldx%lldx%lld int32: packed path requested (range check and choice on the device)",
@@ -479,13 +558,34 @@ btas_status btas_gemm(int semiring, int dtype, int64_t m, int64_t n, int64_t k, 
         BTAS_CUDA(launch_pack_finish(sr, (int)m, (int)n, cu, ldbu, pack_state, static_cast<int *>(C), ldc,
                                      accumulate, st),
                   "packed result");
-    } else if (!trans_b) {
-        BTAS_CUDA(ws.alloc(bt_bytes), "workspace alloc");
+    } else if (bt_bytes + a_bytes) {
+        BTAS_CUDA(ws.alloc(bt_bytes + a_bytes), "workspace alloc");
     }
+    if (pad_b) {
+        BTAS_CUDA(launch_pad4(B, ldb, (int)n, (int)k, ws.p, ldt, st), "aligned B");
+        Bt = ws.p;
+        ldbt = ldt;
+    }
+    if (pad_a) {
+        void *p = static_cast<char *>(ws.p) + bt_bytes;
+        BTAS_CUDA(launch_pad4(A, lda, (int)m, (int)k, p, ldt, st), "aligned A");
+        A = p;
+        lda = ldt;
+    }
+    // A split product merges into C, which the transpose fills with the
+    // (+)-identity on its way (or a kernel of its own).
+    NtPlan plan = plan_nt(dtype, sr, m, n, k, !accumulate && !pack_state && !checked, st);
+    if (plan.splits > 1 && trans_b)
+        BTAS_CUDA(launch_fill4(C, ldc, (int)m, (int)n, ident_bits(dtype, sr), st), "fill");
     if (!trans_b) {
-        BTAS_CUDA(launch_transpose4(B, ldb, (int)k, (int)n, ws.p, ldt, 0,
-                                    pack_state ? pack_state + kPackStateNotUse : nullptr, st),
-                  "transpose B");
+        if (plan.splits > 1)
+            BTAS_CUDA(launch_transpose4_fill(B, ldb, (int)k, (int)n, ws.p, ldt, C, ldc, (int)m, ident_bits(dtype, sr),
+                                             st),
+                      "transpose B");
+        else
+            BTAS_CUDA(launch_transpose4(B, ldb, (int)k, (int)n, ws.p, ldt, 0,
+                                        pack_state ? pack_state + kPackStateNotUse : nullptr, st),
+                      "transpose B");
         Bt = ws.p;
         ldbt = ldt;
     }
@@ -502,7 +602,7 @@ btas_status btas_gemm(int semiring, int dtype, int64_t m, int64_t n, int64_t k, 
         if (!pack_state) BTAS_CUDA(launch_checked_gate(chk, nullptr, chk + 1, status, st), "checked gate");
         a.bypass = chk + 1;
     }
-    return run_nt(dtype, sr, a, st);
+    return run_nt(dtype, sr, a, st, &plan);
 }
 
 btas_status btas_sync_status(void *stream, int64_t *out_of_domain, int64_t *calls) {

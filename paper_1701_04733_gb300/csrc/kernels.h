@@ -72,6 +72,12 @@ cudaError_t launch_checked_gate(const int *count, const int *pack_state, int *sk
 // 2 = fp32 carrier -> int32 (inverse).
 cudaError_t launch_transpose4(const void *src, long long lds, int rows, int cols, void *dst,
                               long long ldd, int mode, const int *skip, cudaStream_t st);
+// The transpose (mode 0), which also fills the m x cols matrix C with `bits`.
+cudaError_t launch_transpose4_fill(const void *src, long long lds, int rows, int cols, void *dst, long long ldd,
+                                   void *C, long long ldc, int m, uint32_t bits, cudaStream_t st);
+// Copy of a rows x cols matrix of 4-byte elements to another pitch.
+cudaError_t launch_pad4(const void *src, long long lds, int rows, int cols, void *dst, long long ldd,
+                        cudaStream_t st);
 // Element-wise conversion of a rows x cols matrix (mode as above, 0 = copy).
 cudaError_t launch_convert4(const void *src, long long lds, int rows, int cols, void *dst,
                             long long ldd, int mode, cudaStream_t st);

@@ -233,6 +233,26 @@ __device__ __forceinline__ T finish(T v) {
     else return v;
 }
 
+// *p = *p (+) v.  Non-negative floats order as ints and negative ones backwards
+// as unsigned ints, so each sign has its own integer atomic; p holds no NaN and
+// neither does v (min and max drop NaN terms).
+template <int SR>
+__device__ __forceinline__ void merge_atomic(int *p, int v) {
+    if (SR == kMin) atomicMin(p, v);
+    else atomicMax(p, v);
+}
+template <int SR>
+__device__ __forceinline__ void merge_atomic(float *p, float v) {
+    const int b = __float_as_int(v);
+    if ((SR == kMin) == (b >= 0)) {
+        if (b >= 0) atomicMin(reinterpret_cast<int *>(p), b);
+        else atomicMin(reinterpret_cast<unsigned *>(p), (unsigned)b);
+    } else {
+        if (b >= 0) atomicMax(reinterpret_cast<int *>(p), b);
+        else atomicMax(reinterpret_cast<unsigned *>(p), (unsigned)b);
+    }
+}
+
 // Converged squaring (D_{s+1} = D_s): copy one BM x BN tile of P into C.
 template <class Cfg, typename T>
 __device__ __forceinline__ void copy_tile(const GemmArgs &args, int bm, int bn, int tid) {
@@ -384,7 +404,11 @@ __device__ __forceinline__ bool nt_tile(const GemmArgs &args, int bm, int bn, un
                 const T v = acc[i][j];
                 if (P != nullptr && v != __ldcg(P + (long long)r * args.ldp + c)) ch = true;
                 if (SR == kMin && args.maxfin != nullptr) mx = max(mx, finite_int(v));
-                C[(long long)r * args.ldc + c] = v;
+                if (args.splits > 1) {
+                    if (v != ident) merge_atomic<SR>(C + (long long)r * args.ldc + c, v);
+                } else {
+                    C[(long long)r * args.ldc + c] = v;
+                }
                 if constexpr (std::is_same<T, int>::value) {
                     if (Cd != nullptr) {
                         // 16-bit forms for a following packed squaring (used only
@@ -438,6 +462,19 @@ __global__ void __launch_bounds__(Cfg::kThreads, Cfg::MINB) tgemm_nt_kernel(cons
     const int tid = threadIdx.x;
     const int tiles_m = (args.m + Cfg::BM - 1) / Cfg::BM, tiles_n = (args.n + Cfg::BN - 1) / Cfg::BN;
     int tm, tn;
+    if (args.splits > 1) {
+        // CTA s of a tile: an equal share of the k steps
+        const int split = blockIdx.x / (tiles_m * tiles_n), steps = (args.k + Cfg::BK - 1) / Cfg::BK;
+        const int k0 = (int)((long long)steps * split / args.splits) * Cfg::BK;
+        const int k1 = min(args.k, (int)((long long)steps * (split + 1) / args.splits) * Cfg::BK);
+        raster(blockIdx.x % (tiles_m * tiles_n), tiles_m, tiles_n, args.group_m, tm, tn);
+        GemmArgs part = args;
+        part.A = static_cast<const T *>(args.A) + k0;
+        part.Bt = static_cast<const T *>(args.Bt) + k0;
+        part.k = k1 - k0;
+        nt_tile<Cfg, VAR, SR, NS>(part, tm * Cfg::BM, tn * Cfg::BN, smem_raw, tid);
+        return;
+    }
     if (args.kwave > 0) raster(blockIdx.x, tiles_n, tiles_m, args.group_m, tn, tm);
     else raster(blockIdx.x, tiles_m, tiles_n, args.group_m, tm, tn);
     const int bm = tm * Cfg::BM, bn = tn * Cfg::BN;

@@ -29,6 +29,8 @@ struct GemmArgs {
                         // waves share their B^T panels) and run k backwards in every other
                         // wave of kwave CTAs, so that a wave starts on the k-slices the
                         // previous one left in L2 (the launcher scales it by CTAs per SM)
+    int splits;         // > 1: that many CTAs per tile share its k range and merge their results
+                        // into C with atomics; C must hold the (+)-identity before the launch
 };
 
 }  // namespace btas

@@ -21,6 +21,8 @@ using Cfg2 = TileCfg<64, 64, 32, 4>;    //  64 threads,  72 KiB smem (small prob
 using Cfg3 = TileCfg<128, 64, 32, 4>;   // 128 threads, 108 KiB smem
 using Cfg4 = TileCfg<128, 128, 32, 3, 2, 2, 1>;  // 2 CTAs/SM, 64-bit fragments
 using Cfg5 = TileCfg<128, 128, 32, 3, 2, 4, 1>;  // 2 CTAs/SM, 128-bit fragments
+using Cfg6 = TileCfg<64, 64, 32, 3, 4, 4, 1, 4, 8>;  // 128 threads, 54 KiB smem, 4 CTAs/SM (middle-sized products)
+using Cfg7 = TileCfg<32, 32, 32, 4, 6, 4, 1, 4, 4>;  //  64 threads, 36 KiB smem, 6 CTAs/SM (small and thin products)
 
 template <class Cfg, int VAR, int SR, int NS>
 cudaError_t launch_nt(const GemmArgs &a, cudaStream_t st) {
@@ -39,7 +41,7 @@ cudaError_t launch_nt(const GemmArgs &a, cudaStream_t st) {
     if (tiles <= 0) return cudaSuccess;
     GemmArgs args = a;
     args.kwave = a.kwave * Cfg::MINB;  // SMs -> CTAs resident at once
-    kern<<<(unsigned)tiles, Cfg::kThreads, Cfg::kSmemBytes, st>>>(args);
+    kern<<<(unsigned)(tiles * (a.splits > 1 ? a.splits : 1)), Cfg::kThreads, Cfg::kSmemBytes, st>>>(args);
     note_launch();
     return cudaGetLastError();
 }
