@@ -682,6 +682,17 @@ void relax_inst_place(BInst &I, char *mem) {
     I.rl.budget = e && *e ? atoll(e) : 4 * relax::budget_cycles(I.n);
 }
 
+// Vectors of 8 targets a relaxation task solves at once.  Rows of 32 and 64
+// bytes conflict less in shared memory (2.1 and 1.5 cycles for 8 lanes' random
+// rows where 16-byte rows take 2.6 to move as much), but make fewer and longer tasks: as
+// wide as shared memory holds while two tasks per CTA remain.  The 512 graphs of
+// the mixed batch alone: 9.11 ms with 16-byte rows, 7.14 ms with 64-byte ones.
+int relax_rows_for(long long n, long long vectors, long long ctas) {
+    int rows = 1;
+    while (rows < 4 && 16 * n * 2 * rows <= batch_smem_words() * 4 && vectors >= 2 * ctas * 2 * rows) rows *= 2;
+    return rows;
+}
+
 long long batch_timeout_cycles(int device) {
     (void)device;  // the current device
     DeviceInfo d{};
@@ -819,17 +830,6 @@ bool relax_allowed(const btas_batch_t *b) {
         if (e && *e) return false;
     }
     return true;
-}
-
-// Vectors of 8 targets a relaxation task solves at once.  Rows of 32 and 64
-// bytes conflict less in shared memory (2.1 and 1.5 cycles for 8 lanes' random
-// rows where 16-byte rows take 2.6 to move as much), but make fewer and longer tasks: as
-// wide as shared memory holds while two tasks per CTA remain.  The 512 graphs of
-// the mixed batch alone: 9.11 ms with 16-byte rows, 7.14 ms with 64-byte ones.
-int relax_rows_for(long long n, long long vectors, long long ctas) {
-    int rows = 1;
-    while (rows < 4 && 16 * n * 2 * rows <= batch_smem_words() * 4 && vectors >= 2 * ctas * 2 * rows) rows *= 2;
-    return rows;
 }
 
 btas_status build_plan(btas_batch_t *b) {

@@ -129,5 +129,8 @@ long long batch_timeout_cycles(int device);
 // (relax_inst_bytes(n) bytes, not initialised).
 size_t relax_inst_bytes(long long n);
 void relax_inst_place(BInst &I, char *mem);
+// Vectors of 8 targets per relaxation task, with `vectors` of them in all and
+// `ctas` resident CTAs.
+int relax_rows_for(long long n, long long vectors, long long ctas);
 
 }  // namespace btas

@@ -16,10 +16,12 @@
 //             cap contributes a chunk of its 128 x 128 output tiles and
 //             continues in the next step, so every step stays short; units
 //             below 5 % of the cap always join.  Short steps let finished
-//             requests leave and new ones join often.  An APSP request with
-//             n <= 1792 is one unit instead when the rest of the work is
-//             light: the whole solve, by the one-block or the cooperative
-//             kernel, launched after the persistent kernel;
+//             requests leave and new ones join often.  An APSP request starts
+//             as one unit of its own kind, the whole solve by relaxation over
+//             sorted edge lists (relax.cuh) as tasks of the same launch; only
+//             one that the relaxation gives up goes on by squarings, or, with
+//             n <= 1792 and light other work, by the one-block or the
+//             cooperative kernel, launched after the persistent kernel;
 //   retire  - a product is finished after its step; an APSP solve after its
 //             last squaring or as soon as a squaring changed nothing (early
 //             exit, same result).  Its result is copied back on the copy
@@ -97,6 +99,9 @@ struct Req {
     int tile_next = 0;   // output tiles of the current unit done in earlier steps
     int take = 0;        // output tiles of the current unit in this step
     bool finished = false;
+    bool relax = false;      // APSP solved by relaxation in this step
+    bool no_relax = false;   // the relaxation was given up
+    int relax_slot = 0;
     bool whole = false;  // APSP solved in one unit (small / cooperative kernel) in this step
     bool bulk = false;   // large request: runs in the bulk lane through the single calls
     bool bad = false;    // W outside the domain (checked on the device before the first squaring): the request fails
@@ -136,6 +141,7 @@ struct btas_server_t {
     void *h_stage[2] = {nullptr, nullptr};
     size_t stage_bytes = 0;
     int *h_flags = nullptr;  // pinned mailbox: change flags, maxima or barrier status, domain-scan results
+    int *h_rstat = nullptr;  // pinned: kRelaxWords words per relaxation of a step
     int *d_flag_slots = nullptr;
     int flag_slots = 0;
     cudaEvent_t step_done[2] = {nullptr, nullptr};
@@ -149,6 +155,7 @@ struct btas_server_t {
     int64_t steps = 0;
     int64_t units = 0;
     int64_t completed = 0;
+    int64_t in_flight = 0;  // submitted and not ended; under mu (the lists above are their threads' own)
     int last_error = 0;
 
     double now() const {
@@ -176,6 +183,8 @@ int squarings_of(long long n) {
 size_t footprint(const Req &r) {
     if (r.kind == 0) {
         const long long ld = r4(r.n), ldu = (r.n + 7) & ~7LL;
+        // (a relaxation's lists, about 8 n min(n, 512) bytes, lie in the space of the
+        // squarings' other buffers: 16 n n bytes and more)
         return 6 * a256((size_t)r.n * ld * 4) + 2 * a256((size_t)r.n * ldu * 2) + a256((size_t)(2 * r.S + 6) * 4);
     }
     return a256((size_t)r.m * r4(r.k) * 4) + a256((size_t)r.k * r4(r.n) * 4) + a256((size_t)r.n * r4(r.k) * 4) +
@@ -262,6 +271,18 @@ int launch_step(btas_server_t *sv, std::vector<Req *> &units) {
         r->whole = sv->allow_whole && r->kind == 0 && r->s == 1 && r->tile_next == 0 && r->n <= apsp_mid_max_n() &&
                    pending - r->unit_terms() < sv->whole_below && (r->n <= apsp_small_limit() || !bulk_busy);
         r->take = 0;
+        r->relax = sv->allow_whole && r->kind == 0 && r->s == 1 && r->tile_next == 0 && !r->no_relax && r->n >= 16 &&
+                   r->n <= kRelaxBatchMaxN;
+        if (r->relax) {
+            // its shared-memory work, as the terms a product computes meanwhile
+            // (n = 1024: about 35 us of the whole GPU)
+            const double w = 600.0 * r->n * r->n;
+            r->whole = false;
+            if (!units.empty() && terms + w > cap && w >= small) continue;
+            units.push_back(r);
+            terms += w;
+            continue;
+        }
         if (r->whole) {
             const double w = r->unit_terms() * std::min(r->S, 6);
             if (!units.empty() && terms + w > cap && w >= small) continue;
@@ -293,6 +314,10 @@ int launch_step(btas_server_t *sv, std::vector<Req *> &units) {
     while (ninst < (int)units.size() && !units[ninst]->whole) ++ninst;
     std::vector<BInst> insts(ninst);
     std::vector<int4> tasks;
+    int nrelax = 0;
+    long long vectors = 0;  // 16-byte vectors of 8 targets, over all relaxations
+    for (int i = 0; i < ninst; ++i)
+        if (units[i]->relax) vectors += (units[i]->n + 7) / 8;
     for (int i = 0; i < ninst; ++i) {
         Req *r = units[i];
         cudaStreamWaitEvent(sv->compute, r->in_ready, 0);
@@ -301,7 +326,18 @@ int launch_step(btas_server_t *sv, std::vector<Req *> &units) {
         I.flag_base = 2 * i;
         I.levels = 1;
         const bool first_chunk = r->tile_next == 0;
-        if (r->kind == 0) {
+        if (r->relax) {
+            I.kind = kInstRelax;
+            I.m = I.n = I.k = r->n;
+            I.A = r->P[0];
+            I.lda = r->ldp;
+            I.C = r->P[1];
+            I.ldc = r->ldp;
+            I.checked = 1;
+            I.relax_rows = relax_rows_for(r->n, vectors, sv->grid);
+            relax_inst_place(I, static_cast<char *>(r->Q[0]));  // fits: see footprint()
+            r->relax_slot = nrelax++;
+        } else if (r->kind == 0) {
             const int s = r->s;
             I.kind = kInstSquare;
             I.sr = kMin;
@@ -371,7 +407,12 @@ int launch_step(btas_server_t *sv, std::vector<Req *> &units) {
     for (int level = 0; level <= 1; ++level)
         for (int i = 0; i < ninst; ++i) {
             const BInst &I = insts[i];
-            if (level == 0) {
+            if (I.kind == kInstRelax) {
+                if (level == 0)
+                    for (int t = 0; t * kRelaxTaskRows < I.n; ++t) tasks.push_back(make_int4(kTaskRelaxLists, i, 0, t));
+                else
+                    for (int t = 0; 8 * I.relax_rows * t < I.n; ++t) tasks.push_back(make_int4(kTaskRelax, i, 1, t));
+            } else if (level == 0) {
                 if (I.t0_rows > 0) {
                     const int nt = ((I.t0_rows + kBT - 1) / kBT) * ((I.t0_cols + kBT - 1) / kBT);
                     for (int t = 0; t < nt; ++t) tasks.push_back(make_int4(kTaskTranspose, i, 0, t));
@@ -383,8 +424,10 @@ int launch_step(btas_server_t *sv, std::vector<Req *> &units) {
                 for (int t = t0; t < t1; ++t) tasks.push_back(make_int4(type, i, 1, t));
             }
         }
-    // staging: [counters (next, status, done[2*ninst], changed[2*ninst]) | insts | tasks]
-    const size_t cnt_bytes = a256((size_t)(2 + 4 * ninst) * 4);
+    // staging: [counters (next, status, done[2*ninst], changed[2*ninst], relaxation tasks
+    // done, solves given up, the relaxations' words) | insts | tasks]
+    const int rstat_at = 2 + 4 * ninst + 2;
+    const size_t cnt_bytes = a256((size_t)(rstat_at + kRelaxWords * nrelax) * 4);
     const size_t inst_bytes = a256((size_t)ninst * sizeof(BInst));
     const size_t task_bytes = a256(tasks.size() * sizeof(int4));
     const size_t need = cnt_bytes + inst_bytes + task_bytes;
@@ -405,6 +448,8 @@ int launch_step(btas_server_t *sv, std::vector<Req *> &units) {
     char *h = static_cast<char *>(sv->h_stage[par]);
     char *d = static_cast<char *>(sv->d_stage[par]);
     memset(h, 0, cnt_bytes);
+    for (int i = 0; i < ninst; ++i)
+        if (units[i]->relax) insts[i].rstat = reinterpret_cast<int *>(d) + rstat_at + kRelaxWords * units[i]->relax_slot;
     memcpy(h + cnt_bytes, insts.data(), (size_t)ninst * sizeof(BInst));
     memcpy(h + cnt_bytes + inst_bytes, tasks.data(), tasks.size() * sizeof(int4));
     cudaMemcpyAsync(d, h, need, cudaMemcpyHostToDevice, sv->compute);
@@ -419,13 +464,14 @@ int launch_step(btas_server_t *sv, std::vector<Req *> &units) {
     p.total = (int)tasks.size();
     p.timeout_cycles = sv->timeout_cycles;
     p.withhold_inst = -1;
-    p.fallback_start = p.total;
+    p.fallback_start = p.total;  // given-up solves go on in later steps
+    p.relax_done = cnt + 2 + 4 * ninst;
     const int grid = std::max(1, std::min(sv->grid, p.total));
     if (launch_batch_kernel(p, grid, sv->compute) != cudaSuccess) return -1;
     // change flags and largest finite entries of this step's squarings ->
     // pinned mailbox
     for (int i = 0; i < ninst; ++i) {
-        if (units[i]->kind != 0) continue;
+        if (units[i]->kind != 0 || units[i]->relax) continue;
         sv->h_flags[2 * sv->flag_slots + 1 + i] = 0;
         if (units[i]->s == 1)
             cudaMemcpyAsync(sv->h_flags + 2 * sv->flag_slots + 1 + i, units[i]->dflag + 2 * units[i]->S + 5, 4,
@@ -435,6 +481,9 @@ int launch_step(btas_server_t *sv, std::vector<Req *> &units) {
                         cudaMemcpyDeviceToHost, sv->compute);
     }
     cudaMemcpyAsync(sv->h_flags + sv->flag_slots, p.status, 4, cudaMemcpyDeviceToHost, sv->compute);
+    if (nrelax > 0)
+        cudaMemcpyAsync(sv->h_rstat, cnt + rstat_at, (size_t)kRelaxWords * nrelax * 4, cudaMemcpyDeviceToHost,
+                        sv->compute);
     } else {
         sv->h_flags[sv->flag_slots] = 0;
     }
@@ -493,6 +542,7 @@ void poll_retiring(btas_server_t *sv, bool block) {
             r->state = r->bad ? kFailed : kDone;
             sv->used -= (long long)r->bytes;
             ++sv->completed;
+            --sv->in_flight;
         } else {
             keep.push_back(r);
         }
@@ -586,6 +636,7 @@ void bulk_loop(btas_server_t *sv) {
             r->state = ok ? kDone : kFailed;
             sv->used -= (long long)r->bytes;
             ++sv->completed;
+            --sv->in_flight;
             ++sv->bulk_runs;
             sv->bulk_busy = false;
         }
@@ -617,6 +668,7 @@ void admit_queued(btas_server_t *sv, bool wait_if_idle) {
             if (!ok) {
                 r->state = kFailed;
                 sv->used -= (long long)r->bytes;
+                --sv->in_flight;
             } else {
                 r->state = kRunning;
             }
@@ -659,7 +711,14 @@ void worker_loop(btas_server_t *sv) {
             Req *r = units[i];
             ++r->steps;
             bool finished = true;
-            if (r->whole) {
+            if (r->relax) {
+                const int *w = sv->h_rstat + kRelaxWords * r->relax_slot;
+                r->bad = w[kRelaxBadEntries] != 0;
+                r->no_relax = w[kRelaxGaveUpWord] != 0;
+                if (!r->bad && r->no_relax) continue;  // by squarings from the next step on
+                r->result_buf = 1;
+                r->s = r->S + 1;
+            } else if (r->whole) {
                 // the one-block kernel reports no barrier status (its slot stays 0)
                 r->bad = sv->h_flags[i] != 0 || (r->n > apsp_small_limit() && sv->h_flags[sv->flag_slots + 1 + i] != 0);
                 r->result_buf = 1;
@@ -730,7 +789,10 @@ btas_status btas_server_create(btas_server_t **out, int64_t hbm_budget_bytes, in
     if (const char *e = getenv("BTAS_SERVER_BULK_TERMS")) sv->bulk_terms = atof(e);
     sv->timeout_cycles = batch_timeout_cycles(sv->device);
     sv->flag_slots = 1 << 16;
-    if (cudaMallocHost(reinterpret_cast<void **>(&sv->h_flags), (size_t)(3 * sv->flag_slots + 1) * 4) != cudaSuccess) {
+    if (cudaMallocHost(reinterpret_cast<void **>(&sv->h_flags), (size_t)(3 * sv->flag_slots + 1) * 4) != cudaSuccess ||
+        cudaMallocHost(reinterpret_cast<void **>(&sv->h_rstat), (size_t)kRelaxWords * sv->flag_slots * 4) !=
+            cudaSuccess) {
+        if (sv->h_flags) cudaFreeHost(sv->h_flags);
         delete sv;
         return sfail(BTAS_ERR_NOMEM, "btas_server_create: pinned mailbox");
     }
@@ -755,10 +817,11 @@ static btas_status enqueue(btas_server_t *sv, Req *r, int64_t *ticket) {
         delete r;
         return sfail(BTAS_ERR_ARG, "btas_server: server is stopping");
     }
-    if ((int64_t)sv->active.size() + (int64_t)sv->queue.size() + (int64_t)sv->bulk_queue.size() >= sv->flag_slots) {
+    if (sv->in_flight >= sv->flag_slots) {
         delete r;
         return sfail(BTAS_ERR_BUDGET, "btas_server: too many requests in flight");
     }
+    ++sv->in_flight;
     r->id = sv->next_id++;
     r->t_submit = sv->now();
     // large requests take the bulk lane (BTAS_SERVER_BULK_TERMS <= 0 turns it off)
@@ -868,6 +931,7 @@ btas_status btas_server_destroy(btas_server_t *sv) {
         if (sv->step_done[q]) cudaEventDestroy(sv->step_done[q]);
     }
     if (sv->h_flags) cudaFreeHost(sv->h_flags);
+    if (sv->h_rstat) cudaFreeHost(sv->h_rstat);
     cudaStreamSynchronize(sv->copy);
     cudaStreamDestroy(sv->compute);
     cudaStreamDestroy(sv->copy);
