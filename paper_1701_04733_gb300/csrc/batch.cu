@@ -693,6 +693,13 @@ int relax_rows_for(long long n, long long vectors, long long ctas) {
     return rows;
 }
 
+// A small task takes about a third of a large one (twice the shared-memory loads
+// per term), and the last round of either runs as long as a whole one.
+bool small_tiles_pay(long long tiles, long long ctas) {
+    const long long large = (tiles + ctas - 1) / ctas, small = (4 * tiles + ctas - 1) / ctas;
+    return 3 * large > small + 1;
+}
+
 long long batch_timeout_cycles(int device) {
     (void)device;  // the current device
     DeviceInfo d{};
@@ -795,12 +802,13 @@ int table_tile(int dev, int kind, long long n) {
     return it == g_tile_table.end() ? 0 : it->second;
 }
 
-int choose_tile(const btas_batch_t *b, int dev, const BInst &I) {
+// few: the batch's products are too few 128 x 128 tiles for the grid.
+int choose_tile(const btas_batch_t *b, int dev, const BInst &I, bool few) {
     if (b->force_tile) return b->force_tile;
     const char *e = getenv("BTAS_BATCH_TILE");
     if (e && *e) return atoi(e) == kBTSmall ? kBTSmall : kBT;
     const int t = table_tile(dev, tile_kind(I), std::max(I.m, I.n));
-    return t == kBTSmall ? kBTSmall : kBT;
+    return t == kBTSmall || (t == 0 && few && I.kind == kInstGemm) ? kBTSmall : kBT;
 }
 
 void release_plan(btas_batch_t *b) {
@@ -874,8 +882,12 @@ btas_status build_plan(btas_batch_t *b) {
     cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
     const long long grid_ctas = (long long)per_sm * sms;
     long long relax_vectors = 0;  // 16-byte vectors of 8 targets, over all relaxations
-    for (const BInst &I : all)
+    long long gemm_tiles = 0;
+    for (const BInst &I : all) {
         if (I.kind == kInstRelax) relax_vectors += (I.n + 7) / 8;
+        if (I.kind == kInstGemm) gemm_tiles += (long long)I.tiles_m * I.tiles_n;
+    }
+    const bool few = small_tiles_pay(gemm_tiles, grid_ctas);
     // workspace per instance and counter bases
     std::vector<BInst> insts(ninst);
     size_t ws = 0;
@@ -892,7 +904,7 @@ btas_status build_plan(btas_batch_t *b) {
     const long long cert_min_n = (cert_min && *cert_min) ? atoll(cert_min) : 256;
     for (size_t i = 0; i < ninst; ++i) {
         BInst I = all[i];
-        I.tile = choose_tile(b, dev, I);
+        I.tile = choose_tile(b, dev, I, few);
         I.tiles_m = (I.m + I.tile - 1) / I.tile;
         I.tiles_n = (I.n + I.tile - 1) / I.tile;
         ws_off[i] = ws;

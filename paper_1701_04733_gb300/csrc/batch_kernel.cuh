@@ -129,6 +129,9 @@ long long batch_timeout_cycles(int device);
 // (relax_inst_bytes(n) bytes, not initialised).
 size_t relax_inst_bytes(long long n);
 void relax_inst_place(BInst &I, char *mem);
+// Whether `tiles` 128 x 128 tasks of about the same length finish sooner on `ctas`
+// CTAs as four 64 x 64 tasks each.
+bool small_tiles_pay(long long tiles, long long ctas);
 // Vectors of 8 targets per relaxation task, with `vectors` of them in all and
 // `ctas` resident CTAs.
 int relax_rows_for(long long n, long long vectors, long long ctas);

@@ -314,6 +314,12 @@ int launch_step(btas_server_t *sv, std::vector<Req *> &units) {
     while (ninst < (int)units.size() && !units[ninst]->whole) ++ninst;
     std::vector<BInst> insts(ninst);
     std::vector<int4> tasks;
+    // 64 x 64 output tiles for whole products while 128 x 128 ones would leave CTAs
+    // idle (see small_tiles_pay)
+    long long tiles128 = 0;
+    for (int i = 0; i < ninst; ++i)
+        if (!units[i]->relax) tiles128 += units[i]->take;
+    const bool small_tiles = small_tiles_pay(tiles128, sv->grid);
     int nrelax = 0;
     long long vectors = 0;  // 16-byte vectors of 8 targets, over all relaxations
     for (int i = 0; i < ninst; ++i)
@@ -383,8 +389,9 @@ int launch_step(btas_server_t *sv, std::vector<Req *> &units) {
             I.m = r->m;
             I.n = r->n;
             I.k = r->k;
-            I.tiles_m = (r->m + kBT - 1) / kBT;
-            I.tiles_n = (r->n + kBT - 1) / kBT;
+            I.tile = small_tiles && r->take == r->unit_tiles() ? kBTSmall : kBT;
+            I.tiles_m = (r->m + I.tile - 1) / I.tile;
+            I.tiles_n = (r->n + I.tile - 1) / I.tile;
             I.A = r->dA;
             I.lda = r->lda_d;
             I.B = r->dB;
@@ -420,7 +427,8 @@ int launch_step(btas_server_t *sv, std::vector<Req *> &units) {
             } else {
                 // this step's chunk of the unit's output tiles
                 const int type = I.kind == kInstSquare ? kTaskSquare : kTaskGemm;
-                const int t0 = units[i]->tile_next, t1 = t0 + units[i]->take;
+                const int t0 = units[i]->tile_next;
+                const int t1 = I.tile == kBTSmall ? I.tiles_m * I.tiles_n : t0 + units[i]->take;
                 for (int t = t0; t < t1; ++t) tasks.push_back(make_int4(type, i, 1, t));
             }
         }
