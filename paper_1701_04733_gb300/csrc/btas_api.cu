@@ -227,26 +227,30 @@ uint32_t ident_bits(int dtype, int sr) {
 struct NtPlan {
     const GemmKernel *kernel = nullptr;
     int group_m = 8;
-    int splits = 1;
+    int splits = 1;    // CTAs to a tile
+    int stream_k = 0;  // or equal shares of all (tile, k step) units, for so many CTAs
+    bool merges() const { return splits > 1 || stream_k > 0; }
 };
 
 // Expected time (us) of an m x n x k product with a kernel's tiles, `splits` CTAs
-// to a tile: the busiest SM's CTAs (with many of them, the mean and a bit) at the
-// rate that so many resident CTAs reach, a launch, and for a split 6 % and the
-// atomics and the filling of C.  Measured on GB300 (terms per clock per SM with
-// every SM full, and the share of it that one CTA alone reaches): 128 x 128 at 2
-// CTAs/SM 57 and 0.9; 64 x 64 with 128 threads 54 and 0.4; 32 x 32 46 (fp32 40)
-// and 0.25; 64 x 64 with 64 threads 45 and 0.2.
+// to a tile: the busiest SM's CTAs at the rate that so many resident CTAs reach,
+// a launch, and for a split the atomics and the filling of C.  Measured on GB300,
+// in terms per 0.5 ns and SM with every SM full, and the share of it that one
+// CTA alone reaches: 128 x 128 tiles at 2 CTAs/SM 66 (int32) and 62 (fp32), 59
+// where parts of a tile are merged, and 0.85; 64 x 64 with 128 threads 59 and
+// 55.5, merged 56.5 and 55, and 0.4; 32 x 32 46 and 40, merged 43 and 38, and
+// 0.25; 64 x 64 with 64 threads 45 and 0.2.
 double nt_time(const GemmKernel &g, int dtype, double m, double n, double k, int splits, int sms) {
-    double rate = 57, alone = 0.9, resident = 2;
-    if (g.bm < 64) rate = dtype == BTAS_F32 ? 40 : 46, alone = 0.25, resident = 6;
+    const bool f32 = dtype == BTAS_F32, merged = splits > 1;
+    double rate = merged ? 59 : f32 ? 62 : 66, alone = 0.85, resident = 2;
+    if (g.bm < 64) rate = f32 ? (merged ? 38 : 40) : (merged ? 43 : 46), alone = 0.25, resident = 6;
     else if (g.bm < 128 && g.threads < 128) rate = 45, alone = 0.2, resident = 3;
-    else if (g.bm < 128) rate = 54, alone = 0.4, resident = 4;
-    double per_sm = std::ceil(m / g.bm) * std::ceil(n / g.bn) * splits / sms;
-    per_sm = per_sm <= 4 ? std::ceil(per_sm) : per_sm + 0.3;
+    else if (g.bm < 128) rate = f32 ? (merged ? 55 : 55.5) : (merged ? 56.5 : 59), alone = 0.4, resident = 4;
+    const double per_sm = std::ceil(std::ceil(m / g.bm) * std::ceil(n / g.bn) * splits / sms);
     const double steps = std::ceil(std::ceil(k / 32) / splits);
-    const double clocks = per_sm * g.bm * g.bn * (32 * steps) / (rate * std::min(1.0, std::min(per_sm, resident) * alone));
-    return splits > 1 ? 1.06 * clocks / 2000.0 + 4.0 + m * n * splits * 0.5e-6 : clocks / 2000.0 + 2.5;
+    const double us = per_sm * g.bm * g.bn * (32 * steps) / (rate * std::min(1.0, std::min(per_sm, resident) * alone)) /
+                      2000.0;
+    return us + (merged ? 4.0 + m * n * splits * 0.5e-6 : 2.5);
 }
 
 // The fastest split of one kernel: at least two k steps to a CTA.
@@ -261,6 +265,15 @@ int nt_splits(const GemmKernel &g, int dtype, long long m, long long n, long lon
         }
     }
     return best;
+}
+
+// Expected time of the 128 x 128 tiles with equal shares of all (tile, k step)
+// units for every resident CTA: no idle SMs, but each part of a tile pays for its
+// own first loads and its merge (about two k steps).
+double nt_stream_time(double m, double n, double k, int sms) {
+    const double tiles = std::ceil(m / 128) * std::ceil(n / 128), ctas = 2.0 * sms;
+    const double steps = tiles * std::ceil(k / 32) / ctas + 2.2 * (1 + tiles / ctas);
+    return steps * 32 * 128 * 128 * 2 / 59 / 2000.0 + 4.0 + m * n * 0.5e-6;
 }
 
 // Kernel choice.  Explicit environment overrides win: BTAS_I32_VARIANT (0 =
@@ -285,7 +298,7 @@ NtPlan plan_nt(int dtype, int sr, long long m, long long n, long long k, bool ma
         plan.kernel = find_gemm_kernel(c.var, sr, c.ns, c.cfg);
         if (plan.kernel) {
             plan.group_m = c.group_m;
-            if (may_split) plan.splits = nt_splits(*plan.kernel, dtype, m, n, k, sms, &time);
+            if (may_split && plan.kernel->merges) plan.splits = nt_splits(*plan.kernel, dtype, m, n, k, sms, &time);
             from = "autotuner";
         }
     }
@@ -303,6 +316,13 @@ NtPlan plan_nt(int dtype, int sr, long long m, long long n, long long k, bool ma
                 plan.kernel = g;
                 plan.splits = s;
             }
+        }
+        // shares of at least four k steps
+        if (may_split && ((m + 127) / 128) * ((n + 127) / 128) * ((k + 31) / 32) >= 8LL * sms &&
+            nt_stream_time((double)m, (double)n, (double)k, sms) < best) {
+            plan.kernel = find_gemm_kernel(dtype == BTAS_F32 ? kF32X2 : kI32Mix, sr, dtype == BTAS_F32 ? 0 : 4, 4);
+            plan.splits = 1;
+            plan.stream_k = 2 * sms;
         }
     }
     if (!plan.kernel) {
@@ -325,11 +345,16 @@ NtPlan plan_nt(int dtype, int sr, long long m, long long n, long long k, bool ma
         if (!kk && dtype == BTAS_F32) kk = find_gemm_kernel(kF32X2, sr, 0, 0);
         plan.kernel = kk;
     }
-    if (may_split && getenv("BTAS_SPLIT")) plan.splits = env_int("BTAS_SPLIT", 1);
+    // BTAS_SPLIT: this many CTAs to a tile, or with 0 equal shares of all units (BTAS_CFG=4)
+    if (may_split && getenv("BTAS_SPLIT")) {
+        const int split = plan.kernel && plan.kernel->merges ? env_int("BTAS_SPLIT", 1) : 1;
+        plan.splits = std::max(1, split);
+        plan.stream_k = split == 0 && plan.kernel->cfg == 4 ? 2 * sms : 0;
+    }
     if (plan.kernel)
-        log_event("product %lldx%lldx%lld %s %s: variant %d ns %d cfg %d group %d splits %d (%s)", m, n, k,
+        log_event("product %lldx%lldx%lld %s %s: variant %d ns %d cfg %d group %d splits %d shares %d (%s)", m, n, k,
                   dtype == BTAS_F32 ? "fp32" : "int32", sr == kMin ? "min-plus" : "max-plus", plan.kernel->var,
-                  plan.kernel->ns, plan.kernel->cfg, plan.group_m, plan.splits, from);
+                  plan.kernel->ns, plan.kernel->cfg, plan.group_m, plan.splits, plan.stream_k, from);
     return plan;
 }
 
@@ -349,7 +374,7 @@ btas_status run_nt(int dtype, int sr, const GemmArgs &a, cudaStream_t st, const 
     if (!plan) {
         const bool only_c = !a.accumulate && !a.prev && !a.changed && !a.skip && !a.maxfin && !a.bypass;
         own = plan_nt(dtype, sr, a.m, a.n, a.k, only_c, st);
-        if (own.splits > 1)
+        if (own.merges())
             BTAS_CUDA(launch_fill4(a.C, a.ldc, a.m, a.n, ident_bits(dtype, sr), st), "fill");
         plan = &own;
     }
@@ -358,6 +383,7 @@ btas_status run_nt(int dtype, int sr, const GemmArgs &a, cudaStream_t st, const 
     GemmArgs args = a;
     args.group_m = plan->group_m;
     args.splits = plan->splits;
+    args.stream_k = plan->stream_k;
     args.one = 1;
     {
         // Grids of two or more waves: groups of 16 tile columns and k run
@@ -367,7 +393,7 @@ btas_status run_nt(int dtype, int sr, const GemmArgs &a, cudaStream_t st, const 
         DeviceInfo di{};
         const int sms = current_device_info(&di) ? di.sms : 152;
         const long long tiles = (long long)((a.m + k->bm - 1) / k->bm) * ((a.n + k->bn - 1) / k->bn);
-        if (args.splits == 1 && tiles >= 4LL * sms && env_int("BTAS_KWAVE", 1) != 0) {
+        if (!plan->merges() && tiles >= 4LL * sms && env_int("BTAS_KWAVE", 1) != 0) {
             args.kwave = sms;
             args.group_m = 16;
         }
@@ -575,10 +601,10 @@ btas_status btas_gemm(int semiring, int dtype, int64_t m, int64_t n, int64_t k, 
     // A split product merges into C, which the transpose fills with the
     // (+)-identity on its way (or a kernel of its own).
     NtPlan plan = plan_nt(dtype, sr, m, n, k, !accumulate && !pack_state && !checked, st);
-    if (plan.splits > 1 && trans_b)
+    if (plan.merges() && trans_b)
         BTAS_CUDA(launch_fill4(C, ldc, (int)m, (int)n, ident_bits(dtype, sr), st), "fill");
     if (!trans_b) {
-        if (plan.splits > 1)
+        if (plan.merges())
             BTAS_CUDA(launch_transpose4_fill(B, ldb, (int)k, (int)n, ws.p, ldt, C, ldc, (int)m, ident_bits(dtype, sr),
                                              st),
                       "transpose B");

@@ -40,6 +40,7 @@ struct GemmKernel {
     int cfg;      // tile configuration id
     int bm, bn, threads, smem;
     cudaError_t (*launch)(const GemmArgs &, cudaStream_t);
+    bool merges;  // takes GemmArgs::splits and stream_k
 };
 const GemmKernel *find_gemm_kernel(int var, int sr, int ns, int cfg);
 int gemm_kernel_count();

@@ -25,9 +25,9 @@
 // lanes/SM/clock, as do FMNMX and IMAD; 3-input min/max does two
 // reductions per issue):
 //   kI32Dpx    one __viaddmin/__viaddmax_s32 per term (ALU pipe only)
-//   kI32Mix    per k-pair and output: on NS of the 8 columns, two IMAD adds
-//              (FMA pipe) + one 3-input min; DPX on the others, balancing the
-//              ALU and FMA pipes
+//   kI32Mix    per k-pair and output: on NS of 8 outputs (a checkerboard where that
+//              is half, else columns), two IMAD adds (FMA pipe) + one 3-input min;
+//              DPX on the others, balancing the ALU and FMA pipes
 //   kF32X2     add.f32x2 (two RN adds, FMA pipe) + one 3-input min.f32
 //   kF32Add2   two scalar RN adds + one 3-input min.f32 per k pair
 //   kF32Scalar FADD + FMNMX per term (reference variant)
@@ -121,6 +121,33 @@ __device__ __forceinline__ uint64_t pack64(uint32_t lo, uint32_t hi) {
     return d;
 }
 
+// Orders in which a step visits its TM x TN outputs.  Terms are bound by the
+// register operands that a scheduler can read per clock, and an operand that the
+// next instruction takes in the same place again is not read twice; so the order
+// of the outputs, and which of two kinds of instruction each takes, decide a tenth
+// of the rate.  Measured at 6144^3 (GB300): int32 12.15 ms with the two kinds
+// alternating like a checkerboard over pairs of columns walked in zigzag, 13.03 to
+// 13.44 ms row by row with IMAD on the first 4 of 8 columns, 12.3 to 13.2 ms for
+// six other patterns in six orders; fp32 12.92 ms with rows walked to and fro, 13.00 ms
+// row by row, 13.27 ms by columns, 13.2 ms and more with scalar adds mixed in.
+template <int TM, int TN, class F>
+__device__ __forceinline__ void visit_zigzag(F f) {  // columns j, j + 1 together, down the rows
+#pragma unroll
+    for (int j = 0; j < TN; j += 2)
+#pragma unroll
+        for (int i = 0; i < TM; ++i) {
+            f(i, j + (i & 1));
+            f(i, j + 1 - (i & 1));
+        }
+}
+template <int TM, int TN, class F>
+__device__ __forceinline__ void visit_snake(F f) {  // rows, every other one backwards
+#pragma unroll
+    for (int i = 0; i < TM; ++i)
+#pragma unroll
+        for (int j = 0; j < TN; ++j) f(i, (i & 1) ? TN - 1 - j : j);
+}
+
 // One FK-deep k slice of the TM x TN register tile.
 template <int VAR, int SR, int NS, int FK, int TM, int TN>
 struct Step;
@@ -144,20 +171,18 @@ struct Step<kI32Mix, SR, NS, FK, TM, TN> {
                                                const Frag32<FK> (&b)[TN], int one) {
 #pragma unroll
         for (int p = 0; p < FK / 2; ++p)
-#pragma unroll
-            for (int i = 0; i < TM; ++i)
-#pragma unroll
-                for (int j = 0; j < TN; ++j) {
-                    const int a0 = (int)a[i].v[2 * p], a1 = (int)a[i].v[2 * p + 1];
-                    const int b0 = (int)b[j].v[2 * p], b1 = (int)b[j].v[2 * p + 1];
-                    if (j < NS) {
-                        const int s0 = imad_add(a0, one, b0);
-                        const int s1 = imad_add(a1, one, b1);
-                        acc[i][j] = isel3<SR>(acc[i][j], s0, s1);
-                    } else {
-                        acc[i][j] = iaddsel<SR>(a1, b1, iaddsel<SR>(a0, b0, acc[i][j]));
-                    }
+            visit_zigzag<TM, TN>([&](int i, int j) {
+                const int a0 = (int)a[i].v[2 * p], a1 = (int)a[i].v[2 * p + 1];
+                const int b0 = (int)b[j].v[2 * p], b1 = (int)b[j].v[2 * p + 1];
+                // half of the outputs: a checkerboard
+                if (2 * NS == TN ? ((i + j) & 1) != 0 : j < NS) {
+                    const int s0 = imad_add(a0, one, b0);
+                    const int s1 = imad_add(a1, one, b1);
+                    acc[i][j] = isel3<SR>(acc[i][j], s0, s1);
+                } else {
+                    acc[i][j] = iaddsel<SR>(a1, b1, iaddsel<SR>(a0, b0, acc[i][j]));
                 }
+            });
     }
 };
 
@@ -167,16 +192,13 @@ struct Step<kF32X2, SR, NS, FK, TM, TN> {
                                                const Frag32<FK> (&b)[TN], int) {
 #pragma unroll
         for (int p = 0; p < FK / 2; ++p)
-#pragma unroll
-            for (int i = 0; i < TM; ++i)
-#pragma unroll
-                for (int j = 0; j < TN; ++j) {
-                    const uint64_t s = fadd2(pack64(a[i].v[2 * p], a[i].v[2 * p + 1]),
-                                             pack64(b[j].v[2 * p], b[j].v[2 * p + 1]));
-                    float lo, hi;
-                    unpack2(s, lo, hi);
-                    acc[i][j] = fsel3<SR>(acc[i][j], lo, hi);
-                }
+            visit_snake<TM, TN>([&](int i, int j) {
+                const uint64_t s = fadd2(pack64(a[i].v[2 * p], a[i].v[2 * p + 1]),
+                                         pack64(b[j].v[2 * p], b[j].v[2 * p + 1]));
+                float lo, hi;
+                unpack2(s, lo, hi);
+                acc[i][j] = fsel3<SR>(acc[i][j], lo, hi);
+            });
     }
 };
 
@@ -315,7 +337,7 @@ __device__ __forceinline__ void copy_tile(const GemmArgs &args, int bm, int bn, 
 // value (values are non-negative APSP distances here).  Loads of data
 // that other CTAs of the same launch may have written go through L2
 // (cp.async.cg, __ldcg), never through the non-coherent L1.
-template <class Cfg, int VAR, int SR, int NS>
+template <class Cfg, int VAR, int SR, int NS, bool MERGE = false>
 __device__ __forceinline__ bool nt_tile(const GemmArgs &args, int bm, int bn, unsigned char *smem_raw, int tid,
                                         void *Ct = nullptr, long long ldct = 0, uint32_t *Cd = nullptr,
                                         long long ldcd = 0, uint16_t *Cu = nullptr, long long ldcu = 0,
@@ -404,7 +426,7 @@ __device__ __forceinline__ bool nt_tile(const GemmArgs &args, int bm, int bn, un
                 const T v = acc[i][j];
                 if (P != nullptr && v != __ldcg(P + (long long)r * args.ldp + c)) ch = true;
                 if (SR == kMin && args.maxfin != nullptr) mx = max(mx, finite_int(v));
-                if (args.splits > 1) {
+                if (MERGE && args.splits > 1) {
                     if (v != ident) merge_atomic<SR>(C + (long long)r * args.ldc + c, v);
                 } else {
                     C[(long long)r * args.ldc + c] = v;
@@ -462,19 +484,6 @@ __global__ void __launch_bounds__(Cfg::kThreads, Cfg::MINB) tgemm_nt_kernel(cons
     const int tid = threadIdx.x;
     const int tiles_m = (args.m + Cfg::BM - 1) / Cfg::BM, tiles_n = (args.n + Cfg::BN - 1) / Cfg::BN;
     int tm, tn;
-    if (args.splits > 1) {
-        // CTA s of a tile: an equal share of the k steps
-        const int split = blockIdx.x / (tiles_m * tiles_n), steps = (args.k + Cfg::BK - 1) / Cfg::BK;
-        const int k0 = (int)((long long)steps * split / args.splits) * Cfg::BK;
-        const int k1 = min(args.k, (int)((long long)steps * (split + 1) / args.splits) * Cfg::BK);
-        raster(blockIdx.x % (tiles_m * tiles_n), tiles_m, tiles_n, args.group_m, tm, tn);
-        GemmArgs part = args;
-        part.A = static_cast<const T *>(args.A) + k0;
-        part.Bt = static_cast<const T *>(args.Bt) + k0;
-        part.k = k1 - k0;
-        nt_tile<Cfg, VAR, SR, NS>(part, tm * Cfg::BM, tn * Cfg::BN, smem_raw, tid);
-        return;
-    }
     if (args.kwave > 0) raster(blockIdx.x, tiles_n, tiles_m, args.group_m, tn, tm);
     else raster(blockIdx.x, tiles_m, tiles_n, args.group_m, tm, tn);
     const int bm = tm * Cfg::BM, bn = tn * Cfg::BN;
@@ -487,6 +496,44 @@ __global__ void __launch_bounds__(Cfg::kThreads, Cfg::MINB) tgemm_nt_kernel(cons
     const bool ch = nt_tile<Cfg, VAR, SR, NS>(args, bm, bn, smem_raw, tid, nullptr, 0, nullptr, 0, nullptr, 0, back);
     if (args.changed != nullptr) {
         if (__any_sync(0xffffffffu, ch) && (tid & 31) == 0) atomicOr(args.changed, 1);
+    }
+}
+
+// The same product with the work of a tile shared by several CTAs, whose results
+// meet in C through atomics (C holds the (+)-identity before).  splits CTAs to a
+// tile, each an equal share of the k steps; or, with stream_k, all (tile, k step)
+// units cut into gridDim.x equal shares, so that every CTA works equally long
+// whatever the number of tiles: a share is the end of one tile's k range, whole
+// tiles, and the start of another.
+template <class Cfg, int VAR, int SR, int NS>
+__global__ void __launch_bounds__(Cfg::kThreads, Cfg::MINB) tgemm_nt_merge_kernel(const GemmArgs args) {
+    using T = typename VarTypes<VAR>::T;
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    const int tiles_m = (args.m + Cfg::BM - 1) / Cfg::BM, tiles_n = (args.n + Cfg::BN - 1) / Cfg::BN;
+    const int tiles = tiles_m * tiles_n, steps = (args.k + Cfg::BK - 1) / Cfg::BK;
+    long long u0, u1;
+    if (args.stream_k > 0) {
+        const long long units = (long long)tiles * steps;
+        u0 = units * blockIdx.x / gridDim.x;
+        u1 = units * (blockIdx.x + 1) / gridDim.x;
+    } else {
+        const int split = blockIdx.x / tiles;
+        const long long first = (long long)(blockIdx.x % tiles) * steps;
+        u0 = first + (long long)steps * split / args.splits;
+        u1 = first + (long long)steps * (split + 1) / args.splits;
+    }
+    while (u0 < u1) {
+        const int s0 = (int)(u0 % steps), s1 = (int)min((long long)steps, s0 + (u1 - u0));
+        int tm, tn;
+        raster((int)(u0 / steps), tiles_m, tiles_n, args.group_m, tm, tn);
+        GemmArgs part = args;
+        part.A = static_cast<const T *>(args.A) + s0 * Cfg::BK;
+        part.Bt = static_cast<const T *>(args.Bt) + s0 * Cfg::BK;
+        part.k = min(args.k, s1 * Cfg::BK) - s0 * Cfg::BK;
+        part.splits = s1 - s0 < steps ? 2 : 1;  // a whole tile needs no atomics
+        nt_tile<Cfg, VAR, SR, NS, true>(part, tm * Cfg::BM, tn * Cfg::BN, smem_raw, threadIdx.x);
+        u0 += s1 - s0;
+        __syncthreads();  // the next part's stages take the same shared memory
     }
 }
 

@@ -31,6 +31,8 @@ struct GemmArgs {
                         // previous one left in L2 (the launcher scales it by CTAs per SM)
     int splits;         // > 1: that many CTAs per tile share its k range and merge their results
                         // into C with atomics; C must hold the (+)-identity before the launch
+    int stream_k;       // > 0: that many CTAs take equal
+                        // contiguous shares of all (tile, k step) units, merged as with splits
 };
 
 }  // namespace btas

@@ -44,6 +44,21 @@ def test_split_tiles(btas, oracle_mod, cfg, dt, sr):
 
 
 @pytest.mark.parametrize("dt", ["i32", "f32"])
+@pytest.mark.parametrize("sr", [0, 1])
+def test_equal_shares(btas, oracle_mod, dt, sr):
+    """All (tile, k step) units in equal shares for 304 CTAs: fewer units than CTAs (empty shares), parts of one tile,
+    and shares that span tiles."""
+    for m, n, k in ((100, 100, 70), (129, 257, 1000), (700, 650, 333)):
+        A, B = operands(dt, sr, m, n, k)
+        os.environ.update(BTAS_CFG="4", BTAS_SPLIT="0")
+        try:
+            C = btas.gemm(dev(A), dev(B), sr)
+        finally:
+            del os.environ["BTAS_CFG"], os.environ["BTAS_SPLIT"]
+        np.testing.assert_array_equal(bits(host(C)), bits(oracle_mod.tgemm(sr, A, B)), err_msg=f"{m}x{n}x{k}")
+
+
+@pytest.mark.parametrize("dt", ["i32", "f32"])
 @pytest.mark.parametrize("m,n,k", [(1, 1, 5000), (33, 40, 3000), (700, 20, 130), (20, 900, 64), (513, 517, 1601)])
 def test_default_choice(btas, oracle_mod, dt, m, n, k):
     """The sizes' own choice of tiles and split, with every form of call; (513, 517, 1601) also copies A, and B^T."""
