@@ -276,9 +276,9 @@ __device__ __noinline__ void relax_lists_task(const BInst &I, int t, unsigned ch
 // tiles) gives the whole solve up.
 template <int R>
 __device__ __noinline__ void relax_task(const BInst &I, int t, unsigned char *smem, int tid, int *done) {
-    constexpr int T = relax::targets<true, R>();
+    constexpr int T = relax::targets<true, R, 4>();
     const int n = I.n, j0 = T * t;
-    uint4 *Y = reinterpret_cast<uint4 *>(smem);
+    auto *Y = reinterpret_cast<relax::Vec<4> *>(smem);
     const int *W = static_cast<const int *>(I.A);
     int *D = static_cast<int *>(I.C);
     const int maxw = ld_acquire(I.rstat + kRelaxMaxW), minw = kInfI32 - ld_acquire(I.rstat + kRelaxMinW);
@@ -300,20 +300,20 @@ __device__ __noinline__ void relax_task(const BInst &I, int t, unsigned char *sm
         return true;
     };
     if (!wide) {
-        relax::load_columns<true, R>(W, I.lda, n, Y, j0);
+        relax::load_columns<true, R, 4>(W, I.lda, n, Y, j0);
         __syncthreads();
-        if (!relax::solve<true, 1, R>(W, I.lda, n, I.rl, Y, minw, give_up)) return;
-        wide = !relax::fits16<R>(Y, n, maxw);
-        if (!wide) relax::store_columns<true, R>(D, I.ldc, n, Y, j0);
+        if (!relax::solve<true, 1, R, 4>(W, I.lda, n, I.rl, Y, minw, give_up)) return;
+        wide = !relax::fits16<R, 4>(Y, n, maxw);
+        if (!wide) relax::store_columns<true, R, 4>(D, I.ldc, n, Y, j0);
         else if (tid == 0) atomicOr(I.rstat + kRelaxWide, 1);
     }
     if (wide) {
         for (int h = 0; h < T && j0 + h < n; h += T / 2) {
             __syncthreads();
-            relax::load_columns<false, R>(W, I.lda, n, Y, j0 + h);
+            relax::load_columns<false, R, 4>(W, I.lda, n, Y, j0 + h);
             __syncthreads();
-            if (!relax::solve<false, 1, R>(W, I.lda, n, I.rl, Y, minw, give_up)) return;
-            relax::store_columns<false, R>(D, I.ldc, n, Y, j0 + h);
+            if (!relax::solve<false, 1, R, 4>(W, I.lda, n, I.rl, Y, minw, give_up)) return;
+            relax::store_columns<false, R, 4>(D, I.ldc, n, Y, j0 + h);
         }
     }
 }

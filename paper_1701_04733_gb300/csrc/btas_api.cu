@@ -2,6 +2,7 @@
 // selection, stream-ordered workspace, and the APSP squaring driver.
 #include <algorithm>
 #include <atomic>
+#include <chrono>
 #include <cmath>
 #include <cstdarg>
 #include <cstdint>
@@ -917,6 +918,20 @@ static cudaError_t thread_workspace(MidThreadState &ts, size_t need, Workspace &
     return cudaSuccess;
 }
 
+// Waits until the kernel's last block has set *word, or for the stream.  The
+// blocks are through with their memory by then (each fences its writes before it
+// counts itself done), and the host sees the word some microseconds before the
+// stream reports its end; a solve longer than the watch waits for the stream.
+static cudaError_t wait_for_word(const int *word, cudaStream_t st) {
+    using clock = std::chrono::steady_clock;
+    const auto until = clock::now() + std::chrono::microseconds(200);
+    do {
+        for (int i = 0; i < 64; ++i)
+            if (__atomic_load_n(word, __ATOMIC_ACQUIRE) != 0) return cudaSuccess;
+    } while (clock::now() < until);
+    return cudaStreamSynchronize(st);
+}
+
 // Relaxation over sorted edge lists (relax.cu).  In place (D == W) it reads a
 // copy of W, left in copy_ws.  Returns a btas_status, or
 // kRelaxGaveUpFallback: D may then hold some columns already, and the caller
@@ -939,7 +954,7 @@ static int apsp_relax_solve(int64_t n, const int32_t *W, int32_t *D, Workspace &
     volatile int *out = ts.mbox;
     out[0] = 0;  // written by the last block as the solve ends
     BTAS_CUDA(launch_relax(W, n, (int)n, D, n, wsp, ts.mbox, st), "relaxation");
-    BTAS_CUDA(cudaStreamSynchronize(st), "relaxation");
+    BTAS_CUDA(wait_for_word(ts.mbox, st), "relaxation");
     const int outcome = out[0], bad = out[1], deg = out[2], wide = out[3];
     if (outcome == kRelaxBad)
         return fail(BTAS_ERR_ARG,

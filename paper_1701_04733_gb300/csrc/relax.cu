@@ -61,7 +61,7 @@ struct RelaxArgs {
     int *D;
     long long ldd;
     int *out;  // host-mapped words (see kernels.h)
-    int halves;  // 2: a second block per 8 targets takes 4 of them where 32 bits are needed from the start
+    int halves;  // 2: a second block takes half of each block's targets where 32 bits are needed from the start
 };
 
 __global__ void __launch_bounds__(kListWarps * 32) relax_lists_kernel(const RelaxArgs a) {
@@ -90,19 +90,19 @@ __global__ void __launch_bounds__(kListWarps * 32) relax_lists_kernel(const Rela
     }
 }
 
-template <int G, int MAXT>
+template <int G, int NV, int MAXT>
 __global__ void __launch_bounds__(MAXT) relax_solve_kernel(const RelaxArgs a) {
     extern __shared__ __align__(16) unsigned char smem_raw[];
-    uint4 *Y = reinterpret_cast<uint4 *>(smem_raw);
+    auto *Y = reinterpret_cast<relax::Vec<NV> *>(smem_raw);
     __shared__ int s_abort, s_wide;
     __shared__ RowStats s_st;
     const long long t0 = clock64();
     const int n = a.n, tid = threadIdx.x;
-    constexpr int R = 1, T = relax::targets<true, R>();  // targets of a block, in 16 bits
+    constexpr int R = 1, T = relax::targets<true, R, NV>();  // targets of a block, in 16 bits
     const int groups = (n + T - 1) / T, part = blockIdx.x >= groups ? 1 : 0;  // the second parts on SMs of their own
     const int j0 = (blockIdx.x - part * groups) * T;
     if (tid == 0) s_st = RowStats{0, 0, kInfI32, 0, 0, 0.0f};
-    if (part == 0) relax::load_columns<true, R>(a.W, a.ldw, n, Y, j0);  // needs no lists
+    if (part == 0) relax::load_columns<true, R, NV>(a.W, a.ldw, n, Y, j0);  // needs no lists
     asm volatile("griddepcontrol.wait;" ::: "memory");
     __syncthreads();
     const int nst = (n + kListWarps - 1) / kListWarps;
@@ -139,9 +139,9 @@ __global__ void __launch_bounds__(MAXT) relax_solve_kernel(const RelaxArgs a) {
             a.ctl[kAbort] = 1;
             return true;
         };
-        if (part == 0 && !wide && relax::solve<true, G, R>(a.W, a.ldw, n, a.lists, Y, st.minw, give_up)) {
-            wide = !relax::fits16<R>(Y, n, st.maxw);
-            if (!wide) relax::store_columns<true, R>(a.D, a.ldd, n, Y, j0);
+        if (part == 0 && !wide && relax::solve<true, G, R, NV>(a.W, a.ldw, n, a.lists, Y, st.minw, give_up)) {
+            wide = !relax::fits16<R, NV>(Y, n, st.maxw);
+            if (!wide) relax::store_columns<true, R, NV>(a.D, a.ldd, n, Y, j0);
             else if (tid == 0) a.ctl[kWide] = 1;
         }
         // in 32 bits, half of the targets at a time
@@ -149,10 +149,10 @@ __global__ void __launch_bounds__(MAXT) relax_solve_kernel(const RelaxArgs a) {
         if (wide && (part == 0 || split)) {
             for (int h = part * T / 2; h < (split ? (part + 1) * T / 2 : T) && j0 + h < n; h += T / 2) {
                 __syncthreads();
-                relax::load_columns<false, R>(a.W, a.ldw, n, Y, j0 + h);
+                relax::load_columns<false, R, NV>(a.W, a.ldw, n, Y, j0 + h);
                 __syncthreads();
-                if (!relax::solve<false, G, R>(a.W, a.ldw, n, a.lists, Y, st.minw, give_up)) break;
-                relax::store_columns<false, R>(a.D, a.ldd, n, Y, j0 + h);
+                if (!relax::solve<false, G, R, NV>(a.W, a.ldw, n, a.lists, Y, st.minw, give_up)) break;
+                relax::store_columns<false, R, NV>(a.D, a.ldd, n, Y, j0 + h);
             }
         }
     }
@@ -164,6 +164,7 @@ __global__ void __launch_bounds__(MAXT) relax_solve_kernel(const RelaxArgs a) {
             a.out[1] = st.bad;
             a.out[2] = st.deg;
             a.out[3] = *(volatile int *)(a.ctl + kWide) | st.far;
+            __threadfence_system();  // the host may watch out[0]
             a.out[0] = st.bad ? kRelaxBad : *(volatile int *)(a.ctl + kAbort) ? kRelaxGaveUp : kRelaxDone;
             __threadfence_system();
         }
@@ -212,27 +213,31 @@ cudaError_t launch_relax(const int *W, long long ldw, int n, int *D, long long l
     a.lists.edges = reinterpret_cast<uint4 *>(p += align256(rows * 4));
     a.lists.wide = reinterpret_cast<int4 *>(p + relax::list_words(n) * 4);
     a.lists.chunks = relax::list_chunks(n);
-    // Two blocks share 8 targets in 32 bits while one wave holds them all (n =
+    // Two blocks share a block's targets in 32 bits while one wave holds them all (n =
     // 1024, w <= 10^6, p = 0.5: 283 -> 158 us per call).
     a.halves = n <= 1216 ? 2 : 1;
     relax_lists_kernel<<<blocks, kListWarps * 32, 0, st>>>(a);
     note_launch();
-    // Two lanes per vertex where one would leave warps idle (n <= 256).  1024
-    // threads where one block per SM holds all targets (n = 1024, p = 0.1: 93 us
-    // per call, 112 with 512 threads) or fills shared memory (n = 8192: 3662 us
-    // against 3779), 512 and two blocks per SM between (n = 4096, p = 0.01: 1060
-    // us against 1118).  Rows of 16 or 32 targets, which pay in the batched
-    // launch, lose more to their fewer blocks than they gain (n = 2048: 265 and
-    // 377 us against 249).
-    const int G = n <= 256 ? 2 : 1, maxt = (n > 608 && n <= 1216) || n > 7000 ? 1024 : 512;
-    void (*kern)(const RelaxArgs) = G == 2 ? relax_solve_kernel<2, 512>
-                                    : maxt == 512 ? relax_solve_kernel<1, 512> : relax_solve_kernel<1, 1024>;
+    // Small graphs take fewer targets per block, so that more SMs share the
+    // sweeps' shared-memory loads: 2 up to n = 304 (46 -> 41 us per call at n = 256,
+    // p = 0.1) and 4 up to 608 (60 -> 55 us at n = 512); two lanes per vertex while
+    // one would leave warps idle.  From there on 8 targets, with 1024 threads where
+    // one block per SM holds all targets (n = 1024, p = 0.1: 93 us, 112 with 512
+    // threads) or fills shared memory (n = 8192: 3662 us against 3779), 512 and two
+    // blocks per SM between (n = 4096, p = 0.01: 1060 us against 1118).  Rows of 16 or
+    // 32 targets, which pay in the batched launch, lose more to their fewer blocks
+    // than they gain (n = 2048: 265 and 377 us against 249).
+    const int words = n <= 304 ? 1 : n <= 608 ? 2 : 4, lanes = n <= 304 ? 2 : 1;
+    const int maxt = (n > 608 && n <= 1216) || n > 7000 ? 1024 : 512;
+    void (*kern)(const RelaxArgs) = words == 1 ? relax_solve_kernel<2, 1, 512>
+                                    : words == 2 ? relax_solve_kernel<1, 2, 512>
+                                    : maxt == 512 ? relax_solve_kernel<1, 4, 512> : relax_solve_kernel<1, 4, 1024>;
     cudaError_t e = set_smem_once(reinterpret_cast<const void *>(kern), kSolveSmem);
     if (e != cudaSuccess) return e;
     cudaLaunchConfig_t cfg{};
-    cfg.gridDim = dim3((n + 7) / 8 * a.halves);
-    cfg.blockDim = dim3(std::min(maxt, (n * G + 31) / 32 * 32));
-    cfg.dynamicSmemBytes = (size_t)n * 16;
+    cfg.gridDim = dim3((n + 2 * words - 1) / (2 * words) * a.halves);
+    cfg.blockDim = dim3(std::min(maxt, (n * lanes + 31) / 32 * 32));
+    cfg.dynamicSmemBytes = (size_t)n * 4 * words;
     cfg.stream = st;
     cudaLaunchAttribute at{};
     at.id = cudaLaunchAttributeProgrammaticStreamSerialization;

@@ -313,81 +313,101 @@ __device__ __forceinline__ RowStats build_row(const int *W, long long ldw, int n
 }
 
 // -------------------------------------------------------------- relaxing
-// Y in shared memory: a row of 16 R bytes per vertex v, the distances from v to
-// 8 R targets in 16 bits (0x7FFF: none known) or to 4 R in 32.  Only v's own
-// lanes write its row, and a stale read costs a further sweep and no more, so the
-// accesses of a sweep are relaxed ones.
-__device__ __forceinline__ uint4 lds_relaxed(const uint4 *p) {
-    uint4 v;
-    asm volatile("ld.relaxed.cta.shared.v4.b32 {%0, %1, %2, %3}, [%4];"
-                 : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w)
-                 : "r"(smem_u32(p))
-                 : "memory");
+// Y in shared memory: a row of R vectors of NV words per vertex v, the distances
+// from v to 2 NV R targets in 16 bits (0x7FFF: none known) or to NV R in 32.  Each
+// vector has its own lane.  Only v's own lanes write its row, and a stale read
+// costs a further sweep and no more, so the accesses of a sweep are relaxed ones.
+template <int NV>
+struct __align__(4 * NV) Vec {
+    unsigned w[NV];
+};
+
+template <int NV>
+__device__ __forceinline__ Vec<NV> lds_relaxed(const Vec<NV> *p) {
+    Vec<NV> v;
+    if constexpr (NV == 4)
+        asm volatile("ld.relaxed.cta.shared.v4.b32 {%0, %1, %2, %3}, [%4];"
+                     : "=r"(v.w[0]), "=r"(v.w[1]), "=r"(v.w[2]), "=r"(v.w[3])
+                     : "r"(smem_u32(p))
+                     : "memory");
+    else if constexpr (NV == 2)
+        asm volatile("ld.relaxed.cta.shared.v2.b32 {%0, %1}, [%2];"
+                     : "=r"(v.w[0]), "=r"(v.w[1])
+                     : "r"(smem_u32(p))
+                     : "memory");
+    else
+        asm volatile("ld.relaxed.cta.shared.b32 %0, [%1];" : "=r"(v.w[0]) : "r"(smem_u32(p)) : "memory");
     return v;
 }
-__device__ __forceinline__ void sts_relaxed(uint4 *p, uint4 v) {
-    asm volatile("st.relaxed.cta.shared.v4.b32 [%0], {%1, %2, %3, %4};" ::"r"(smem_u32(p)), "r"(v.x), "r"(v.y),
-                 "r"(v.z), "r"(v.w)
-                 : "memory");
+template <int NV>
+__device__ __forceinline__ void sts_relaxed(Vec<NV> *p, const Vec<NV> &v) {
+    if constexpr (NV == 4)
+        asm volatile("st.relaxed.cta.shared.v4.b32 [%0], {%1, %2, %3, %4};" ::"r"(smem_u32(p)), "r"(v.w[0]),
+                     "r"(v.w[1]), "r"(v.w[2]), "r"(v.w[3])
+                     : "memory");
+    else if constexpr (NV == 2)
+        asm volatile("st.relaxed.cta.shared.v2.b32 [%0], {%1, %2};" ::"r"(smem_u32(p)), "r"(v.w[0]), "r"(v.w[1])
+                     : "memory");
+    else
+        asm volatile("st.relaxed.cta.shared.b32 [%0], %1;" ::"r"(smem_u32(p)), "r"(v.w[0]) : "memory");
 }
-template <bool U16>
-__device__ __forceinline__ int top(const uint4 &y) {
+template <bool U16, int NV>
+__device__ __forceinline__ int top(const Vec<NV> &y) {
+    unsigned m = y.w[0];
     if (U16) {
-        const unsigned m = __vmaxu2(__vmaxu2(y.x, y.y), __vmaxu2(y.z, y.w));
+#pragma unroll
+        for (int q = 1; q < NV; ++q) m = __vmaxu2(m, y.w[q]);
         return (int)max(m >> 16, m & 0xFFFFu);
     }
-    return max(max((int)y.x, (int)y.y), max((int)y.z, (int)y.w));
+#pragma unroll
+    for (int q = 1; q < NV; ++q) m = (unsigned)max((int)m, (int)y.w[q]);
+    return (int)m;
 }
 // acc = min(acc, y + w); w: the weight in both halves with U16
-template <bool U16>
-__device__ __forceinline__ void relax4(uint4 &acc, const uint4 &y, unsigned w) {
-    if (U16) {
-        acc.x = u16x2_addmin(y.x, w, acc.x);
-        acc.y = u16x2_addmin(y.y, w, acc.y);
-        acc.z = u16x2_addmin(y.z, w, acc.z);
-        acc.w = u16x2_addmin(y.w, w, acc.w);
-    } else {
-        acc.x = (unsigned)__viaddmin_s32((int)y.x, (int)w, (int)acc.x);
-        acc.y = (unsigned)__viaddmin_s32((int)y.y, (int)w, (int)acc.y);
-        acc.z = (unsigned)__viaddmin_s32((int)y.z, (int)w, (int)acc.z);
-        acc.w = (unsigned)__viaddmin_s32((int)y.w, (int)w, (int)acc.w);
+template <bool U16, int NV>
+__device__ __forceinline__ void relax_edge(Vec<NV> &acc, const Vec<NV> &y, unsigned w) {
+#pragma unroll
+    for (int q = 0; q < NV; ++q)
+        acc.w[q] = U16 ? u16x2_addmin(y.w[q], w, acc.w[q])
+                       : (unsigned)__viaddmin_s32((int)y.w[q], (int)w, (int)acc.w[q]);
+}
+// acc = min(acc, the same vector of lane ^ o)
+template <bool U16, int NV>
+__device__ __forceinline__ void min_with_lane(Vec<NV> &acc, int o) {
+#pragma unroll
+    for (int q = 0; q < NV; ++q) {
+        const unsigned b = __shfl_xor_sync(0xffffffffu, acc.w[q], o);
+        acc.w[q] = U16 ? __vminu2(acc.w[q], b) : (unsigned)min((int)acc.w[q], (int)b);
     }
 }
-template <bool U16>
-__device__ __forceinline__ uint4 min4(const uint4 &a, const uint4 &b) {
-    if (U16) return make_uint4(__vminu2(a.x, b.x), __vminu2(a.y, b.y), __vminu2(a.z, b.z), __vminu2(a.w, b.w));
-    return make_uint4((unsigned)min((int)a.x, (int)b.x), (unsigned)min((int)a.y, (int)b.y),
-                      (unsigned)min((int)a.z, (int)b.z), (unsigned)min((int)a.w, (int)b.w));
+template <int NV>
+__device__ __forceinline__ void clamp(Vec<NV> &v) {
+#pragma unroll
+    for (int q = 0; q < NV; ++q) v.w[q] = (unsigned)clamp_i32<kMin>((int)v.w[q]);
 }
-__device__ __forceinline__ uint4 shfl_xor4(const uint4 &a, int o) {
-    return make_uint4(__shfl_xor_sync(0xffffffffu, a.x, o), __shfl_xor_sync(0xffffffffu, a.y, o),
-                      __shfl_xor_sync(0xffffffffu, a.z, o), __shfl_xor_sync(0xffffffffu, a.w, o));
-}
-__device__ __forceinline__ uint4 clamp4(const uint4 &v) {
-    return make_uint4((unsigned)clamp_i32<kMin>((int)v.x), (unsigned)clamp_i32<kMin>((int)v.y),
-                      (unsigned)clamp_i32<kMin>((int)v.z), (unsigned)clamp_i32<kMin>((int)v.w));
-}
-__device__ __forceinline__ bool differ(const uint4 &a, const uint4 &b) {
-    return ((a.x ^ b.x) | (a.y ^ b.y) | (a.z ^ b.z) | (a.w ^ b.w)) != 0;
+template <int NV>
+__device__ __forceinline__ bool differ(const Vec<NV> &a, const Vec<NV> &b) {
+    unsigned d = 0;
+#pragma unroll
+    for (int q = 0; q < NV; ++q) d |= a.w[q] ^ b.w[q];
+    return d != 0;
 }
 
-// A vertex's row is R vectors of 16 bytes, each with its own lane: 8 R targets
-// in 16 bits, 4 R in 32.
-template <bool U16, int R>
-constexpr int targets() { return (U16 ? 8 : 4) * R; }
+template <bool U16, int R, int NV>
+constexpr int targets() { return (U16 ? 2 : 1) * NV * R; }
 
 // Columns [j0, j0 + targets) of W -> Y: the paths of one edge.
-template <bool U16, int R>
-__device__ __forceinline__ void load_columns(const int *W, long long ldw, int n, uint4 *Y, int j0) {
-    constexpr int S = targets<U16, 1>();
-    const bool vec = (ldw & 3) == 0 && (reinterpret_cast<uintptr_t>(W) & 15) == 0;
+template <bool U16, int R, int NV>
+__device__ __forceinline__ void load_columns(const int *W, long long ldw, int n, Vec<NV> *Y, int j0) {
+    constexpr int S = targets<U16, 1, NV>();
+    const bool vec = S % 4 == 0 && (ldw & 3) == 0 && (reinterpret_cast<uintptr_t>(W) & 15) == 0;
     for (int i = threadIdx.x; i < n * R; i += blockDim.x) {
         const int j = j0 + (i % R) * S;
         int x[S];
         const int *p = W + (long long)(i / R) * ldw + j;
         if (vec && j + S <= n) {
 #pragma unroll
-            for (int s = 0; s < S; s += 4) {
+            for (int s = 0; s + 4 <= S; s += 4) {
                 const int4 q = __ldg(reinterpret_cast<const int4 *>(p + s));
                 x[s] = q.x, x[s + 1] = q.y, x[s + 2] = q.z, x[s + 3] = q.w;
             }
@@ -395,39 +415,40 @@ __device__ __forceinline__ void load_columns(const int *W, long long ldw, int n,
 #pragma unroll
             for (int s = 0; s < S; ++s) x[s] = j + s < n ? __ldg(p + s) : 0;  // an absent target: nothing to lower
         }
-        if constexpr (U16) {
+        Vec<NV> y;
 #pragma unroll
-            for (int s = 0; s < S; ++s) x[s] = min(x[s], BTAS_INF_U16);
-            Y[i] = make_uint4(x[0] | x[1] << 16, x[2] | x[3] << 16, x[4] | x[5] << 16, x[6] | x[7] << 16);
-        } else {
-            Y[i] = make_uint4(x[0], x[1], x[2], x[3]);
+        for (int q = 0; q < NV; ++q) {
+            if constexpr (U16) y.w[q] = min(x[2 * q], BTAS_INF_U16) | min(x[2 * q + 1], BTAS_INF_U16) << 16;
+            else y.w[q] = (unsigned)x[q];
         }
+        Y[i] = y;
     }
 }
 
 // Y -> columns [j0, j0 + targets) of D.
-template <bool U16, int R>
-__device__ __forceinline__ void store_columns(int *D, long long ldd, int n, const uint4 *Y, int j0) {
-    constexpr int S = targets<U16, 1>();
-    const bool vec = (ldd & 3) == 0 && (reinterpret_cast<uintptr_t>(D) & 15) == 0;
+template <bool U16, int R, int NV>
+__device__ __forceinline__ void store_columns(int *D, long long ldd, int n, const Vec<NV> *Y, int j0) {
+    constexpr int S = targets<U16, 1, NV>();
+    const bool vec = S % 4 == 0 && (ldd & 3) == 0 && (reinterpret_cast<uintptr_t>(D) & 15) == 0;
     for (int i = threadIdx.x; i < n * R; i += blockDim.x) {
         const int j = j0 + (i % R) * S;
-        const uint4 y = Y[i];
-        const unsigned ws[4] = {y.x, y.y, y.z, y.w};
+        const Vec<NV> y = Y[i];
         int x[S];
 #pragma unroll
-        for (int s = 0; s < S; ++s) {
-            if (U16) {
-                x[s] = (int)((ws[(s >> 1) & 3] >> (16 * (s & 1))) & 0xFFFFu);
-                if (x[s] == BTAS_INF_U16) x[s] = kInfI32;
+        for (int q = 0; q < NV; ++q) {
+            if constexpr (U16) {
+                x[2 * q] = (int)(y.w[q] & 0xFFFFu);
+                x[2 * q + 1] = (int)(y.w[q] >> 16);
+                if (x[2 * q] == BTAS_INF_U16) x[2 * q] = kInfI32;
+                if (x[2 * q + 1] == BTAS_INF_U16) x[2 * q + 1] = kInfI32;
             } else {
-                x[s] = (int)ws[s & 3];
+                x[q] = (int)y.w[q];
             }
         }
         int *p = D + (long long)(i / R) * ldd + j;
         if (vec && j + S <= n) {
 #pragma unroll
-            for (int s = 0; s < S; s += 4)
+            for (int s = 0; s + 4 <= S; s += 4)
                 *reinterpret_cast<int4 *>(p + s) = make_int4(x[s], x[s + 1], x[s + 2], x[s + 3]);
         } else {
 #pragma unroll
@@ -449,13 +470,14 @@ __device__ __forceinline__ void store_columns(int *D, long long ldd, int n, cons
 //
 // One thread asks give_up() from time to time; returns false if it said so.
 // Called by the whole block.
-template <bool U16, int G, int R, class GiveUp>
-__device__ __forceinline__ bool solve(const int *W, long long ldw, int n, const Lists &l, uint4 *Y, int minw,
+template <bool U16, int G, int R, int NV, class GiveUp>
+__device__ __forceinline__ bool solve(const int *W, long long ldw, int n, const Lists &l, Vec<NV> *Y, int minw,
                                       GiveUp give_up) {
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, nwarps = blockDim.x >> 5;
     constexpr int VW = 32 / (G * R);  // vertices of a warp
+    static_assert(G <= kPadChunks, "every lane's share of a list ends with a pad chunk");
     const int sub = lane % R, g = (lane / R) % G;
-    const uint4 *Ys = Y + sub;  // Ys[v * R]: this lane's part of v's row
+    const Vec<NV> *Ys = Y + sub;  // Ys[v * R]: this lane's part of v's row
     int sweeps = 0;
     for (;;) {
         for (;;) {
@@ -466,9 +488,9 @@ __device__ __forceinline__ bool solve(const int *W, long long ldw, int n, const 
                 const int v = v0 + lane / (G * R);
                 if (G == 1 && v >= n) break;
                 const int vc = G == 1 ? v : min(v, n - 1);
-                const uint4 old = lds_relaxed(Ys + vc * R);
-                uint4 acc = old;
-                int lim = top<U16>(acc) - minw;
+                const Vec<NV> old = lds_relaxed(Ys + vc * R);
+                Vec<NV> acc = old;
+                int lim = top<U16, NV>(acc) - minw;
                 const uint4 *pe = l.edges + chunk_at(l, vc, g);
                 const int4 *pw = l.wide + chunk_at(l, vc, g);
                 uint4 e = *pe;
@@ -477,8 +499,8 @@ __device__ __forceinline__ bool solve(const int *W, long long ldw, int n, const 
                 const int heavy = 4 * (U16 ? (int)(e.x >> 16) : w.x);
                 for (int c = g;;) {
                     if ((U16 ? (int)(e.x >> 16) : w.x) >= lim) break;
-                    const uint4 y0 = lds_relaxed(Ys + (e.x & 0xFFFFu) * R), y1 = lds_relaxed(Ys + (e.y & 0xFFFFu) * R);
-                    const uint4 y2 = lds_relaxed(Ys + (e.z & 0xFFFFu) * R), y3 = lds_relaxed(Ys + (e.w & 0xFFFFu) * R);
+                    const Vec<NV> y0 = lds_relaxed(Ys + (e.x & 0xFFFFu) * R), y1 = lds_relaxed(Ys + (e.y & 0xFFFFu) * R);
+                    const Vec<NV> y2 = lds_relaxed(Ys + (e.z & 0xFFFFu) * R), y3 = lds_relaxed(Ys + (e.w & 0xFFFFu) * R);
                     const unsigned w0 = U16 ? __byte_perm(e.x, 0, 0x3232) : (unsigned)w.x;
                     const unsigned w1 = U16 ? __byte_perm(e.y, 0, 0x3232) : (unsigned)w.y;
                     const unsigned w2 = U16 ? __byte_perm(e.z, 0, 0x3232) : (unsigned)w.z;
@@ -493,12 +515,12 @@ __device__ __forceinline__ bool solve(const int *W, long long ldw, int n, const 
                             w = *pw;
                         }
                     }
-                    relax4<U16>(acc, y0, w0);
-                    relax4<U16>(acc, y1, w1);
-                    relax4<U16>(acc, y2, w2);
-                    relax4<U16>(acc, y3, w3);
+                    relax_edge<U16, NV>(acc, y0, w0);
+                    relax_edge<U16, NV>(acc, y1, w1);
+                    relax_edge<U16, NV>(acc, y2, w2);
+                    relax_edge<U16, NV>(acc, y3, w3);
                     if (!more) break;
-                    lim = top<U16>(acc) - minw;
+                    lim = top<U16, NV>(acc) - minw;
                     // an early sweep leaves the heavier edges for later
                     if (c >= early_c && (U16 ? (int)(e.x >> 16) : w.x) >= heavy) {
                         cut = true;
@@ -508,9 +530,9 @@ __device__ __forceinline__ bool solve(const int *W, long long ldw, int n, const 
                 if (G > 1) {
                     __syncwarp();
 #pragma unroll
-                    for (int o = G * R / 2; o >= R; o >>= 1) acc = min4<U16>(acc, shfl_xor4(acc, o));
+                    for (int o = G * R / 2; o >= R; o >>= 1) min_with_lane<U16, NV>(acc, o);
                 }
-                if (!U16) acc = clamp4(acc);
+                if (!U16) clamp(acc);
                 if (differ(acc, old) && (G == 1 || (g == 0 && v < n))) {
                     sts_relaxed(Y + v * R + sub, acc);
                     ch = true;
@@ -522,23 +544,24 @@ __device__ __forceinline__ bool solve(const int *W, long long ldw, int n, const 
         bool ch = false;
         for (int v0 = warp * VW; v0 < n; v0 += nwarps * VW) {
             const int vv = min(v0 + lane / (G * R), n - 1);
-            const bool need = l.next[vv] < top<U16>(lds_relaxed(Ys + vv * R)) - minw;
+            const bool need = l.next[vv] < top<U16, NV>(lds_relaxed(Ys + vv * R)) - minw;
             for (unsigned m = __ballot_sync(0xffffffffu, need); m;) {
                 const int first = (__ffs(m) - 1) / (G * R);  // the row's number in the warp
                 m &= ~(((1u << (G * R)) - 1u) << (first * G * R));
                 const int v = min(v0 + first, n - 1);
-                const uint4 old = lds_relaxed(Ys + v * R);
-                uint4 acc = old;
+                const Vec<NV> old = lds_relaxed(Ys + v * R);
+                Vec<NV> acc = old;
                 const int *wr = W + (long long)v * ldw;
                 for (int k = lane / R; k < n; k += 32 / R) {
                     const int w = __ldg(wr + k);
                     if (w < (U16 ? BTAS_INF_U16 : kInfI32))
-                        relax4<U16>(acc, lds_relaxed(Ys + k * R), U16 ? (unsigned)w * 0x10001u : (unsigned)w);
+                        relax_edge<U16, NV>(acc, lds_relaxed(Ys + k * R),
+                                            U16 ? (unsigned)w * 0x10001u : (unsigned)w);
                 }
                 __syncwarp();
 #pragma unroll
-                for (int o = 16; o >= R; o >>= 1) acc = min4<U16>(acc, shfl_xor4(acc, o));
-                if (!U16) acc = clamp4(acc);
+                for (int o = 16; o >= R; o >>= 1) min_with_lane<U16, NV>(acc, o);
+                if (!U16) clamp(acc);
                 if (differ(acc, old)) {
                     if (lane < R) sts_relaxed(Y + v * R + sub, acc);
                     ch = true;
@@ -553,15 +576,14 @@ __device__ __forceinline__ bool solve(const int *W, long long ldw, int n, const 
 // Whether 16 bits were enough.  Saturating sums commute with the minimum, so
 // Y = min(distance, 0x7FFF); an entry at 0x7FFF is a missing path when no
 // finite distance plus one edge, and no path of n - 1 edges, reaches 0x7FFF.
-template <int R>
-__device__ __forceinline__ bool fits16(const uint4 *Y, int n, int maxw) {
+template <int R, int NV>
+__device__ __forceinline__ bool fits16(const Vec<NV> *Y, int n, int maxw) {
     int inf = 0, fin = 0;
     for (int i = threadIdx.x; i < n * R; i += blockDim.x) {
-        const uint4 y = Y[i];
-        const unsigned ws[4] = {y.x, y.y, y.z, y.w};
+        const Vec<NV> y = Y[i];
 #pragma unroll
-        for (int s = 0; s < 8; ++s) {
-            const int x = (int)((ws[s >> 1] >> (16 * (s & 1))) & 0xFFFFu);
+        for (int s = 0; s < 2 * NV; ++s) {
+            const int x = (int)((y.w[s >> 1] >> (16 * (s & 1))) & 0xFFFFu);
             if (x == BTAS_INF_U16) inf = 1;
             else fin = max(fin, x);
         }
