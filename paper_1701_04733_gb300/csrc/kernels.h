@@ -96,10 +96,11 @@ cudaError_t launch_apsp_scan(const int *W, long long n, int *out, cudaStream_t s
 // Keyed path squaring (paths.cu): while every finite entry of D is <=
 // paths_key_max() and n <= paths_key_max_n(), one int32 min-plus product of
 // A' = D << 13 and B' = (D << 13) | k gives distances and smallest
-// minimising k together.  encode: A' (pitch n) and B'^T (pitch ldt);
+// minimising k together.  encode: A' and B'^T (both pitch ldt);
 // decode: keys -> D', N' (K may be Dn), change flag, largest finite entry.
 int paths_key_max();
 int paths_key_max_n();
+int paths_key_shift();
 cudaError_t launch_paths_encode(const int *D, int n, int *Ak, int *BkT, long long ldt, cudaStream_t st);
 cudaError_t launch_paths_decode(const int *K, const int *D, const int *N, long long n, int *Dn, int *Nn, int *changed,
                                 int *maxfin, cudaStream_t st);
@@ -193,6 +194,15 @@ size_t relax_workspace(long long n);
 int relax_max_n();
 cudaError_t launch_relax(const int *W, long long ldw, int n, int *D, long long ldd, void *ws, int *out,
                          cudaStream_t st);
+// The edge lists alone (ws: edge_lists_workspace(n) bytes), and in out (device, 3
+// ints): entries of W outside the domain, the largest weight, the most edges of a
+// row (INT_MAX if some list holds less than its row).  launch_sparse_keys then writes the first squaring's keys (value << shift)
+// | smallest minimising k, or INF, to K (n x n, n <= 8192) from them; it needs
+// every edge in the lists, and pays from sparse_keys_pay on.
+size_t edge_lists_workspace(long long n);
+cudaError_t launch_edge_lists(const int *W, int n, void *ws, int *out, cudaStream_t st);
+bool sparse_keys_pay(long long n, int most_edges);
+cudaError_t launch_sparse_keys(const int *W, int n, void *ws, int shift, int *K, cudaStream_t st);
 // Entries from INF - 2^28 on become INF, as the squarings leave them.
 cudaError_t launch_clamp(int *D, size_t count, cudaStream_t st);
 

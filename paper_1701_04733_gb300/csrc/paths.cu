@@ -269,7 +269,7 @@ __global__ void paths_encode_kernel(const int *__restrict__ D, int n, int *__res
         const int k = k0 + r, j = j0 + threadIdx.x;
         if (k < n && j < n) {
             const int v = D[(long long)k * n + j];
-            Ak[(long long)k * n + j] = key_a(v);
+            Ak[(long long)k * ldt + j] = key_a(v);
             tile[r][threadIdx.x] = v;
         }
     }
@@ -375,6 +375,7 @@ cudaError_t launch_paths_scan_f32(const float *W, long long n, int *bad, cudaStr
 
 int paths_key_max() { return 49151; }
 int paths_key_max_n() { return kKeyMaxN; }
+int paths_key_shift() { return kKeyShift; }
 
 cudaError_t launch_paths_encode(const int *D, int n, int *Ak, int *BkT, long long ldt, cudaStream_t st) {
     if (n <= 0) return cudaSuccess;

@@ -85,6 +85,7 @@ __global__ void __launch_bounds__(kListWarps * 32) relax_lists_kernel(const Rela
             st.deg = max(st.deg, o.deg);
             st.far |= o.far;
             st.light += o.light;
+            st.cut |= o.cut;
         }
         a.stats[blockIdx.x] = st;
     }
@@ -171,6 +172,54 @@ __global__ void __launch_bounds__(MAXT) relax_solve_kernel(const RelaxArgs a) {
     }
 }
 
+// out[0] = entries outside the domain, out[1] = largest weight, out[2] = most
+// edges of a row, or INT_MAX if some list holds less than its row.  One block.
+__global__ void __launch_bounds__(256) relax_stats_kernel(const RowStats *stats, int blocks, int *out) {
+    __shared__ int s[3];
+    if (threadIdx.x < 3) s[threadIdx.x] = 0;
+    __syncthreads();
+    for (int i = threadIdx.x; i < blocks; i += blockDim.x) {
+        if (stats[i].bad) atomicAdd(s, stats[i].bad);
+        atomicMax(s + 1, stats[i].maxw);
+        atomicMax(s + 2, stats[i].cut ? 0x7FFFFFFF : stats[i].deg);
+    }
+    __syncthreads();
+    if (threadIdx.x < 3) out[threadIdx.x] = s[threadIdx.x];
+}
+
+// The first squaring of W with smallest minimising k, as keys (value << shift) |
+// k, from the lists: row i of K in shared memory starts with the terms k = i and k
+// = j, both W[i][j], and takes the terms of every pair of edges (i, k), (k, j).
+// One block per row; its warps take row i's edges in turn and read row k's list
+// along their lanes.
+__global__ void __launch_bounds__(256) sparse_key_kernel(const int *W, int n, Lists l, int shift, int *K) {
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    int *key = reinterpret_cast<int *>(smem_raw);
+    const int i = blockIdx.x, lane = threadIdx.x & 31, warp = threadIdx.x >> 5, warps = blockDim.x >> 5;
+    for (int j = threadIdx.x; j < n; j += blockDim.x) {
+        const int w = W[(long long)i * n + j];
+        key[j] = w < kInfI32 ? (w << shift) | min(i, j) : kInfI32;
+    }
+    __syncthreads();
+    const int own = l.len[i];
+    for (int e = warp; e < own; e += warps) {
+        const size_t at = relax::chunk_at(l, i, e >> 2) * 4 + (e & 3);
+        const int k = (int)(reinterpret_cast<const unsigned *>(l.edges)[at] & 0xFFFFu);
+        const int w1 = reinterpret_cast<const int *>(l.wide)[at], len = l.len[k];
+        for (int c = lane; 4 * c < len; c += 32) {
+            const uint4 to = l.edges[relax::chunk_at(l, k, c)];
+            const int4 w2 = l.wide[relax::chunk_at(l, k, c)];
+            const unsigned j[4] = {to.x & 0xFFFFu, to.y & 0xFFFFu, to.z & 0xFFFFu, to.w & 0xFFFFu};
+            const int w[4] = {w2.x, w2.y, w2.z, w2.w};
+#pragma unroll
+            for (int q = 0; q < 4; ++q)
+                if (4 * c + q < len) atomicMin(key + j[q], ((w1 + w[q]) << shift) | k);
+        }
+    }
+    __syncthreads();
+    for (int j = threadIdx.x; j < n; j += blockDim.x) K[(long long)i * n + j] = key[j];
+}
+
 __global__ void clamp_kernel(int *D, size_t count) {
     for (size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x; i < count; i += (size_t)gridDim.x * blockDim.x)
         if (D[i] >= kClampI32) D[i] = kInfI32;
@@ -193,11 +242,52 @@ size_t relax_workspace(long long n) {
            relax::list_words(n) * 8;
 }
 
+namespace {
+// Places in a workspace of relax_workspace(n) bytes.
+void place(void *ws, int n, int **ctl, RowStats **stats, Lists *lists) {
+    const size_t rows = (size_t)((n + 31) & ~31);
+    char *p = static_cast<char *>(ws);
+    *ctl = reinterpret_cast<int *>(p);
+    *stats = reinterpret_cast<RowStats *>(p += 256);
+    lists->next = reinterpret_cast<int *>(p += align256((n + kListWarps - 1) / kListWarps * sizeof(RowStats)));
+    lists->edges = reinterpret_cast<uint4 *>(p += align256(rows * 4));
+    lists->wide = reinterpret_cast<int4 *>(p + relax::list_words(n) * 4);
+    lists->chunks = relax::list_chunks(n);
+}
+}  // namespace
+
+size_t edge_lists_workspace(long long n) { return relax_workspace(n) + align256((size_t)n * 4); }
+
+cudaError_t launch_edge_lists(const int *W, int n, void *ws, int *out, cudaStream_t st) {
+    const int blocks = (n + kListWarps - 1) / kListWarps;
+    RelaxArgs a{};
+    a.W = W;
+    a.ldw = n;
+    a.n = n;
+    place(ws, n, &a.ctl, &a.stats, &a.lists);
+    a.lists.len = reinterpret_cast<int *>(static_cast<char *>(ws) + relax_workspace(n));
+    relax_lists_kernel<<<blocks, kListWarps * 32, 0, st>>>(a);
+    relax_stats_kernel<<<1, 256, 0, st>>>(a.stats, blocks, out);
+    note_launch(2);
+    return cudaGetLastError();
+}
+
+bool sparse_keys_pay(long long n, int most_edges) { return most_edges <= relax::kCap && 6LL * most_edges <= n; }
+
+cudaError_t launch_sparse_keys(const int *W, int n, void *ws, int shift, int *K, cudaStream_t st) {
+    Lists l{};
+    int *ctl;
+    RowStats *stats;
+    place(ws, n, &ctl, &stats, &l);
+    l.len = reinterpret_cast<int *>(static_cast<char *>(ws) + relax_workspace(n));
+    sparse_key_kernel<<<n, 256, (size_t)n * 4, st>>>(W, n, l, shift, K);
+    note_launch();
+    return cudaGetLastError();
+}
+
 cudaError_t launch_relax(const int *W, long long ldw, int n, int *D, long long ldd, void *ws, int *out,
                          cudaStream_t st) {
-    const size_t rows = (size_t)((n + 31) & ~31);
     const int blocks = (n + kListWarps - 1) / kListWarps;
-    char *p = static_cast<char *>(ws);
     RelaxArgs a{};
     a.W = W;
     a.ldw = ldw;
@@ -207,12 +297,7 @@ cudaError_t launch_relax(const int *W, long long ldw, int n, int *D, long long l
     a.out = out;
     const char *bud = getenv("BTAS_RELAX_BUDGET");
     a.lists.budget = bud && *bud ? atoll(bud) : relax::budget_cycles(n);
-    a.ctl = reinterpret_cast<int *>(p);
-    a.stats = reinterpret_cast<RowStats *>(p += 256);
-    a.lists.next = reinterpret_cast<int *>(p += align256(blocks * sizeof(RowStats)));
-    a.lists.edges = reinterpret_cast<uint4 *>(p += align256(rows * 4));
-    a.lists.wide = reinterpret_cast<int4 *>(p + relax::list_words(n) * 4);
-    a.lists.chunks = relax::list_chunks(n);
+    place(ws, n, &a.ctl, &a.stats, &a.lists);
     // Two blocks share a block's targets in 32 bits while one wave holds them all (n =
     // 1024, w <= 10^6, p = 0.5: 283 -> 158 us per call).
     a.halves = n <= 1216 ? 2 : 1;

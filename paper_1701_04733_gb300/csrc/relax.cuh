@@ -32,6 +32,7 @@ struct Lists {
     uint4 *edges;  // [ceil(n / 32)][chunks][32]
     int4 *wide;    // the weights in 32 bits, same places
     int *next;     // n words
+    int *len;      // optional: edges in each list
     int chunks;    // capacity / 4
     long long budget;  // clock cycles after which a block gives up
 };
@@ -44,6 +45,7 @@ struct RowStats {
     int deg;    // most edges of a row
     int far;    // 1: some row's lightest edge does not fit 16 bits
     float light;  // sum of the rows' lightest weights
+    int cut;      // 1: some list holds less than its row
 };
 
 // Clock cycles a block of 8 targets is worth: about twice what the slowest
@@ -295,7 +297,10 @@ __device__ __forceinline__ RowStats build_row(const int *W, long long ldw, int n
         cut = select_cut(wr, row, n, kTruncTarget, mn, mx, hist, lane, ties);
         cnt = min(cap, scan_row(wr, n, row, cut, ties, buf, lane, st, mn, mx, deg));
     }
-    if (lane == 0) l.next[row] = cnt < deg ? cut : kInfI32;
+    if (lane == 0) {
+        l.next[row] = cnt < deg ? cut : kInfI32;
+        if (l.len != nullptr) l.len[row] = cnt;
+    }
     const bool k32 = (cnt < deg ? cut : mx) - mn < 0xFFFF;
     if (cnt <= 128) {
         if (k32) sort_and_store<true, 4>(buf, cnt, row, mn, l, lane);
@@ -309,6 +314,7 @@ __device__ __forceinline__ RowStats build_row(const int *W, long long ldw, int n
     st.deg = deg;
     st.far = deg > 0 && mn >= BTAS_INF_U16;
     st.light = deg > 0 ? (float)mn : 0.0f;
+    st.cut = cnt < deg;
     return st;
 }
 
