@@ -1413,7 +1413,7 @@ btas_status btas_apsp_paths(int64_t n, const int32_t *W, int32_t *D, int32_t *Ne
     bool sparse = false;
     if (lists) {
         int host[3] = {0, 0, 0};
-        BTAS_CUDA(launch_edge_lists(W, (int)n, lists, dflags + 2 * S, st), "edge lists");
+        BTAS_CUDA(launch_edge_lists(W, (int)n, paths_key_max(), lists, dflags + 2 * S, st), "edge lists");
         BTAS_CUDA(read_back(host, dflags + 2 * S, 12, st), "lists readback");
         if (host[0] != 0) return fail(BTAS_ERR_ARG, "btas_apsp_paths: %d entries outside the domain", host[0]);
         mval = host[1];

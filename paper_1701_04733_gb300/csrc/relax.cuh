@@ -35,6 +35,9 @@ struct Lists {
     int *len;      // optional: edges in each list
     int chunks;    // capacity / 4
     long long budget;  // clock cycles after which a block gives up
+    // > 0: only lists of whole rows are of use, of at most `whole` edges, none
+    // heavier than `top`; other rows are counted and no more
+    int whole, top;
 };
 
 // What building the lists of some rows finds out.
@@ -272,7 +275,7 @@ __device__ __forceinline__ RowStats build_row(const int *W, long long ldw, int n
     bool ties = false;
     // A long row is read once: its first entries say whether it will overflow
     // and, if so, about where to cut.
-    if (n >= 2 * kSample) {
+    if (n >= 2 * kSample && l.whole == 0) {
         int d = 0, mn = kInfI32, mx = 0;
 #pragma unroll 8
         for (int j = lane; j < kSample; j += 32) {
@@ -293,6 +296,13 @@ __device__ __forceinline__ RowStats build_row(const int *W, long long ldw, int n
     }
     int mn, mx, deg;
     int cnt = scan_row(wr, n, row, cut, ties, buf, lane, st, mn, mx, deg);
+    if (l.whole > 0 && (deg > l.whole || mx > l.top)) {
+        st.maxw = mx;
+        st.minw = mn;
+        st.deg = deg;
+        st.cut = 1;
+        return st;
+    }
     if (cnt > cap || (cnt < deg && cnt < 64)) {
         cut = select_cut(wr, row, n, kTruncTarget, mn, mx, hist, lane, ties);
         cnt = min(cap, scan_row(wr, n, row, cut, ties, buf, lane, st, mn, mx, deg));

@@ -25,10 +25,10 @@ def graph(n, p, lo, hi, seed):
     return np.where((W < INF) & ~np.eye(n, dtype=bool), W - 1 + lo, W).astype(np.int32)
 
 
-def hub(n):
-    """Two rows with n // 6 edges, the longest that still take the sparse squaring, and two with more."""
+def hub(n, more=0):
+    """A row with n // 6 edges, the most that still takes the sparse squaring, and one with `more` above that."""
     W = graph(n, 2.0 / n, 1, 9, 83)
-    for r, m in ((1, n // 6), (n - 2, n // 6)):
+    for r, m in ((1, n // 6), (n - 2, n // 6 + more)):
         W[r] = INF
         W[r, :m + 1] = 3 + np.arange(m + 1) % 5
         W[r, r] = 0
@@ -36,6 +36,7 @@ def hub(n):
 
 
 CASES = {"ties": lambda n: graph(n, 0.05, 1, 3, 81), "zeros": lambda n: graph(n, 0.05, 0, 2, 82), "hub": hub,
+         "one row too long": lambda n: hub(n, 1), "too heavy": lambda n: graph(n, 0.04, 49000, 49400, 88),
          "heavy": lambda n: graph(n, 0.04, 1, 49151, 84), "dense": lambda n: graph(n, 0.5, 1, 1000, 85),
          "empty": lambda n: graph(n, 0.0, 1, 1, 86)}
 
