@@ -160,12 +160,13 @@ __device__ __forceinline__ void sort_and_store(const unsigned long long *buf, in
 
 // A weight such that about `target` of the edges among the row's first m
 // entries are lighter (at most `target`; at least half of it unless weights
-// repeat too often: then ties is set and the edges at the cutoff weight
-// itself fill up the list).  Histograms of 256 equal bins of [lo, hi], refined
-// around the bin that does not fit.  `hist`: 256 words of the warp's own.
+// repeat too often: then ties is set and edges at the cutoff weight itself
+// may fill up the list).  `below`: how many are lighter.  Histograms of 256 equal
+// bins of [lo, hi], refined around the bin that does not fit.  `hist`: 256
+// words of the warp's own.
 __device__ __forceinline__ int select_cut(const int *wr, int row, int m, int target, int lo, int hi, int *hist,
-                                          int lane, bool &ties) {
-    int below = 0;  // edges lighter than lo
+                                          int lane, bool &ties, int &below) {
+    below = 0;  // edges lighter than lo
     ties = false;
     for (;;) {
         const int sh = max(0, 24 - __clz(max(hi - lo, 1)));  // (hi - lo) >> sh <= 255
@@ -222,13 +223,14 @@ __device__ __forceinline__ int select_cut(const int *wr, int row, int m, int tar
 }
 
 // One pass over row `row` of W by one warp: the domain check, the statistics,
-// and the edges lighter than `cut` (or as light, with ties) to buf, kCap of
-// them at most.  Returns how many there are; deg: all of the row's edges.
-__device__ __forceinline__ int scan_row(const int *wr, int n, int row, int cut, bool ties, unsigned long long *buf,
+// and the edges lighter than `cut`, with the first `room` of those as light as
+// it, to buf, kCap of them at most.  Returns how many there are; deg: all of
+// the row's edges.
+__device__ __forceinline__ int scan_row(const int *wr, int n, int row, int cut, int room, unsigned long long *buf,
                                         int lane, RowStats &st, int &mn, int &mx, int &deg) {
     constexpr int U = 8;
     const unsigned lt = (1u << lane) - 1u;
-    int cnt = 0;
+    int cnt = 0, tied = 0;
     deg = 0;
     mn = kInfI32;
     mx = 0;
@@ -249,7 +251,13 @@ __device__ __forceinline__ int scan_row(const int *wr, int n, int row, int cut, 
             deg += edge;
             mx = max(mx, edge ? v[u] : 0);
             mn = min(mn, edge ? v[u] : kInfI32);
-            const bool keep = edge && (v[u] < cut || (ties && v[u] == cut));
+            bool keep = edge && v[u] < cut;
+            if (room > 0) {
+                const bool tie = edge && v[u] == cut;
+                const unsigned m = __ballot_sync(0xffffffffu, tie);
+                keep = keep || (tie && tied + __popc(m & lt) < room);
+                tied += __popc(m);
+            }
             const unsigned m = __ballot_sync(0xffffffffu, keep);
             const int q = cnt + __popc(m & lt);
             if (keep && q < kCap) buf[q] = ((unsigned long long)(unsigned)v[u] << 32) | (unsigned)j;
@@ -273,6 +281,7 @@ __device__ __forceinline__ RowStats build_row(const int *W, long long ldw, int n
     RowStats st{};
     int cut = kInfI32;
     bool ties = false;
+    int below;
     // A long row is read once: its first entries say whether it will overflow
     // and, if so, about where to cut.
     if (n >= 2 * kSample && l.whole == 0) {
@@ -291,11 +300,11 @@ __device__ __forceinline__ RowStats build_row(const int *W, long long ldw, int n
         mx = __reduce_max_sync(0xffffffffu, mx);
         if ((long long)d * n > (long long)cap * kSample * 9 / 10)
             cut = select_cut(wr, row, kSample, max(4, (int)((long long)kTruncTarget * kSample / n)), mn, mx, hist,
-                             lane, ties);
-        if (ties) cut = kInfI32, ties = false;
+                             lane, ties, below);
+        if (ties) cut = kInfI32;
     }
     int mn, mx, deg;
-    int cnt = scan_row(wr, n, row, cut, ties, buf, lane, st, mn, mx, deg);
+    int cnt = scan_row(wr, n, row, cut, 0, buf, lane, st, mn, mx, deg);
     if (l.whole > 0 && (deg > l.whole || mx > l.top)) {
         st.maxw = mx;
         st.minw = mn;
@@ -304,8 +313,9 @@ __device__ __forceinline__ RowStats build_row(const int *W, long long ldw, int n
         return st;
     }
     if (cnt > cap || (cnt < deg && cnt < 64)) {
-        cut = select_cut(wr, row, n, kTruncTarget, mn, mx, hist, lane, ties);
-        cnt = min(cap, scan_row(wr, n, row, cut, ties, buf, lane, st, mn, mx, deg));
+        // every lighter edge (at most kTruncTarget) and as many at the cutoff as fit
+        cut = select_cut(wr, row, n, kTruncTarget, mn, mx, hist, lane, ties, below);
+        cnt = scan_row(wr, n, row, cut, ties ? cap - below : 0, buf, lane, st, mn, mx, deg);
     }
     if (lane == 0) {
         l.next[row] = cnt < deg ? cut : kInfI32;

@@ -59,6 +59,15 @@ def zeros(n):
     return W
 
 
+def equal_but_few(n):
+    """Rows of equal weights, longer than a list, with light edges anywhere among them: the list keeps every
+    light edge."""
+    light = gen.random_graph(gen.BASE_SEED, 47 + n, n, 0.02, 1, 20)
+    W = np.where(light < INF, light, 1000).astype(np.int32)
+    np.fill_diagonal(W, 0)
+    return W
+
+
 def clamped(n):
     """Weights up to 2^28: three of them reach the clamp, and the distance is INF."""
     W = gen.random_graph(gen.BASE_SEED, 41 + n, n, 3.0 / n, 1 << 27, 1 << 28)
@@ -72,6 +81,7 @@ def random(p, w):
 
 GRAPHS = {"empty": empty, "path": path, "two_blocks": two_blocks, "zeros": zeros, "clamped": clamped,
           "sparse": random(0.02, 100), "sparse_heavy": random(0.03, 10 ** 6), "dense_ties": random(1.0, 2),
+          "equal_but_few": equal_but_few,
           "dense_heavy": random(0.6, 10 ** 6), "border": random(0.05, 12000)}
 
 
