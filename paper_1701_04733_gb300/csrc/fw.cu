@@ -30,10 +30,16 @@ constexpr int FT = 256;  // threads: 16 x 16, each owning 8 rows x 8 columns of 
 // loads are contiguous 16-byte chunks: no bank conflicts).
 __device__ __forceinline__ int fw_col(int tx, int c) { return (c < 4 ? 0 : 64 - 4) + tx * 4 + c; }
 
+// Whether the rows of D start on 16 bytes: n a multiple of 4 and D aligned (the
+// caller's D may be a view at any element).
+__device__ __forceinline__ bool rows_aligned(const int *D, long long n) {
+    return (n & 3) == 0 && (reinterpret_cast<uintptr_t>(D) & 15) == 0;
+}
+
 // Load tile (r0, c0) of D into shared memory (INF outside the matrix), in
-// 16-byte vectors where the rows allow (n a multiple of 4).
+// 16-byte vectors where the rows allow.
 __device__ __forceinline__ void load_tile(int *sm, const int *D, long long n, int r0, int c0) {
-    const bool vec = (n & 3) == 0;
+    const bool vec = rows_aligned(D, n);
     for (int idx = threadIdx.x; idx < FB * FB / 4; idx += blockDim.x) {
         const int r = idx / (FB / 4), c = (idx % (FB / 4)) * 4;
         const long long gr = r0 + r, gc = c0 + c;
@@ -51,7 +57,7 @@ __device__ __forceinline__ void load_tile(int *sm, const int *D, long long n, in
 }
 // Store the tile; with pmax, also atomicMax the largest finite value stored.
 __device__ __forceinline__ void store_tile(const int *sm, int *D, long long n, int r0, int c0, int *pmax) {
-    const bool vec = (n & 3) == 0;
+    const bool vec = rows_aligned(D, n);
     int mx = -1;
     for (int idx = threadIdx.x; idx < FB * FB / 4; idx += blockDim.x) {
         const int r = idx / (FB / 4), c = (idx % (FB / 4)) * 4;
