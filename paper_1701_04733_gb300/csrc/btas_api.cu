@@ -1059,8 +1059,6 @@ static btas_status apsp_impl(int64_t n, const int32_t *W, int32_t *D, int flags,
         if (n >= 2048) {
             const btas_status r = btas_apsp_fw(n, W, D, st);
             if (r != BTAS_OK) return r;
-            // Floyd-Warshall clamps in its third phase only
-            BTAS_CUDA(launch_clamp(D, nn, st), "clamp");
             log_event("apsp n=%lld: tiled kernels range, blocked Floyd-Warshall", (long long)n);
             return BTAS_OK;
         }

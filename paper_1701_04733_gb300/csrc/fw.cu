@@ -55,7 +55,9 @@ __device__ __forceinline__ void load_tile(int *sm, const int *D, long long n, in
         *reinterpret_cast<int4 *>(sm + r * FB + c) = v;
     }
 }
-// Store the tile; with pmax, also atomicMax the largest finite value stored.
+// Store the tile, in the encoding (a value from INF - 2^28 on is INF, as in
+// phase 3: a path through it is as long, so clamping here or there is the
+// same); with pmax, also atomicMax the largest finite value stored.
 __device__ __forceinline__ void store_tile(const int *sm, int *D, long long n, int r0, int c0, int *pmax) {
     const bool vec = rows_aligned(D, n);
     int mx = -1;
@@ -64,9 +66,9 @@ __device__ __forceinline__ void store_tile(const int *sm, int *D, long long n, i
         const long long gr = r0 + r, gc = c0 + c;
         if (gr >= n) continue;
         const int4 v = *reinterpret_cast<const int4 *>(sm + r * FB + c);
-        const int t[4] = {v.x, v.y, v.z, v.w};
+        const int t[4] = {clamp_i32<kMin>(v.x), clamp_i32<kMin>(v.y), clamp_i32<kMin>(v.z), clamp_i32<kMin>(v.w)};
         if (vec && gc + 4 <= n) {
-            *reinterpret_cast<int4 *>(D + gr * n + gc) = v;
+            *reinterpret_cast<int4 *>(D + gr * n + gc) = make_int4(t[0], t[1], t[2], t[3]);
 #pragma unroll
             for (int e = 0; e < 4; ++e)
                 if (t[e] < kInfI32) mx = max(mx, t[e]);

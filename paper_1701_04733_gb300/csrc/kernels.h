@@ -205,8 +205,6 @@ size_t edge_lists_workspace(long long n);
 cudaError_t launch_edge_lists(const int *W, int n, int max_weight, void *ws, int *found, cudaStream_t st);
 bool sparse_keys_pay(long long n, int most_edges);
 cudaError_t launch_sparse_keys(const int *W, int n, void *ws, int shift, int *K, cudaStream_t st);
-// Entries from INF - 2^28 on become INF, as the squarings leave them.
-cudaError_t launch_clamp(int *D, size_t count, cudaStream_t st);
 
 // ---- blocked Floyd-Warshall (fw.cu): phases 1 and 2 of pivot block kb
 // pmax (optional): atomicMax of the largest finite value the phases store

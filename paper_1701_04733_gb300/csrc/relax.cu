@@ -213,19 +213,8 @@ __global__ void __launch_bounds__(256) sparse_key_kernel(const int *W, int n, Li
     for (int j = threadIdx.x; j < n; j += blockDim.x) K[(long long)i * n + j] = key[j];
 }
 
-__global__ void clamp_kernel(int *D, size_t count) {
-    for (size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x; i < count; i += (size_t)gridDim.x * blockDim.x)
-        if (D[i] >= kClampI32) D[i] = kInfI32;
-}
-
 size_t align256(size_t v) { return (v + 255) & ~size_t(255); }
 }  // namespace
-
-cudaError_t launch_clamp(int *D, size_t count, cudaStream_t st) {
-    clamp_kernel<<<(unsigned)std::min<size_t>((count + 255) / 256, 152 * 8), 256, 0, st>>>(D, count);
-    note_launch();
-    return cudaGetLastError();
-}
 
 int relax_max_n() { return kSolveSmem / 16; }
 

@@ -1,4 +1,5 @@
-"""Blocked Floyd-Warshall where its rows do not start on 16 bytes, called directly and as what btas.apsp falls back to."""
+"""Blocked Floyd-Warshall where its rows do not start on 16 bytes, called directly and
+as what btas.apsp falls back to, and its encoding of long distances."""
 import os
 
 import numpy as np
@@ -8,6 +9,8 @@ import gen
 from tests.gpu_util import dev, host
 
 pytestmark = pytest.mark.gpu
+
+INF = 0x3FFFFFFF
 
 
 @pytest.fixture(scope="module")
@@ -68,3 +71,21 @@ def test_apsp_falls_back_to_it_at_any_element(btas, in_place):
         del os.environ["BTAS_RELAX_BUDGET"]
     np.testing.assert_array_equal(host(d), ref)
     assert untouched(dbuf, 1, n)
+
+
+@pytest.mark.parametrize("ahead", ["0", "1"])
+@pytest.mark.parametrize("n", [3, 5, 128, 129, 300, 517])
+def test_long_distances_keep_the_encoding(btas, oracle_mod, n, ahead):
+    """Weights up to 2^28: three or more of them reach INF - 2^28, and the entry is INF, in every tile: the last
+    pivot block's, which no product touches afterwards, included."""
+    W = gen.random_graph(gen.BASE_SEED, 41 + n, n, min(0.5, 3.0 / n), 1 << 27, 1 << 28)
+    W[np.arange(n - 1), np.arange(1, n)] = 1 << 28
+    ref = oracle_mod.floyd_warshall(W)
+    assert n < 128 or ((ref >= INF - (1 << 28)) & (ref < INF)).any()  # some entries need it
+    ref[ref >= INF - (1 << 28)] = INF
+    os.environ["BTAS_FW_NO_LOOKAHEAD"] = "0" if ahead == "1" else "1"
+    try:
+        np.testing.assert_array_equal(host(btas.apsp_fw(dev(W))), ref)
+    finally:
+        del os.environ["BTAS_FW_NO_LOOKAHEAD"]
+    np.testing.assert_array_equal(host(btas.apsp(dev(W))), ref)
