@@ -283,11 +283,17 @@ __device__ __noinline__ void relax_task(const BInst &I, int t, unsigned char *sm
     int *D = static_cast<int *>(I.C);
     const int maxw = ld_acquire(I.rstat + kRelaxMaxW), minw = kInfI32 - ld_acquire(I.rstat + kRelaxMinW);
     const float light = __int_as_float(ld_acquire(I.rstat + kRelaxLight));
-    // the same in every thread: two words that other tasks may set meanwhile
+    // the same in every thread: two words that other tasks may set meanwhile.
+    // solve() needs W's domain: its bounds, and the pads that end a list, hold for
+    // no other values, and a lane that runs past them reads rows that are not
+    // there.  Where the domain is assumed, a W outside it is left to the
+    // squarings, which compute something for any values.
     __shared__ int s_word[2];
     if (tid == 0) {
+        const int bad = ld_acquire(I.rstat + kRelaxBadEntries);
+        if (bad != 0 && !I.checked && atomicExch(I.rstat + kRelaxGaveUpWord, 1) == 0) atomicAdd(done + 1, 1);
         s_word[0] = ld_acquire(I.rstat + kRelaxWide);
-        s_word[1] = ld_acquire(I.rstat + kRelaxGaveUpWord) | (I.checked ? ld_acquire(I.rstat + kRelaxBadEntries) : 0);
+        s_word[1] = ld_acquire(I.rstat + kRelaxGaveUpWord) | bad;
     }
     __syncthreads();
     bool wide = s_word[0] != 0 || relax::expects_wide(n, light);

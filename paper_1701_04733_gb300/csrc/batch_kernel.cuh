@@ -88,7 +88,7 @@ struct BInst {
     int2 *lists;
     int *deg;
     // relaxation: its lists, its words, and whether W's domain is checked (C
-    // is then not written where it is violated)
+    // is then not written where it is violated; else such a solve is given up)
     relax::Lists rl;
     int *rstat;
     int checked;
