@@ -62,7 +62,15 @@ static cudaError_t device_pool(cudaMemPool_t *out) {
     return cudaSuccess;
 }
 
+// Fault injection (tests only): BTAS_WS_LIMIT=bytes refuses every larger piece of
+// workspace, as a full device does.
+static bool ws_refused(size_t bytes) {
+    const char *v = getenv("BTAS_WS_LIMIT");
+    return v && *v && bytes > strtoull(v, nullptr, 10);
+}
+
 cudaError_t ws_alloc(void **p, size_t bytes, cudaStream_t st) {
+    if (ws_refused(bytes)) return cudaErrorMemoryAllocation;
     cudaMemPool_t pool = nullptr;
     cudaError_t e = device_pool(&pool);
     if (e != cudaSuccess) return e;
