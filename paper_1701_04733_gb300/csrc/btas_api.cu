@@ -703,9 +703,10 @@ btas_status btas_sssp(int64_t n, const int32_t *W, int64_t src, int32_t *dist, i
     // product checks the domain on its way through W), else
     // (BTAS_SSSP_NO_COOP=1, or no cooperative launch on this device) below
     if (n > 1 && n <= INT32_MAX / 4 && env_int("BTAS_SSSP_NO_COOP", 0) == 0) {
+        // (no room for the edge lists, up to n n bytes, is one more reason for the latter)
         Workspace cw(st);
-        BTAS_CUDA(cw.alloc(sssp_coop_workspace(n)), "workspace alloc");
-        const cudaError_t le = launch_sssp_coop(W, n, (int)src, dist, cw.p, st);
+        cudaError_t le = cw.alloc(sssp_coop_workspace(n));
+        if (le == cudaSuccess) le = launch_sssp_coop(W, n, (int)src, dist, cw.p, st);
         if (le == cudaSuccess) {
             int host[4] = {0, 0, 0, 0};
             BTAS_CUDA(read_back(host, sssp_coop_info(cw.p), 16, st), "info readback");
@@ -715,7 +716,7 @@ btas_status btas_sssp(int64_t n, const int32_t *W, int64_t src, int32_t *dist, i
             log_event("sssp n=%lld: cooperative kernel, %d changing products", (long long)n, host[0]);
             return BTAS_OK;
         }
-        if (le != cudaErrorCooperativeLaunchTooLarge && le != cudaErrorNotSupported)
+        if (le != cudaErrorCooperativeLaunchTooLarge && le != cudaErrorNotSupported && le != cudaErrorMemoryAllocation)
             return fail(BTAS_ERR_CUDA, "btas_sssp: %s", cudaGetErrorString(le));
         cudaGetLastError();
     }

@@ -1,0 +1,39 @@
+"""Calls on a device with little room left (BTAS_WS_LIMIT refuses larger pieces of workspace): what faster paths ask for
+beyond the ways they replaced is not needed, and the results are the same."""
+import contextlib
+import os
+
+import numpy as np
+import pytest
+
+import gen
+from tests.gpu_util import bits, dev, f32_matrix, host, int_matrix
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def btas():
+    import paper_1701_04733_gb300 as m
+    return m
+
+
+@contextlib.contextmanager
+def limit(nbytes):
+    os.environ["BTAS_WS_LIMIT"] = str(nbytes)
+    try:
+        yield
+    finally:
+        del os.environ["BTAS_WS_LIMIT"]
+
+
+@pytest.mark.parametrize("n", [40, 300, 1030])
+def test_sssp_without_edge_lists(btas, oracle_mod, n):
+    """Two vectors and 256 bytes, as one launch per product takes."""
+    W = gen.random_graph(gen.BASE_SEED, 61 + n, n, 0.1, 1, 1000)
+    want, info = btas.sssp(dev(W), 3, info=True)
+    with limit(256 + 2 * ((4 * n + 255) // 256 * 256)):
+        d, info1 = btas.sssp(dev(W), 3, info=True)
+    np.testing.assert_array_equal(host(d), host(want))
+    np.testing.assert_array_equal(host(d), oracle_mod.sssp(W, 3)[0])
+    assert info1["iterations"] == info["iterations"]
