@@ -559,8 +559,8 @@ btas_status btas_gemm(int semiring, int dtype, int64_t m, int64_t n, int64_t k, 
     // and 5.13 ms).  An operand that enough tiles read is copied to aligned rows
     // first, where that is more than the copy's launch costs (from 20 us of work).
     const bool worth = !(packed && dtype == BTAS_I32) && (double)m * n * k >= 4e8;
-    const bool pad_a = worth && n >= 512 && !aligned16(A, lda), pad_b = worth && trans_b && m >= 512 && !aligned16(B, ldb);
-    const size_t bt_bytes = trans_b && !pad_b ? 0 : align256((size_t)n * ldt * 4);
+    bool pad_a = worth && n >= 512 && !aligned16(A, lda), pad_b = worth && trans_b && m >= 512 && !aligned16(B, ldb);
+    size_t bt_bytes = trans_b && !pad_b ? 0 : align256((size_t)n * ldt * 4);
     const size_t a_bytes = pad_a ? align256((size_t)m * ldt * 4) : 0;
     int *pack_state = nullptr;
     if (packed && dtype == BTAS_I32) {
@@ -594,7 +594,14 @@ btas_status btas_gemm(int semiring, int dtype, int64_t m, int64_t n, int64_t k, 
                                      accumulate, st),
                   "packed result");
     } else if (bt_bytes + a_bytes) {
-        BTAS_CUDA(ws.alloc(bt_bytes + a_bytes), "workspace alloc");
+        cudaError_t e = ws.alloc(bt_bytes + a_bytes);
+        if (e == cudaErrorMemoryAllocation && (pad_a || pad_b)) {  // no room for the copies: staged as they are
+            cudaGetLastError();
+            pad_a = pad_b = false;
+            if (trans_b) bt_bytes = 0;
+            e = ws.alloc(bt_bytes);
+        }
+        BTAS_CUDA(e, "workspace alloc");
     }
     if (pad_b) {
         BTAS_CUDA(launch_pad4(B, ldb, (int)n, (int)k, ws.p, ldt, st), "aligned B");

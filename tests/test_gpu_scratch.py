@@ -37,3 +37,16 @@ def test_sssp_without_edge_lists(btas, oracle_mod, n):
     np.testing.assert_array_equal(host(d), host(want))
     np.testing.assert_array_equal(host(d), oracle_mod.sssp(W, 3)[0])
     assert info1["iterations"] == info["iterations"]
+
+
+@pytest.mark.parametrize("dt", ["i32", "f32"])
+@pytest.mark.parametrize("trans_b", [False, True])
+def test_product_without_aligned_copies(btas, oracle_mod, dt, trans_b):
+    """Rows off 16 bytes, in a product large enough for aligned copies: room for B's transpose, or for nothing."""
+    m, n, k = 700, 800, 801
+    make = int_matrix if dt == "i32" else f32_matrix
+    A, B = make(15, (m, k), 0), make(17, (k, n), 0)
+    Bd = dev(np.ascontiguousarray(B.T)) if trans_b else dev(B)
+    with limit(0 if trans_b else n * ((k + 3) // 4 * 4) * 4):
+        C = btas.gemm(dev(A), Bd, 0, trans_b=trans_b)
+    np.testing.assert_array_equal(bits(host(C)), bits(oracle_mod.tgemm(0, A, B)))
