@@ -926,7 +926,11 @@ static cudaError_t thread_workspace(MidThreadState &ts, size_t need, Workspace &
         return e;
     }
     if (ts.ws_bytes < need) {
-        if ((e = cudaMalloc(&ts.ws, kMidCachedWs)) != cudaSuccess) return e;
+        if (ws_refused(kMidCachedWs)) return cudaErrorMemoryAllocation;
+        if ((e = cudaMalloc(&ts.ws, kMidCachedWs)) != cudaSuccess) {
+            ts.ws = nullptr;
+            return e;
+        }
         ts.ws_bytes = kMidCachedWs;
         ts.ws_dev = dev;
     }
@@ -949,21 +953,27 @@ static cudaError_t wait_for_word(const int *word, cudaStream_t st) {
 }
 
 // Relaxation over sorted edge lists (relax.cu).  In place (D == W) it reads a
-// copy of W, left in copy_ws.  Returns a btas_status, or
-// kRelaxGaveUpFallback: D may then hold some columns already, and the caller
-// solves W (the copy, if there is one) another way.
+// copy of W.  Returns a btas_status, or kRelaxGaveUpFallback: W is then whole
+// (D, if it is another matrix, may hold some columns already), no scratch is
+// held any more, and the caller solves it another way.  No room for the
+// scratch is one more reason for that.
 constexpr int kRelaxGaveUpFallback = -1;
 constexpr int64_t kRelaxMinN = 48;  // up to it the one-block kernel is as fast (n = 48: 34-38 us per call both)
 
-static int apsp_relax_solve(int64_t n, const int32_t *W, int32_t *D, Workspace &copy_ws, cudaStream_t st) {
+static int apsp_relax_solve(int64_t n, const int32_t *W, int32_t *D, cudaStream_t st) {
     MidThreadState &ts = thread_state();
     if (!ts.mbox) return kRelaxGaveUpFallback;
-    Workspace ws(st);
+    Workspace ws(st), copy_ws(st);
     void *wsp = nullptr;
-    BTAS_CUDA(thread_workspace(ts, relax_workspace(n), ws, &wsp), "workspace alloc");
-    if (W == D) {
-        const size_t bytes = (size_t)n * (size_t)n * 4;
-        BTAS_CUDA(copy_ws.alloc(bytes), "workspace alloc");
+    const size_t bytes = (size_t)n * (size_t)n * 4;
+    cudaError_t e = thread_workspace(ts, relax_workspace(n), ws, &wsp);
+    if (e == cudaSuccess && W == D) e = copy_ws.alloc(bytes);
+    if (e == cudaErrorMemoryAllocation) {
+        cudaGetLastError();
+        return kRelaxGaveUpFallback;
+    }
+    BTAS_CUDA(e, "workspace alloc");
+    if (copy_ws.p) {
         BTAS_CUDA(cudaMemcpyAsync(copy_ws.p, W, bytes, cudaMemcpyDeviceToDevice, st), "copy");
         W = static_cast<const int32_t *>(copy_ws.p);
     }
@@ -988,7 +998,9 @@ static int apsp_relax_solve(int64_t n, const int32_t *W, int32_t *D, Workspace &
               n <= apsp_small_limit() ? "one-block kernel"
               : !dense && n <= kMidSparseMaxN ? "cooperative kernel" : "tiled kernels",
               wide ? "32" : "16", outcome == kRelaxDone ? "" : ", given up");
-    return outcome == kRelaxDone ? BTAS_OK : kRelaxGaveUpFallback;
+    if (outcome == kRelaxDone) return BTAS_OK;
+    if (copy_ws.p) BTAS_CUDA(cudaMemcpyAsync(D, copy_ws.p, bytes, cudaMemcpyDeviceToDevice, st), "copy");
+    return kRelaxGaveUpFallback;
 }
 
 static int apsp_mid_solve(int64_t n, const int32_t *W, int32_t *D, int S, bool early, bool packed_ok,
@@ -1064,13 +1076,11 @@ static btas_status apsp_impl(int64_t n, const int32_t *W, int32_t *D, int flags,
     // reach (from n = 2048; below it the squarings are as fast, 1.4-2.2 ms
     // against 1.6-2.2 ms).  Calls that ask for facts of the squaring
     // sequence (its length, its representations) run it.
-    Workspace copy_ws(st);
     if (!squarings_done && !bound_out && !path_out && flags == BTAS_APSP_EARLY_EXIT && n > kRelaxMinN &&
         !apsp_regime_pinned()) {
         if (n <= relax_max_n()) {
-            const int r = apsp_relax_solve(n, W, D, copy_ws, st);
+            const int r = apsp_relax_solve(n, W, D, st);
             if (r != kRelaxGaveUpFallback) return static_cast<btas_status>(r);
-            if (copy_ws.p) W = static_cast<const int32_t *>(copy_ws.p);
         }
         if (n >= 2048) {
             const btas_status r = btas_apsp_fw(n, W, D, st);

@@ -50,3 +50,25 @@ def test_product_without_aligned_copies(btas, oracle_mod, dt, trans_b):
     with limit(0 if trans_b else n * ((k + 3) // 4 * 4) * 4):
         C = btas.gemm(dev(A), Bd, 0, trans_b=trans_b)
     np.testing.assert_array_equal(bits(host(C)), bits(oracle_mod.tgemm(0, A, B)))
+
+
+@pytest.mark.parametrize("n", [100, 1000, 2100])
+def test_apsp_in_place_without_a_copy(btas, n):
+    """Room for the squarings' workspace that the thread keeps (or Floyd-Warshall's panels), not for a copy of W."""
+    W = gen.random_graph(gen.BASE_SEED, 63 + n, n, 0.02 if n > 100 else 0.2, 1, 100)
+    want = host(btas.apsp(dev(W)))
+    t = dev(W)
+    with limit(n * n * 4 - 1):
+        btas.apsp(t, out=t)
+    np.testing.assert_array_equal(host(t), want)
+
+
+def test_apsp_without_edge_lists(btas):
+    """n = 8200: the lists take more than the 32 MiB a thread keeps, Floyd-Warshall's panels a third of that."""
+    import torch
+    W = dev(gen.random_graph(gen.BASE_SEED, 65, 8200, 0.002, 1, 1000))
+    want = btas.apsp(W)
+    with limit(12 << 20):
+        D = btas.apsp(W)
+        btas.apsp(W, out=W)
+    assert torch.equal(D, want) and torch.equal(W, want)
