@@ -1416,8 +1416,14 @@ btas_status btas_apsp_paths(int64_t n, const int32_t *W, int32_t *D, int32_t *Ne
     const size_t flag_bytes = align256((size_t)(2 * S + 4) * 4);
     const size_t ak_bytes = keyed_ok ? align256((size_t)n * ldt * 4) : 0;
     const size_t list_bytes = keyed_ok ? edge_lists_workspace(n) : 0;
-    BTAS_CUDA(ws.alloc(flag_bytes + 4 * align256(nn * 4) + align256((size_t)n * ldt * 4) + ak_bytes + list_bytes),
-              "workspace alloc");
+    const size_t base_bytes = flag_bytes + 4 * align256(nn * 4) + align256((size_t)n * ldt * 4) + ak_bytes;
+    cudaError_t we = ws.alloc(base_bytes + list_bytes);
+    const bool list_room = list_bytes > 0 && we != cudaErrorMemoryAllocation;
+    if (we == cudaErrorMemoryAllocation && list_bytes > 0) {  // without the lists, then
+        cudaGetLastError();
+        we = ws.alloc(base_bytes);
+    }
+    BTAS_CUDA(we, "workspace alloc");
     char *base = static_cast<char *>(ws.p);
     int *dflags = reinterpret_cast<int *>(base);  // [2s] changed, [2s + 1] largest finite entry after squaring s
     int *Db[2], *Nb[2];
@@ -1433,7 +1439,7 @@ btas_status btas_apsp_paths(int64_t n, const int32_t *W, int32_t *D, int32_t *Ne
     // The first squaring of a sparse graph runs over edge lists (paths.cu's keys, one
     // term per pair of edges): n = 2048, p = 0.05: 532 -> 108 us.  Building the lists
     // checks the domain as well.
-    void *lists = keyed_ok ? reinterpret_cast<char *>(Ak) + ak_bytes : nullptr;
+    void *lists = list_room ? reinterpret_cast<char *>(Ak) + ak_bytes : nullptr;
     bool sparse = false;
     if (lists) {
         int host[3] = {0, 0, 0};

@@ -72,3 +72,23 @@ def test_apsp_without_edge_lists(btas):
         D = btas.apsp(W)
         btas.apsp(W, out=W)
     assert torch.equal(D, want) and torch.equal(W, want)
+
+
+@pytest.mark.parametrize("n", [130, 515])
+def test_next_hops_without_edge_lists(btas, n):
+    """Room for the matrices of the keyed squarings only; a sparse graph, whose first squaring would use the lists, and
+    a W outside the domain, which they would have found."""
+    W = gen.random_graph(gen.BASE_SEED, 67 + n, n, 0.05, 1, 100)
+    D, N, info = btas.apsp_paths(dev(W), info=True)
+    up = lambda x: (x + 255) // 256 * 256  # noqa: E731
+    S = int(np.ceil(np.log2(n - 1)))
+    pitch = (n + 3) // 4 * 4
+    with limit(up((2 * S + 4) * 4) + 4 * up(n * n * 4) + 2 * up(n * pitch * 4)):
+        D1, N1, info1 = btas.apsp_paths(dev(W), info=True)
+        W[3, 5] = -1
+        with pytest.raises(btas.BtasError) as ei:
+            btas.apsp_paths(dev(W))
+    assert ei.value.status == 1
+    np.testing.assert_array_equal(host(D1), host(D))
+    np.testing.assert_array_equal(host(N1), host(N))
+    assert info1["squarings"] == info["squarings"]
