@@ -1,5 +1,6 @@
-"""Batched APSP of matrices outside the domain, which a batch assumes and does not check: whatever the squarings make
-of them, and the graphs beside them unharmed."""
+"""Batched APSP of matrices outside the domain, which a batch assumes and does not check: the graphs beside them are
+unharmed, and in 32 bits the result is whatever the squarings make of them.  (Packed squarings rely on the domain to
+know which operands the next one needs, so theirs is not a function of W outside it.)"""
 import os
 
 import numpy as np
@@ -50,6 +51,7 @@ def test_as_the_squarings_give_them(btas, oracle_mod, value, where):
     finally:
         del os.environ["BTAS_BATCH_NO_RELAX"]
     for i, (x, y) in enumerate(zip(got, want)):
-        np.testing.assert_array_equal(x, y)
+        if i % 2 or (i // 2 == 2 and value > 0):  # n = 200: distances too large for the packed squarings
+            np.testing.assert_array_equal(x, y)
         if i % 2:
             np.testing.assert_array_equal(x, oracle_mod.floyd_warshall(graphs[i]))
