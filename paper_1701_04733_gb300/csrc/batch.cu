@@ -933,11 +933,16 @@ btas_status build_plan(btas_batch_t *b) {
                 }
             }
         } else if (I.kind == kInstRelax) {
-            I.relax_rows = relax_rows_for(I.n, relax_vectors, grid_ctas);
-            ws += al256(relax_inst_bytes(I.n));
+            I.relax_rows = relax_rows_for(I.n, relax_vectors, grid_ctas);  // its lists: with its squarings, below
         } else if (!I.trans_b) {
             I.ldq = (I.k + 3) & ~3LL;
             ws += al256((size_t)I.n * I.ldq * 4);
+        }
+        if (I.fallback) {
+            // no task of these squarings starts before every relaxation is done: the
+            // relaxation's lists lie in the same space
+            ws_off[I.relax_of] = ws_off[i];
+            ws = std::max(ws, ws_off[i] + al256(relax_inst_bytes(I.n)));
         }
         I.done_base = counters;
         I.flag_base = counters;

@@ -92,3 +92,33 @@ def test_next_hops_without_edge_lists(btas, n):
     np.testing.assert_array_equal(host(D1), host(D))
     np.testing.assert_array_equal(host(N1), host(N))
     assert info1["squarings"] == info["squarings"]
+
+
+def test_batch_needs_the_squarings_space_only(btas, oracle_mod):
+    """A solve's lists lie in the space of its squarings; with no time for the relaxations the squarings take it over."""
+    graphs = [gen.random_graph(gen.BASE_SEED, 69 + n, n, 0.1 if n > 10 else 0.5, 1, 100) for n in (3, 5, 9, 33, 300, 530)]
+
+    def batch():
+        b = btas.Batch()
+        outs = [b.add_apsp(dev(W), dev(np.zeros_like(W))) for W in graphs]
+        b.launch()
+        b.wait()
+        nbytes = b.workspace_bytes
+        b.close()
+        for W, D in zip(graphs, outs):
+            np.testing.assert_array_equal(host(D), oracle_mod.floyd_warshall(W))
+        return nbytes
+
+    got = batch()
+    os.environ["BTAS_RELAX_BUDGET"] = "-1"
+    try:
+        assert batch() == got
+    finally:
+        del os.environ["BTAS_RELAX_BUDGET"]
+    os.environ["BTAS_BATCH_NO_RELAX"] = "1"
+    try:
+        squarings = batch()
+    finally:
+        del os.environ["BTAS_BATCH_NO_RELAX"]
+    # lists of 32 rows are larger than the squarings' buffers of the smallest graphs only
+    assert squarings <= got <= squarings + 3 * 4096
