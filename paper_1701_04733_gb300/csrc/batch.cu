@@ -271,9 +271,8 @@ __device__ __noinline__ void relax_lists_task(const BInst &I, int t, unsigned ch
     }
 }
 
-// Relaxation, level 1: columns 8 R t .. 8 R t + 8 R - 1 of D.  A task that runs too long
-// (about four times what a random graph takes on an SM shared with product
-// tiles) gives the whole solve up.
+// Relaxation, level 1: columns 8 R t .. 8 R t + 8 R - 1 of D.  A task at the end of its
+// patience gives the whole solve up.
 template <int R>
 __device__ __noinline__ void relax_task(const BInst &I, int t, unsigned char *smem, int tid, int *done) {
     constexpr int T = relax::targets<true, R, 4>();
@@ -298,17 +297,16 @@ __device__ __noinline__ void relax_task(const BInst &I, int t, unsigned char *sm
     __syncthreads();
     bool wide = s_word[0] != 0 || relax::expects_wide(n, light);
     if (s_word[1] != 0) return;
-    const long long t0 = clock64(), budget = I.rl.budget;
-    auto give_up = [&]() {
+    const long long t0 = clock64();
+    auto give_up = [&](bool late) {
         if (ld_acquire(I.rstat + kRelaxGaveUpWord) != 0) return true;
-        if (clock64() - t0 <= (wide ? 2 : 1) * budget) return false;
-        if (atomicExch(I.rstat + kRelaxGaveUpWord, 1) == 0) atomicAdd(done + 1, 1);
-        return true;
+        if (late && atomicExch(I.rstat + kRelaxGaveUpWord, 1) == 0) atomicAdd(done + 1, 1);
+        return late;
     };
     if (!wide) {
         relax::load_columns<true, R, 4>(W, I.lda, n, Y, j0);
         __syncthreads();
-        if (!relax::solve<true, 1, R, 4>(W, I.lda, n, I.rl, Y, minw, give_up)) return;
+        if (!relax::solve<true, 1, R, 4>(W, I.lda, n, I.rl, Y, minw, t0, give_up)) return;
         wide = !relax::fits16<R, 4>(Y, n, maxw);
         if (!wide) relax::store_columns<true, R, 4>(D, I.ldc, n, Y, j0);
         else if (tid == 0) atomicOr(I.rstat + kRelaxWide, 1);
@@ -318,7 +316,7 @@ __device__ __noinline__ void relax_task(const BInst &I, int t, unsigned char *sm
             __syncthreads();
             relax::load_columns<false, R, 4>(W, I.lda, n, Y, j0 + h);
             __syncthreads();
-            if (!relax::solve<false, 1, R, 4>(W, I.lda, n, I.rl, Y, minw, give_up)) return;
+            if (!relax::solve<false, 1, R, 4>(W, I.lda, n, I.rl, Y, minw, t0, give_up)) return;
             relax::store_columns<false, R, 4>(D, I.ldc, n, Y, j0 + h);
         }
     }
@@ -684,8 +682,22 @@ void relax_inst_place(BInst &I, char *mem) {
     I.rl.edges = reinterpret_cast<uint4 *>(mem);
     I.rl.wide = reinterpret_cast<int4 *>(mem + relax::list_words(I.n) * 4);
     I.rl.next = reinterpret_cast<int *>(mem + relax::list_words(I.n) * 8);
+    // The patience of one task, with others on its SM: its share of the squarings'
+    // terms, at about the rate that they reach on half an SM (n = 1024: 6.4 M cycles
+    // for a task of 32 columns, measured 7.0 M).
+    I.rl.patience = relax::Patience{};
     const char *e = getenv("BTAS_RELAX_BUDGET");
-    I.rl.budget = e && *e ? atoll(e) : 4 * relax::budget_cycles(I.n);
+    if (e && *e) {
+        I.rl.patience.cycles = atoll(e);
+        return;
+    }
+    int squarings = 0;
+    while ((1LL << squarings) < I.n - 1) ++squarings;
+    const double worth = 300e3 + (double)squarings * I.n * I.n * I.relax_rows / 6.0;
+    I.rl.patience.by_share = true;
+    I.rl.patience.cycles = 4 * relax::budget_cycles(I.n);
+    I.rl.patience.worth16 = (long long)worth;
+    I.rl.patience.worth32 = (long long)(0.85 * worth);  // 1.7 times as much, in two halves
 }
 
 // Vectors of 8 targets a relaxation task solves at once.  Rows of 32 and 64

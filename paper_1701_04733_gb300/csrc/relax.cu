@@ -142,13 +142,12 @@ __global__ void __launch_bounds__(MAXT) relax_solve_kernel(const RelaxArgs a) {
     const bool wide_first = st.far != 0 || relax::expects_wide(n, st.light);  // the same in every block
     if (st.bad == 0 && s_abort == 0) {
         bool wide = wide_first || s_wide != 0;
-        auto give_up = [&]() {
+        auto give_up = [&](bool late) {
             if (*(volatile int *)(a.ctl + kAbort) != 0) return true;
-            if (clock64() - t0 <= (wide ? 2 : 1) * a.lists.budget) return false;
-            a.ctl[kAbort] = 1;
-            return true;
+            if (late) a.ctl[kAbort] = 1;
+            return late;
         };
-        if (part == 0 && !wide && relax::solve<true, G, R, NV>(a.W, a.ldw, n, a.lists, Y, st.minw, give_up)) {
+        if (part == 0 && !wide && relax::solve<true, G, R, NV>(a.W, a.ldw, n, a.lists, Y, st.minw, t0, give_up)) {
             wide = !relax::fits16<R, NV>(Y, n, st.maxw);
             if (!wide) relax::store_columns<true, R, NV>(a.D, a.ldd, n, Y, j0);
             else if (tid == 0) a.ctl[kWide] = 1;
@@ -160,7 +159,7 @@ __global__ void __launch_bounds__(MAXT) relax_solve_kernel(const RelaxArgs a) {
                 __syncthreads();
                 relax::load_columns<false, R, NV>(a.W, a.ldw, n, Y, j0 + h);
                 __syncthreads();
-                if (!relax::solve<false, G, R, NV>(a.W, a.ldw, n, a.lists, Y, st.minw, give_up)) break;
+                if (!relax::solve<false, G, R, NV>(a.W, a.ldw, n, a.lists, Y, st.minw, t0, give_up)) break;
                 relax::store_columns<false, R, NV>(a.D, a.ldd, n, Y, j0 + h);
             }
         }
@@ -273,6 +272,26 @@ cudaError_t launch_sparse_keys(const int *W, int n, void *ws, int shift, int *K,
     return cudaGetLastError();
 }
 
+// A block's patience in a call of its own, `resident` blocks running at once.
+// What a call takes where its relaxation is given up, in cycles (chains, GB300):
+// below n = 2048 the squarings, 68 us at n = 128, 148 at 512, 555 at 1024, 3280 at 2047
+// in 16 bits and 73, 180, 805, 5300 in 32; from there on blocked Floyd-Warshall,
+// 2.1 ms at n = 2048, 5.4 at 4096.
+static relax::Patience relax_patience(long long n, int blocks, int resident, bool split) {
+    relax::Patience p{};
+    if (const char *e = getenv("BTAS_RELAX_BUDGET"); e && *e) {
+        p.cycles = atoll(e);
+        return p;
+    }
+    p.by_share = true;
+    p.cycles = relax::budget_cycles(n);
+    const double n3 = (double)n * n * n, share = std::min(1.0, (double)resident / blocks);
+    p.worth16 = (long long)(share * (n < 2048 ? 110e3 + 120.0 * n + n3 / 1500 : 1730.0 * n + n3 / 20000));
+    p.worth32 = (long long)(share * (n < 2048 ? 110e3 + 120.0 * n + n3 / 900 : 1730.0 * n + n3 / 20000));
+    if (!split) p.worth32 /= 2;  // one half of the targets after the other
+    return p;
+}
+
 cudaError_t launch_relax(const int *W, long long ldw, int n, int *D, long long ldd, void *ws, int *out,
                          cudaStream_t st) {
     const int blocks = (n + kListWarps - 1) / kListWarps;
@@ -283,8 +302,6 @@ cudaError_t launch_relax(const int *W, long long ldw, int n, int *D, long long l
     a.D = D;
     a.ldd = ldd;
     a.out = out;
-    const char *bud = getenv("BTAS_RELAX_BUDGET");
-    a.lists.budget = bud && *bud ? atoll(bud) : relax::budget_cycles(n);
     place(ws, n, &a.ctl, &a.stats, &a.lists);
     // Two blocks share a block's targets in 32 bits while one wave holds them all (n =
     // 1024, w <= 10^6, p = 0.5: 283 -> 158 us per call).
@@ -317,6 +334,9 @@ cudaError_t launch_relax(const int *W, long long ldw, int n, int *D, long long l
     at.val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = &at;
     cfg.numAttrs = 1;
+    DeviceInfo di{};
+    a.lists.patience = relax_patience(n, cfg.gridDim.x, (maxt == 1024 ? 1 : 2) * (current_device_info(&di) ? di.sms : 152),
+                                      a.halves == 2);
     e = cudaLaunchKernelEx(&cfg, kern, a);
     if (e == cudaSuccess) note_launch();
     return e;

@@ -28,13 +28,30 @@ constexpr int kPadChunks = 2;      // chunks of pads after a list: one per lane 
 constexpr int kEarlySweeps = 2, kEarlyChunks = 2;  // solve's first sweeps
 constexpr int kSample = 1024;      // entries the first guess of a long row's cutoff is taken from
 
+// When a block gives its solve up.  Random graphs, of any density and any
+// weights, are solved in 10 to 23 sweeps (n = 49 ... 8192).  Shortest paths of
+// many edges take more, and there are two kinds of graphs with such paths.
+// - Distances are still missing after 8 sweeps (chains, rings, grids, lattices,
+//   and the sparsest random graphs).  They are found at an even pace or a growing
+//   one until all are, so the share found, or what the last 8 sweeps added to it,
+//   says what the solve will take.  From kSettle sweeps on it goes on while that
+//   is less than what solving otherwise is worth.
+// - All are known by then and some still improve: nothing tells for how long,
+//   and `cycles` end it.
+struct Patience {
+    bool by_share;     // false: `cycles` alone counts (tests)
+    long long cycles;  // about twice what the slowest random graphs take
+    long long worth16, worth32;  // a block's share of what solving otherwise takes, where 16 bits do and where not
+};
+constexpr int kSettle = 24;
+
 struct Lists {
     uint4 *edges;  // [ceil(n / 32)][chunks][32]
     int4 *wide;    // the weights in 32 bits, same places
     int *next;     // n words
     int *len;      // optional: edges in each list
     int chunks;    // capacity / 4
-    long long budget;  // clock cycles after which a block gives up
+    Patience patience;
     // > 0: only lists of whole rows are of use, of at most `whole` edges, none
     // heavier than `top`; other rows are counted and no more
     int whole, top;
@@ -484,6 +501,45 @@ __device__ __forceinline__ void store_columns(int *D, long long ldd, int n, cons
     }
 }
 
+struct Looks {   // in shared memory, cleared by thread 0 before a solve's first sweep
+    int found;     // entries
+    bool finding;  // distances were missing after 8 sweeps
+    float last_found, last_t;
+};
+
+// Whether the block's patience is at its end, asked after every 8 sweeps; valid in
+// thread 0.  t0, start: the clock when the solve and when the block began.
+// Called by the whole block, rarely: it stays out of the sweeps' registers.
+template <bool U16, int R, int NV>
+__device__ __noinline__ bool late(const Patience &p, const Vec<NV> *Y, int n, int sweeps, long long t0,
+                                  long long start, Looks &k) {
+    if (sweeps > 8 && !k.finding) return threadIdx.x == 0 && clock64() - start > (U16 ? 1 : 2) * p.cycles;
+    if (threadIdx.x == 0) k.found = 0;
+    int c = 0;
+    for (int i = threadIdx.x; i < n * R; i += blockDim.x) {
+        const Vec<NV> y = lds_relaxed(Y + i);
+#pragma unroll
+        for (int q = 0; q < NV; ++q) {
+            if (U16) c += ((y.w[q] & 0xFFFFu) != BTAS_INF_U16) + ((y.w[q] >> 16) != BTAS_INF_U16);
+            else c += (int)y.w[q] < kInfI32;
+        }
+    }
+    c = __reduce_add_sync(0xffffffffu, c);
+    __syncthreads();
+    if ((threadIdx.x & 31) == 0) atomicAdd(&k.found, c);
+    __syncthreads();
+    if (threadIdx.x != 0) return false;
+    const float found = (float)k.found / ((float)n * (float)targets<U16, R, NV>());
+    if (sweeps == 8) k.finding = p.by_share && found < 0.9f;
+    if (!k.finding) return clock64() - start > (U16 ? 1 : 2) * p.cycles;
+    const float t = (float)(clock64() - t0), worth = (float)(U16 ? p.worth16 : p.worth32);
+    const float more = (1.0f - found) * (t - k.last_t) / fmaxf(found - k.last_found, 1e-6f);
+    k.last_found = found;
+    k.last_t = t;
+    if (found >= 0.9f) return t > 1.5f * worth;  // near its end: worth a little more
+    return sweeps < kSettle ? t > worth : fminf(t / found, t + more) > worth;
+}
+
 // Sweeps over all vertices until Y is the closure's columns.  A sweep lowers
 // every Y[v] through v's edges, R lanes to a vertex's row and G sets of them to
 // a vertex (set g takes chunks g, g + G, ...).  A path of two or more edges that
@@ -494,17 +550,21 @@ __device__ __forceinline__ void store_columns(int *D, long long ldd, int n, cons
 // from W itself, and the sweeps go on if that lowered anything.  In the end
 // every edge that could lower an entry has been tried against final values.
 //
-// One thread asks give_up() from time to time; returns false if it said so.
-// Called by the whole block.
+// One thread asks give_up(late) from time to time, late: this block's patience
+// is at its end; returns false if it said so.  start: the clock when the block
+// began, earlier solves included.  Called by the whole block.
 template <bool U16, int G, int R, int NV, class GiveUp>
 __device__ __forceinline__ bool solve(const int *W, long long ldw, int n, const Lists &l, Vec<NV> *Y, int minw,
-                                      GiveUp give_up) {
+                                      long long start, GiveUp give_up) {
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, nwarps = blockDim.x >> 5;
     constexpr int VW = 32 / (G * R);  // vertices of a warp
     static_assert(G <= kPadChunks, "every lane's share of a list ends with a pad chunk");
     const int sub = lane % R, g = (lane / R) % G;
     const Vec<NV> *Ys = Y + sub;  // Ys[v * R]: this lane's part of v's row
     int sweeps = 0;
+    const long long t0 = clock64();
+    __shared__ Looks looks;
+    if (tid == 0) looks = Looks{0, false, 0.0f, 0.0f};
     for (;;) {
         for (;;) {
             bool ch = false, cut = false;
@@ -565,7 +625,10 @@ __device__ __forceinline__ bool solve(const int *W, long long ldw, int n, const 
                 }
             }
             if (!__syncthreads_or(ch || cut)) break;
-            if ((sweeps & 7) == 0 && __syncthreads_or(tid == 0 && give_up())) return false;
+            if ((sweeps & 7) == 0) {
+                const bool l8 = late<U16, R, NV>(l.patience, Y, n, sweeps, t0, start, looks);
+                if (__syncthreads_or(tid == 0 && give_up(l8))) return false;
+            }
         }
         bool ch = false;
         for (int v0 = warp * VW; v0 < n; v0 += nwarps * VW) {
@@ -595,7 +658,8 @@ __device__ __forceinline__ bool solve(const int *W, long long ldw, int n, const 
             }
         }
         if (!__syncthreads_or(ch)) return true;
-        if (__syncthreads_or(tid == 0 && give_up())) return false;
+        // (reading whole rows takes many sweeps' time)
+        if (__syncthreads_or(tid == 0 && give_up(clock64() - start > (U16 ? 1 : 2) * l.patience.cycles))) return false;
     }
 }
 
