@@ -535,6 +535,12 @@ btas_status btas_apsp_noalloc_status(void *stream, int *squarings_done);
  *                  winner's raster groups, stores the best in the table and
  *                  fills *out (may be NULL).  Synchronises `stream`; takes
  *                  about 20 ms per candidate plus four products each.
+ *                  Candidates are timed with whole k ranges.  A product
+ *                  that only writes C (no accumulate, checked or packed)
+ *                  may share a tile's k range over several CTAs; where the
+ *                  untuned choice, timed as such a call runs it, is faster
+ *                  than the winner, the entry says so and such products
+ *                  stay untuned ("defaults": 1 in a saved line).
  *                  semiring: BTAS_MINPLUS/BTAS_MAXPLUS; dtype: BTAS_I32,
  *                  BTAS_F32, or BTAS_U16 (min-plus only).  m, n, k >= 1.
  * btas_tune_lookup: 1 and *out filled if the table has an entry for the

@@ -285,55 +285,69 @@ double nt_stream_time(double m, double n, double k, int sms) {
     return steps * 32 * 128 * 128 * 2 / 59 / 2000.0 + 4.0 + m * n * 0.5e-6;
 }
 
+// The untuned choice: int32 = IMAD/3-input-min mix, fp32 = add.f32x2 + 3-input
+// min, on the tiles that nt_time() expects to be fastest: 128 x 128 at 2 CTAs/SM
+// for large products (8192^3: at the measured issue ceilings of their instruction
+// mixes), 64 x 64 and 32 x 32 where those would leave SMs idle.
+NtPlan default_plan(int dtype, int sr, long long m, long long n, long long k, bool may_split, int sms) {
+    NtPlan plan;
+    double best = 0, time = 0;
+    for (int cfg : {4, 6, 7}) {
+        const int ns = dtype == BTAS_F32 ? 0 : cfg == 7 ? 2 : 4;
+        const GemmKernel *g = find_gemm_kernel(dtype == BTAS_F32 ? kF32X2 : kI32Mix, sr, ns, cfg);
+        if (!g) continue;
+        int s = 1;
+        if (may_split) s = nt_splits(*g, dtype, m, n, k, sms, &time);
+        else time = nt_time(*g, dtype, (double)m, (double)n, (double)k, 1, sms);
+        if (!plan.kernel || time < best) {
+            best = time;
+            plan.kernel = g;
+            plan.splits = s;
+        }
+    }
+    // shares of at least four k steps
+    if (may_split && ((m + 127) / 128) * ((n + 127) / 128) * ((k + 31) / 32) >= 8LL * sms &&
+        nt_stream_time((double)m, (double)n, (double)k, sms) < best) {
+        plan.kernel = find_gemm_kernel(dtype == BTAS_F32 ? kF32X2 : kI32Mix, sr, dtype == BTAS_F32 ? 0 : 4, 4);
+        plan.splits = 1;
+        plan.stream_k = 2 * sms;
+    }
+    return plan;
+}
+
+NtPlan tuned_plan(const GemmKernel *g, int group_m, int dtype, long long m, long long n, long long k, bool may_split,
+                  int sms) {
+    NtPlan plan;
+    double time = 0;
+    plan.kernel = g;
+    plan.group_m = group_m;
+    if (may_split && g->merges) plan.splits = nt_splits(*g, dtype, m, n, k, sms, &time);
+    return plan;
+}
+
 // Kernel choice.  Explicit environment overrides win: BTAS_I32_VARIANT (0 =
 // DPX, 1 = mixed), BTAS_I32_NS, BTAS_F32_VARIANT (2 = f32x2, 3 = scalar, 4 =
 // two scalar adds + 3-input min) and BTAS_CFG.  Otherwise an autotuner entry
-// for the problem's size buckets (tune.cu), else int32 = IMAD/3-input-min mix,
-// fp32 = add.f32x2 + 3-input min, on the tiles that nt_time() expects to be
-// fastest: 128 x 128 at 2 CTAs/SM for large products (8192^3: at the measured
-// issue ceilings of their instruction mixes), 64 x 64 and 32 x 32 where those
-// would leave SMs idle.  may_split: the k range of a tile may be shared out over
-// several CTAs (products that only write C), except with BTAS_CFG.
+// for the problem's size buckets (tune.cu), unless the tuner found the untuned
+// choice faster, else that choice.  may_split: the k range of a tile may be
+// shared out over several CTAs (products that only write C), except with
+// BTAS_CFG.
 NtPlan plan_nt(int dtype, int sr, long long m, long long n, long long k, bool may_split, cudaStream_t st) {
     NtPlan plan;
     DeviceInfo di{};
     const int sms = current_device_info(&di) ? di.sms : 152;
     const bool forced = getenv("BTAS_I32_VARIANT") || getenv("BTAS_I32_NS") || getenv("BTAS_F32_VARIANT") ||
                         getenv("BTAS_CFG");
-    double time = 0;
     TuneChoice c{};
     const char *from = forced ? "environment" : "defaults";
-    if (!forced && tune_choice(sr, dtype, m, n, k, st, &c)) {
-        plan.kernel = find_gemm_kernel(c.var, sr, c.ns, c.cfg);
-        if (plan.kernel) {
-            plan.group_m = c.group_m;
-            if (may_split && plan.kernel->merges) plan.splits = nt_splits(*plan.kernel, dtype, m, n, k, sms, &time);
+    if (!forced && tune_choice(sr, dtype, m, n, k, st, &c) && !(may_split && c.defaults)) {
+        const GemmKernel *g = find_gemm_kernel(c.var, sr, c.ns, c.cfg);
+        if (g) {
+            plan = tuned_plan(g, c.group_m, dtype, m, n, k, may_split, sms);
             from = "autotuner";
         }
     }
-    if (!plan.kernel && !forced) {
-        double best = 0;
-        for (int cfg : {4, 6, 7}) {
-            const int ns = dtype == BTAS_F32 ? 0 : cfg == 7 ? 2 : 4;
-            const GemmKernel *g = find_gemm_kernel(dtype == BTAS_F32 ? kF32X2 : kI32Mix, sr, ns, cfg);
-            if (!g) continue;
-            int s = 1;
-            if (may_split) s = nt_splits(*g, dtype, m, n, k, sms, &time);
-            else time = nt_time(*g, dtype, (double)m, (double)n, (double)k, 1, sms);
-            if (!plan.kernel || time < best) {
-                best = time;
-                plan.kernel = g;
-                plan.splits = s;
-            }
-        }
-        // shares of at least four k steps
-        if (may_split && ((m + 127) / 128) * ((n + 127) / 128) * ((k + 31) / 32) >= 8LL * sms &&
-            nt_stream_time((double)m, (double)n, (double)k, sms) < best) {
-            plan.kernel = find_gemm_kernel(dtype == BTAS_F32 ? kF32X2 : kI32Mix, sr, dtype == BTAS_F32 ? 0 : 4, 4);
-            plan.splits = 1;
-            plan.stream_k = 2 * sms;
-        }
-    }
+    if (!plan.kernel && !forced) plan = default_plan(dtype, sr, m, n, k, may_split, sms);
     if (!plan.kernel) {
         int var, ns = 0;
         if (dtype == BTAS_F32) {
@@ -415,6 +429,19 @@ btas_status run_nt(int dtype, int sr, const GemmArgs &a, cudaStream_t st, const 
 
 
 }  // namespace
+
+cudaError_t btas::launch_nt_product(int dtype, int sr, const GemmArgs &a, const GemmKernel *g, int group_m,
+                                    cudaStream_t st) {
+    DeviceInfo di{};
+    const int sms = current_device_info(&di) ? di.sms : 152;
+    const NtPlan plan = g ? tuned_plan(g, group_m, dtype, a.m, a.n, a.k, true, sms)
+                          : default_plan(dtype, sr, a.m, a.n, a.k, true, sms);
+    if (plan.merges()) {
+        const cudaError_t e = launch_fill4(a.C, a.ldc, a.m, a.n, ident_bits(dtype, sr), st);
+        if (e != cudaSuccess) return e;
+    }
+    return run_nt(dtype, sr, a, st, &plan) == BTAS_OK ? cudaSuccess : cudaErrorInvalidDeviceFunction;
+}
 
 namespace btas {
 void record_error(const char *msg) { g_err = msg; }

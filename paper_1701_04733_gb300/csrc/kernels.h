@@ -49,7 +49,11 @@ const GemmKernel *gemm_kernel_at(int i);
 // ---- autotuner (tune.cu)
 struct TuneChoice {
     int var, ns, cfg, group_m;  // var 16: packed u16x2 kernel (ns = its IMAD split)
+    bool defaults;  // a product that only writes C ran faster untuned: tiles and k split by expected time
 };
+// A product that only writes C, as a call runs it untuned (g null) or tuned to kernel
+// g: with its k split and the filling of C that a split needs.
+cudaError_t launch_nt_product(int dtype, int sr, const GemmArgs &a, const GemmKernel *g, int group_m, cudaStream_t st);
 // Tuned kernel for (sr, dtype, m, n, k) on the current device: a table entry,
 // or -- when BTAS_TUNE=1 and `st` is not capturing -- a tuning run on the
 // spot.  false: no choice (use the defaults).

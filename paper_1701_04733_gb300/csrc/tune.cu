@@ -8,8 +8,12 @@
 // that all candidates agree bit for bit, then tries the winner with several
 // tile-raster group heights, and keeps the fastest in a process-wide table
 // keyed by (compute capability, SM count, semiring, dtype, ceil(log2) size
-// buckets of m, n, k).  The table can be saved to and loaded from a file of
-// JSON lines.
+// buckets of m, n, k).  The candidates are timed with whole k ranges.  A call
+// that only writes C may share a tile's k range over several CTAs, and untuned
+// it also knows smaller tiles and other shares; so the winner is timed once more
+// as such a call runs it, beside the untuned choice, and where that is faster the
+// entry says so and such calls stay untuned.  The table can be saved to and
+// loaded from a file of JSON lines.
 #include <algorithm>
 #include <cmath>
 #include <cstdio>
@@ -42,6 +46,7 @@ struct Key {
 struct Entry {
     int var, ns, cfg, group_m, candidates, tile_m, tile_n;
     double seconds, tps;
+    bool defaults;  // a product that only writes C ran faster untuned
 };
 
 std::mutex g_mu;
@@ -74,9 +79,10 @@ bool make_key(int sr, int dtype, long long m, long long n, long long k, Key *key
 #define BTAS_TUNE_LINE(F)                                                                                     \
     "{\"arch\": %d, \"sms\": %d, \"semiring\": %d, \"dtype\": %d, \"m_bucket\": %d, \"n_bucket\": %d, "         \
     "\"k_bucket\": %d, \"variant\": %d, \"ns\": %d, \"cfg\": %d, \"group_m\": %d, \"candidates\": %d, "         \
-    "\"tile_m\": %d, \"tile_n\": %d, \"seconds\": " F ", \"terms_per_second\": " F "}"
+    "\"tile_m\": %d, \"tile_n\": %d, \"seconds\": " F ", \"terms_per_second\": " F
 const char *kReadFmt = BTAS_TUNE_LINE("%lg");
 const char *kWriteFmt = BTAS_TUNE_LINE("%.9g");
+const char *kDefaults = "\"defaults\": 1";  // optional last key
 
 bool valid_entry(const Key &k, const Entry &e) {
     if (k.sr != kMin && k.sr != kMax) return false;
@@ -116,6 +122,7 @@ int load_file(const char *path, std::string *err) {
                    (got_n != 16 ? " is not a tuning entry" : " names a kernel this build does not have");
             return -1;
         }
+        e.defaults = strstr(p, kDefaults) != nullptr;
         got.emplace_back(k, e);
     }
     fclose(f);
@@ -141,7 +148,7 @@ int save_file(const char *path, std::string *err) {
         const Entry &e = kv.second;
         fprintf(f, kWriteFmt, k.arch, k.sms, k.sr, k.dtype, k.mb, k.nb, k.kb, e.var, e.ns, e.cfg, e.group_m,
                 e.candidates, e.tile_m, e.tile_n, e.seconds, e.tps);
-        fputc('\n', f);
+        fprintf(f, "%s%s}\n", e.defaults ? ", " : "", e.defaults ? kDefaults : "");
     }
     const bool ok = fflush(f) == 0;
     fclose(f);
@@ -289,7 +296,7 @@ int tune_run(int sr, int dtype, long long m, long long n, long long k, cudaStrea
         for (int i = 0; i < gemm_kernel_count(); ++i) {
             const GemmKernel *g = gemm_kernel_at(i);
             const bool is_f32 = g->var == kF32X2 || g->var == kF32Scalar || g->var == kF32Add2;
-            // (the 32 x 32 tiles live from the k split, which is not timed here)
+            // (the 32 x 32 tiles live from the k split: among the untuned choices below)
             if (g->sr == sr && is_f32 == (dtype == BTAS_F32) && g->bm >= 64)
                 cands.push_back(Candidate{g->var, g->ns, g->cfg, g->bm, g->bn, g});
         }
@@ -346,6 +353,14 @@ int tune_run(int sr, int dtype, long long m, long long n, long long k, cudaStrea
             return c.k->launch(a, st);
         };
     };
+    // entries of C that differ from R
+    auto differing = [&](unsigned long long *h) -> cudaError_t {
+        cudaMemsetAsync(cnt, 0, 8, st);
+        tune_diff_kernel<<<grid_of(m * n), 256, 0, st>>>(C, R, m, n, ldn, es, cnt);
+        note_launch();
+        const cudaError_t d = cudaMemcpyAsync(h, cnt, 8, cudaMemcpyDeviceToHost, st);
+        return d == cudaSuccess ? cudaStreamSynchronize(st) : d;
+    };
     Events ev;
     double best = 1e30;
     int bi = -1;
@@ -359,12 +374,8 @@ int tune_run(int sr, int dtype, long long m, long long n, long long k, cudaStrea
         if (i == 0) {
             e = cudaMemcpyAsync(R, C, (size_t)m * ldn * es, cudaMemcpyDeviceToDevice, st);
         } else {
-            cudaMemsetAsync(cnt, 0, 8, st);
-            tune_diff_kernel<<<grid_of(m * n), 256, 0, st>>>(C, R, m, n, ldn, es, cnt);
-            note_launch();
             unsigned long long h = 0;
-            e = cudaMemcpyAsync(&h, cnt, 8, cudaMemcpyDeviceToHost, st);
-            if (e == cudaSuccess) e = cudaStreamSynchronize(st);
+            e = differing(&h);
             if (e == cudaSuccess && h != 0) {
                 char b[256];
                 snprintf(b, sizeof b,
@@ -400,13 +411,37 @@ int tune_run(int sr, int dtype, long long m, long long n, long long k, cudaStrea
         }
     }
     const Candidate &w = cands[bi];
+    bool defaults = false;
+    if (w.k) {
+        GemmArgs a{};
+        a.m = (int)m; a.n = (int)n; a.k = (int)k;
+        a.A = A; a.lda = ldk;
+        a.Bt = B; a.ldb = ldk;
+        a.C = C; a.ldc = ldn;
+        a.vec_a = a.vec_b = 1;
+        double tuned = 0, untuned = 0;
+        e = time_call([&] { return launch_nt_product(dtype, sr, a, w.k, best_group, st); }, st, ev, &tuned);
+        if (e == cudaSuccess)
+            e = time_call([&] { return launch_nt_product(dtype, sr, a, nullptr, 8, st); }, st, ev, &untuned);
+        unsigned long long h = 0;
+        if (e == cudaSuccess) e = differing(&h);
+        if (e != cudaSuccess) {
+            *msg = std::string("btas_tune_gemm: ") + cudaGetErrorString(e);
+            return BTAS_ERR_CUDA;
+        }
+        if (h != 0) {
+            *msg = "btas_tune_gemm: the untuned choice differs from the candidates";
+            return BTAS_ERR_INTERNAL;
+        }
+        defaults = untuned < 0.98 * tuned;
+    }
     Entry ent{w.var, w.ns, w.cfg, best_group, (int)cands.size(), w.tile_m, w.tile_n, best,
-              (double)m * n * k / best};
+              (double)m * n * k / best, defaults};
     {
         std::lock_guard<std::mutex> lk(g_mu);
         g_table[key] = ent;
     }
-    if (choice) *choice = TuneChoice{ent.var, ent.ns, ent.cfg, ent.group_m};
+    if (choice) *choice = TuneChoice{ent.var, ent.ns, ent.cfg, ent.group_m, ent.defaults};
     if (res) *res = btas_tune_result{ent.var, ent.ns, ent.cfg, ent.tile_m, ent.tile_n, ent.group_m,
                                      ent.candidates, ent.seconds, ent.tps};
     return BTAS_OK;
@@ -420,7 +455,7 @@ bool tune_choice(int sr, int dtype, long long m, long long n, long long k, cudaS
         std::lock_guard<std::mutex> lk(g_mu);
         auto it = g_table.find(key);
         if (it != g_table.end()) {
-            *out = TuneChoice{it->second.var, it->second.ns, it->second.cfg, it->second.group_m};
+            *out = TuneChoice{it->second.var, it->second.ns, it->second.cfg, it->second.group_m, it->second.defaults};
             return true;
         }
     }
