@@ -1016,12 +1016,12 @@ static int apsp_relax_solve(int64_t n, const int32_t *W, int32_t *D, cudaStream_
                     bad);
     if (outcome != kRelaxDone && outcome != kRelaxGaveUp)
         return fail((btas_status)BTAS_ERR_INTERNAL, "btas_apsp: the relaxation left no outcome");
-    // the log names the size regime of the squarings that this replaces
+    // the log also names the kernels that the squarings would have run on
     const bool dense = n > apsp_mid_max_n() && n <= kMidSparseMaxN && deg > apsp_mid_list_cap(n);
     if (dense)
-        log_event("apsp n=%lld: too dense for the cooperative kernel's edge lists (%d edges in a row)", (long long)n,
+        log_event("apsp n=%lld: too dense for the cooperative kernel's edge lists (a row of %d edges)", (long long)n,
                   deg);
-    log_event("apsp n=%lld: %s range, relaxation over sorted edge lists in %s bits%s", (long long)n,
+    log_event("apsp n=%lld: %s replaced by relaxation over sorted edge lists in %s bits%s", (long long)n,
               n <= apsp_small_limit() ? "one-block kernel"
               : !dense && n <= kMidSparseMaxN ? "cooperative kernel" : "tiled kernels",
               wide ? "32" : "16", outcome == kRelaxDone ? "" : ", given up");
@@ -1112,7 +1112,7 @@ static btas_status apsp_impl(int64_t n, const int32_t *W, int32_t *D, int flags,
         if (n >= 2048) {
             const btas_status r = btas_apsp_fw(n, W, D, st);
             if (r != BTAS_OK) return r;
-            log_event("apsp n=%lld: tiled kernels range, blocked Floyd-Warshall", (long long)n);
+            log_event("apsp n=%lld: tiled kernels replaced by blocked Floyd-Warshall", (long long)n);
             return BTAS_OK;
         }
     }
