@@ -141,7 +141,7 @@ struct btas_server_t {
     void *h_stage[2] = {nullptr, nullptr};
     size_t stage_bytes = 0;
     int *h_flags = nullptr;  // pinned mailbox: change flags, maxima or barrier status, domain-scan results
-    int *h_rstat = nullptr;  // pinned: kRelaxWords words per relaxation of a step
+    const int *h_rstat = nullptr;  // kRelaxWords words per relaxation of the latest step, in its pinned staging
     int *d_flag_slots = nullptr;
     int flag_slots = 0;
     cudaEvent_t step_done[2] = {nullptr, nullptr};
@@ -489,9 +489,12 @@ int launch_step(btas_server_t *sv, std::vector<Req *> &units) {
                         cudaMemcpyDeviceToHost, sv->compute);
     }
     cudaMemcpyAsync(sv->h_flags + sv->flag_slots, p.status, 4, cudaMemcpyDeviceToHost, sv->compute);
-    if (nrelax > 0)
-        cudaMemcpyAsync(sv->h_rstat, cnt + rstat_at, (size_t)kRelaxWords * nrelax * 4, cudaMemcpyDeviceToHost,
-                        sv->compute);
+    if (nrelax > 0) {
+        // back to the place they were cleared from
+        int *words = reinterpret_cast<int *>(h) + rstat_at;
+        cudaMemcpyAsync(words, cnt + rstat_at, (size_t)kRelaxWords * nrelax * 4, cudaMemcpyDeviceToHost, sv->compute);
+        sv->h_rstat = words;
+    }
     } else {
         sv->h_flags[sv->flag_slots] = 0;
     }
@@ -797,10 +800,7 @@ btas_status btas_server_create(btas_server_t **out, int64_t hbm_budget_bytes, in
     if (const char *e = getenv("BTAS_SERVER_BULK_TERMS")) sv->bulk_terms = atof(e);
     sv->timeout_cycles = batch_timeout_cycles(sv->device);
     sv->flag_slots = 1 << 16;
-    if (cudaMallocHost(reinterpret_cast<void **>(&sv->h_flags), (size_t)(3 * sv->flag_slots + 1) * 4) != cudaSuccess ||
-        cudaMallocHost(reinterpret_cast<void **>(&sv->h_rstat), (size_t)kRelaxWords * sv->flag_slots * 4) !=
-            cudaSuccess) {
-        if (sv->h_flags) cudaFreeHost(sv->h_flags);
+    if (cudaMallocHost(reinterpret_cast<void **>(&sv->h_flags), (size_t)(3 * sv->flag_slots + 1) * 4) != cudaSuccess) {
         delete sv;
         return sfail(BTAS_ERR_NOMEM, "btas_server_create: pinned mailbox");
     }
@@ -939,7 +939,6 @@ btas_status btas_server_destroy(btas_server_t *sv) {
         if (sv->step_done[q]) cudaEventDestroy(sv->step_done[q]);
     }
     if (sv->h_flags) cudaFreeHost(sv->h_flags);
-    if (sv->h_rstat) cudaFreeHost(sv->h_rstat);
     cudaStreamSynchronize(sv->copy);
     cudaStreamDestroy(sv->compute);
     cudaStreamDestroy(sv->copy);
