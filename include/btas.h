@@ -696,10 +696,15 @@ btas_status btas_batch_select_tiles(btas_batch_t *b, void *stream, int *mode, do
  * squaring) in one persistent launch; requests arriving meanwhile join the
  * next step.  A product completes after its step; an APSP solve after its
  * last squaring or as soon as a squaring changed nothing.  An APSP request
- * with n <= 1792 is instead solved whole in one unit, by the one-block or
- * the cooperative kernel of btas_apsp (the same size boundary), launched in the step
- * after the persistent kernel (BTAS_SERVER_NO_WHOLE=1 in the environment at
- * creation turns this off).  Results are bit-identical to btas_gemm /
+ * with 16 <= n <= 1792 starts as one unit of its own, the whole solve by
+ * relaxation as in btas_apsp, as tasks of the step's launch; a solve that is
+ * given up goes on as above from the next step
+ * (BTAS_SERVER_NO_RELAX=1 in the environment at creation: no relaxations).
+ * Where the rest of the pending work is light, such a solve, or one of n < 16,
+ * is done whole by the one-block or the cooperative kernel of btas_apsp
+ * instead, launched in the step after the persistent kernel.
+ * BTAS_SERVER_NO_WHOLE=1 at creation turns both off.  Larger requests take a
+ * lane of their own, through the single calls.  Results are bit-identical to btas_gemm /
  * btas_apsp.  Buffers must stay valid until the request is done.
  *
  * btas_server_create      : budget in bytes (> 0); flags must be 0.  The

@@ -151,6 +151,7 @@ struct btas_server_t {
     double step_terms = 1.5e10;  // work cap of one step (terms), keeps steps short
     int allow_u16 = 1;         // BTAS_SERVER_NO_U16=1 keeps every squaring in int32
     int allow_whole = 1;       // BTAS_SERVER_NO_WHOLE=1 runs every APSP squaring by squaring
+    int allow_relax = 1;       // BTAS_SERVER_NO_RELAX=1: whole solves and squarings only
     double whole_below = 1.5e10;  // whole solves only when the other pending work is below this (terms)
     int64_t steps = 0;
     int64_t units = 0;
@@ -271,8 +272,8 @@ int launch_step(btas_server_t *sv, std::vector<Req *> &units) {
         r->whole = sv->allow_whole && r->kind == 0 && r->s == 1 && r->tile_next == 0 && r->n <= apsp_mid_max_n() &&
                    pending - r->unit_terms() < sv->whole_below && (r->n <= apsp_small_limit() || !bulk_busy);
         r->take = 0;
-        r->relax = sv->allow_whole && r->kind == 0 && r->s == 1 && r->tile_next == 0 && !r->no_relax && r->n >= 16 &&
-                   r->n <= kRelaxBatchMaxN;
+        r->relax = sv->allow_whole && sv->allow_relax && r->kind == 0 && r->s == 1 && r->tile_next == 0 &&
+                   !r->no_relax && r->n >= 16 && r->n <= kRelaxBatchMaxN;
         if (r->relax) {
             // its shared-memory work, as the terms a product computes meanwhile
             // (n = 1024: about 35 us of the whole GPU)
@@ -797,6 +798,7 @@ btas_status btas_server_create(btas_server_t **out, int64_t hbm_budget_bytes, in
     if (const char *e = getenv("BTAS_SERVER_STEP_TERMS")) sv->step_terms = atof(e) > 0 ? atof(e) : sv->step_terms;
     if (const char *e = getenv("BTAS_SERVER_NO_U16")) sv->allow_u16 = (*e && atoi(e) != 0) ? 0 : 1;
     if (const char *e = getenv("BTAS_SERVER_NO_WHOLE")) sv->allow_whole = (*e && atoi(e) != 0) ? 0 : 1;
+    if (const char *e = getenv("BTAS_SERVER_NO_RELAX")) sv->allow_relax = (*e && atoi(e) != 0) ? 0 : 1;
     if (const char *e = getenv("BTAS_SERVER_BULK_TERMS")) sv->bulk_terms = atof(e);
     sv->timeout_cycles = batch_timeout_cycles(sv->device);
     sv->flag_slots = 1 << 16;

@@ -1,0 +1,98 @@
+"""Served APSP beyond the relaxation: solves it gives up go on by squarings or as whole solves in buffers that its lists
+lay over, and with BTAS_SERVER_NO_RELAX=1 the one-block and the cooperative kernel solve from the start."""
+import contextlib
+import os
+
+import numpy as np
+import pytest
+
+import gen
+
+pytestmark = pytest.mark.gpu
+
+INF = 0x3FFFFFFF
+
+
+@pytest.fixture(scope="module")
+def btas():
+    import paper_1701_04733_gb300 as m
+    return m
+
+
+@contextlib.contextmanager
+def env(**kv):
+    os.environ.update(kv)
+    try:
+        yield
+    finally:
+        for k in kv:
+            del os.environ[k]
+
+
+def chain(n, w):
+    W = np.full((n, n), INF, np.int32)
+    np.fill_diagonal(W, 0)
+    W[np.arange(n - 1), np.arange(1, n)] = w
+    return W
+
+
+def graphs(heavy):
+    """Chains, which no relaxation without time finishes, in 16 and in 32 bits, and random graphs beside them."""
+    w = 40000 if heavy else 3
+    return [g for n in (16, 17, 33, 130, 300, 700)
+            for g in (chain(n, w), gen.random_graph(gen.BASE_SEED, 101 + n, n, 0.1 if n > 40 else 0.4, 1, 100 * w))]
+
+
+def serve(btas, Ws, together):
+    """The outputs, final states and number of steps; requests all at once or one after another."""
+    import torch
+    srv = btas.Server(8 << 30)
+    bufs = [(torch.from_numpy(W).pin_memory(), torch.full(W.shape, 77, dtype=torch.int32).pin_memory()) for W in Ws]
+    tickets = []
+    for W, D in bufs:
+        tickets.append(srv.submit_apsp(W, D))
+        if not together:
+            srv.wait_all(120)
+    srv.wait_all(300)
+    states = [srv.poll(t)["state"] for t in tickets]
+    stats = srv.stats()
+    srv.close()
+    assert stats["completed"] == len(Ws) and stats["bytes_in_use"] == 0
+    return [D.numpy() for _, D in bufs], states, stats["steps"]
+
+
+# one at a time: whole solves; together: a step takes a few tiles of one squaring
+MODES = {"alone": {}, "chunks": {"BTAS_SERVER_STEP_TERMS": "2e7"}}
+
+
+@pytest.mark.parametrize("heavy", [False, True])
+@pytest.mark.parametrize("mode", sorted(MODES))
+def test_given_up(btas, oracle_mod, mode, heavy):
+    Ws = graphs(heavy)
+    bad = graphs(heavy)[9].copy()
+    bad[5, 4] = -3
+    with env(**MODES[mode]):
+        _, _, steps0 = serve(btas, Ws + [bad], mode == "chunks")
+        with env(BTAS_RELAX_BUDGET="-1"):
+            outs, states, steps = serve(btas, Ws + [bad], mode == "chunks")
+    assert states == [2] * len(Ws) + [3]
+    assert (outs[-1] == 77).all()
+    for W, D in zip(Ws, outs):
+        np.testing.assert_array_equal(D, oracle_mod.floyd_warshall(W))
+    # a step at least for each of the four larger chains (the others may be done by the first look)
+    assert steps >= steps0 + (4 if mode == "alone" else 1)
+
+
+def test_whole_solves(btas, oracle_mod):
+    """The one-block kernel (n <= 64) and the cooperative kernel, each with its own domain check."""
+    Ws = graphs(False)
+    for n in (40, 300):
+        W = gen.random_graph(gen.BASE_SEED, 109 + n, n, 0.2, 1, 100)
+        W[n // 2, 1] = -1
+        Ws.append(W)
+    with env(BTAS_SERVER_NO_RELAX="1"):
+        outs, states, _ = serve(btas, Ws, False)
+    assert states == [2] * (len(Ws) - 2) + [3, 3]
+    for W, D in zip(Ws[:-2], outs):
+        np.testing.assert_array_equal(D, oracle_mod.floyd_warshall(W))
+    assert (outs[-1] == 77).all() and (outs[-2] == 77).all()
