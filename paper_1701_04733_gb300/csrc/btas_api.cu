@@ -248,12 +248,11 @@ struct NtPlan {
 // CTA alone reaches: 128 x 128 tiles at 2 CTAs/SM 66 (int32) and 62 (fp32), 59
 // where parts of a tile are merged, and 0.85; 64 x 64 with 128 threads 59 and
 // 55.5, merged 56.5 and 55, and 0.4; 32 x 32 46 and 40, merged 43 and 38, and
-// 0.25; 64 x 64 with 64 threads 45 and 0.2.
+// 0.25.  For the kernels that have a merging form.
 double nt_time(const GemmKernel &g, int dtype, double m, double n, double k, int splits, int sms) {
     const bool f32 = dtype == BTAS_F32, merged = splits > 1;
     double rate = merged ? 59 : f32 ? 62 : 66, alone = 0.85, resident = 2;
     if (g.bm < 64) rate = f32 ? (merged ? 38 : 40) : (merged ? 43 : 46), alone = 0.25, resident = 6;
-    else if (g.bm < 128 && g.threads < 128) rate = 45, alone = 0.2, resident = 3;
     else if (g.bm < 128) rate = f32 ? (merged ? 55 : 55.5) : (merged ? 56.5 : 59), alone = 0.4, resident = 4;
     const double per_sm = std::ceil(std::ceil(m / g.bm) * std::ceil(n / g.bn) * splits / sms);
     const double steps = std::ceil(std::ceil(k / 32) / splits);
