@@ -49,6 +49,8 @@ using relax::RowStats;
 
 constexpr int kListWarps = 8;               // rows of a block of the list kernel
 constexpr int kSolveSmem = 225 * 1024;       // most dynamic shared memory of the solve kernel
+constexpr int kTwoBlocksMaxN = 7000;         // 16 n bytes, twice, with what each block takes besides
+static_assert(2 * (16 * kTwoBlocksMaxN + 2048) <= 228 * 1024, "two blocks per SM");
 enum Ctl { kAbort = 0, kWide = 1, kDone = 2 };  // control words, cleared by the list kernel
 
 struct RelaxArgs {
@@ -272,11 +274,12 @@ cudaError_t launch_sparse_keys(const int *W, int n, void *ws, int shift, int *K,
     return cudaGetLastError();
 }
 
-// A block's patience in a call of its own, `resident` blocks running at once.
-// What a call takes where its relaxation is given up, in cycles (chains, GB300):
-// below n = 2048 the squarings, 68 us at n = 128, 148 at 512, 555 at 1024, 3280 at 2047
-// in 16 bits and 73, 180, 805, 5300 in 32; from there on blocked Floyd-Warshall,
-// 2.1 ms at n = 2048, 5.4 at 4096.
+// A block's patience in a call of its own: `blocks` with all targets, `resident`
+// of them at once; split: in 32 bits twice as many with half of them each, else one
+// half after the other.  What a call takes where its relaxation is given up, in
+// cycles (chains, GB300): below n = 2048 the squarings, 68 us at n = 128, 148 at 512,
+// 555 at 1024, 3280 at 2047 in 16 bits and 73, 180, 805, 5300 in 32; from there on
+// blocked Floyd-Warshall, 2.1 ms at n = 2048, 5.4 at 4096.
 static relax::Patience relax_patience(long long n, int blocks, int resident, bool split) {
     relax::Patience p{};
     if (const char *e = getenv("BTAS_RELAX_BUDGET"); e && *e) {
@@ -285,10 +288,12 @@ static relax::Patience relax_patience(long long n, int blocks, int resident, boo
     }
     p.by_share = true;
     p.cycles = relax::budget_cycles(n);
-    const double n3 = (double)n * n * n, share = std::min(1.0, (double)resident / blocks);
-    p.worth16 = (long long)(share * (n < 2048 ? 110e3 + 120.0 * n + n3 / 1500 : 1730.0 * n + n3 / 20000));
-    p.worth32 = (long long)(share * (n < 2048 ? 110e3 + 120.0 * n + n3 / 900 : 1730.0 * n + n3 / 20000));
-    if (!split) p.worth32 /= 2;  // one half of the targets after the other
+    const double n3 = (double)n * n * n, fw = 1730.0 * n + n3 / 20000;
+    const double worth16 = n < 2048 ? 110e3 + 120.0 * n + n3 / 1500 : fw;
+    const double worth32 = n < 2048 ? 110e3 + 120.0 * n + n3 / 900 : fw;
+    p.worth16 = (long long)(worth16 * std::min(1.0, (double)resident / blocks));
+    p.worth32 = (long long)(worth32 * (split ? std::min(1.0, 0.5 * resident / blocks)
+                                             : 0.5 * std::min(1.0, (double)resident / blocks)));
     return p;
 }
 
@@ -303,22 +308,25 @@ cudaError_t launch_relax(const int *W, long long ldw, int n, int *D, long long l
     a.ldd = ldd;
     a.out = out;
     place(ws, n, &a.ctl, &a.stats, &a.lists);
+    DeviceInfo di{};
+    const int sms = current_device_info(&di) ? di.sms : 152;
     // Two blocks share a block's targets in 32 bits while one wave holds them all (n =
     // 1024, w <= 10^6, p = 0.5: 283 -> 158 us per call).
-    a.halves = n <= 1216 ? 2 : 1;
+    a.halves = n <= 8 * sms ? 2 : 1;
     relax_lists_kernel<<<blocks, kListWarps * 32, 0, st>>>(a);
     note_launch();
     // Small graphs take fewer targets per block, so that more SMs share the
-    // sweeps' shared-memory loads: 2 up to n = 304 (46 -> 41 us per call at n = 256,
-    // p = 0.1) and 4 up to 608 (60 -> 55 us at n = 512); two lanes per vertex while
-    // one would leave warps idle.  From there on 8 targets, with 1024 threads where
-    // one block per SM holds all targets (n = 1024, p = 0.1: 93 us, 112 with 512
-    // threads) or fills shared memory (n = 8192: 3662 us against 3779), 512 and two
-    // blocks per SM between (n = 4096, p = 0.01: 1060 us against 1118).  Rows of 16 or
-    // 32 targets, which pay in the batched launch, lose more to their fewer blocks
-    // than they gain (n = 2048: 265 and 377 us against 249).
-    const int words = n <= 304 ? 1 : n <= 608 ? 2 : 4, lanes = n <= 304 ? 2 : 1;
-    const int maxt = (n > 608 && n <= 1216) || n > 7000 ? 1024 : 512;
+    // sweeps' shared-memory loads: 2 while that makes at most a block per SM (n <= 304
+    // on 152 SMs; 46 -> 41 us per call at n = 256, p = 0.1) and 4 likewise (n <= 608; 60
+    // -> 55 us at n = 512); two lanes per vertex while one would leave warps idle.
+    // From there on 8 targets, with 1024 threads where one block per SM holds all
+    // targets (n = 1024, p = 0.1: 93 us, 112 with 512 threads) or fills shared memory (n
+    // = 8192: 3662 us against 3779), 512 and two blocks per SM between (n = 4096, p =
+    // 0.01: 1060 us against 1118).  Rows of 16 or 32 targets, which pay in the batched
+    // launch, lose more to their fewer blocks than they gain (n = 2048: 265 and 377 us
+    // against 249).
+    const int words = n <= 2 * sms ? 1 : n <= 4 * sms ? 2 : 4, lanes = words == 1 ? 2 : 1;
+    const int maxt = (words == 4 && n <= 8 * sms) || n > kTwoBlocksMaxN ? 1024 : 512;
     void (*kern)(const RelaxArgs) = words == 1 ? relax_solve_kernel<2, 1, 512>
                                     : words == 2 ? relax_solve_kernel<1, 2, 512>
                                     : maxt == 512 ? relax_solve_kernel<1, 4, 512> : relax_solve_kernel<1, 4, 1024>;
@@ -334,9 +342,7 @@ cudaError_t launch_relax(const int *W, long long ldw, int n, int *D, long long l
     at.val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = &at;
     cfg.numAttrs = 1;
-    DeviceInfo di{};
-    a.lists.patience = relax_patience(n, cfg.gridDim.x, (maxt == 1024 ? 1 : 2) * (current_device_info(&di) ? di.sms : 152),
-                                      a.halves == 2);
+    a.lists.patience = relax_patience(n, cfg.gridDim.x / a.halves, (maxt == 1024 ? 1 : 2) * sms, a.halves == 2);
     e = cudaLaunchKernelEx(&cfg, kern, a);
     if (e == cudaSuccess) note_launch();
     return e;

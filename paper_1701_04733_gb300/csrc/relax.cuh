@@ -509,12 +509,11 @@ struct Looks {   // in shared memory, cleared by thread 0 before a solve's first
 
 // Whether the block's patience is at its end, asked after every 8 sweeps; valid in
 // thread 0.  t0, start: the clock when the solve and when the block began.
-// Called by the whole block, rarely: it stays out of the sweeps' registers.
+// Called by the whole block, rarely.
 template <bool U16, int R, int NV>
-__device__ __noinline__ bool late(const Patience &p, const Vec<NV> *Y, int n, int sweeps, long long t0,
+__device__ __forceinline__ bool late(const Patience &p, const Vec<NV> *Y, int n, int sweeps, long long t0,
                                   long long start, Looks &k) {
     if (sweeps > 8 && !k.finding) return threadIdx.x == 0 && clock64() - start > (U16 ? 1 : 2) * p.cycles;
-    if (threadIdx.x == 0) k.found = 0;
     int c = 0;
     for (int i = threadIdx.x; i < n * R; i += blockDim.x) {
         const Vec<NV> y = lds_relaxed(Y + i);
@@ -525,11 +524,11 @@ __device__ __noinline__ bool late(const Patience &p, const Vec<NV> *Y, int n, in
         }
     }
     c = __reduce_add_sync(0xffffffffu, c);
-    __syncthreads();
     if ((threadIdx.x & 31) == 0) atomicAdd(&k.found, c);
     __syncthreads();
     if (threadIdx.x != 0) return false;
     const float found = (float)k.found / ((float)n * (float)targets<U16, R, NV>());
+    k.found = 0;  // for the next look, some barriers from here
     if (sweeps == 8) k.finding = p.by_share && found < 0.9f;
     if (!k.finding) return clock64() - start > (U16 ? 1 : 2) * p.cycles;
     const float t = (float)(clock64() - t0), worth = (float)(U16 ? p.worth16 : p.worth32);
@@ -538,6 +537,15 @@ __device__ __noinline__ bool late(const Patience &p, const Vec<NV> *Y, int n, in
     k.last_t = t;
     if (found >= 0.9f) return t > 1.5f * worth;  // near its end: worth a little more
     return sweeps < kSettle ? t > worth : fminf(t / found, t + more) > worth;
+}
+
+// The same out of the sweeps' registers, for rows of 4 words (in line n = 1024 takes 1.3 %
+// longer and the batched launch loses 2 %; the smaller kernels lose as much to the
+// call).
+template <bool U16, int R, int NV>
+__device__ __noinline__ bool late_apart(const Patience &p, const Vec<NV> *Y, int n, int sweeps, long long t0,
+                                        long long start, Looks &k) {
+    return late<U16, R, NV>(p, Y, n, sweeps, t0, start, k);
 }
 
 // Sweeps over all vertices until Y is the closure's columns.  A sweep lowers
@@ -626,8 +634,10 @@ __device__ __forceinline__ bool solve(const int *W, long long ldw, int n, const 
             }
             if (!__syncthreads_or(ch || cut)) break;
             if ((sweeps & 7) == 0) {
-                const bool l8 = late<U16, R, NV>(l.patience, Y, n, sweeps, t0, start, looks);
-                if (__syncthreads_or(tid == 0 && give_up(l8))) return false;
+                bool at_end;
+                if constexpr (NV == 4) at_end = late_apart<U16, R, NV>(l.patience, Y, n, sweeps, t0, start, looks);
+                else at_end = late<U16, R, NV>(l.patience, Y, n, sweeps, t0, start, looks);
+                if (__syncthreads_or(tid == 0 && give_up(at_end))) return false;
             }
         }
         bool ch = false;
