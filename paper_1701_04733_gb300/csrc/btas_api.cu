@@ -1474,6 +1474,8 @@ btas_status btas_apsp_paths(int64_t n, const int32_t *W, int32_t *D, int32_t *Ne
         if (host[0] != 0) return fail(BTAS_ERR_ARG, "btas_apsp_paths: %d entries outside the domain", host[0]);
         mval = host[1];
         sparse = sparse_keys_pay(n, host[2]) && mval <= paths_key_max();
+        if (sparse)
+            log_event("apsp_paths n=%lld: first squaring over edge lists (rows of up to %d edges)", (long long)n, host[2]);
     } else {
         int host[2] = {0, 0};
         BTAS_CUDA(launch_apsp_scan(W, n, dflags + 2 * S + 1, st), "domain scan");

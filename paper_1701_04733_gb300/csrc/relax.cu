@@ -241,6 +241,15 @@ void place(void *ws, int n, int **ctl, RowStats **stats, Lists *lists) {
 
 size_t edge_lists_workspace(long long n) { return relax_workspace(n) + align256((size_t)n * 4); }
 
+// Most edges of a row with which the pairs of edges pay.  us per call, dense first
+// squaring / over the lists, all rows with n / 8, n / 7, n / 6 and n / 5 edges: n = 300
+// 284/270, 274/261, 278/270, 273/263; n = 600 410/385, 406/394, 410/403, 408/415; n =
+// 1000 725/708, 726/721, 726/761, 725/801; n = 2048 3492/3465, 4049/4192, 3490/3866,
+// 3487/4252; n = 3000 10009/9987, 11671/12095, 10019/11165.
+static int sparse_row(long long n) { return (int)std::max(1LL, std::min<long long>(relax::kCap, n / (n < 800 ? 6 : 8))); }
+
+bool sparse_keys_pay(long long n, int most_edges) { return most_edges <= sparse_row(n); }
+
 // A row too full or too heavy decides against sparse_keys_pay, so its list is
 // not sorted or stored: with every list built a whole call on n = 519, p = 0.35
 // took 9 us longer than with a plain scan of W (453 against 444), so it takes 6
@@ -253,15 +262,13 @@ cudaError_t launch_edge_lists(const int *W, int n, int max_weight, void *ws, int
     a.n = n;
     place(ws, n, &a.ctl, &a.stats, &a.lists);
     a.lists.len = reinterpret_cast<int *>(static_cast<char *>(ws) + relax_workspace(n));
-    a.lists.whole = std::max(1, std::min(relax::kCap, n / 6));
+    a.lists.whole = sparse_row(n);
     a.lists.top = max_weight;
     a.found = found;
     relax_lists_kernel<<<blocks, kListWarps * 32, 0, st>>>(a);
     note_launch();
     return cudaGetLastError();
 }
-
-bool sparse_keys_pay(long long n, int most_edges) { return most_edges <= relax::kCap && 6LL * most_edges <= n; }
 
 cudaError_t launch_sparse_keys(const int *W, int n, void *ws, int shift, int *K, cudaStream_t st) {
     Lists l{};
