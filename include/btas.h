@@ -700,9 +700,11 @@ btas_status btas_batch_select_tiles(btas_batch_t *b, void *stream, int *mode, do
  * relaxation as in btas_apsp, as tasks of the step's launch; a solve that is
  * given up goes on as above from the next step
  * (BTAS_SERVER_NO_RELAX=1 in the environment at creation: no relaxations).
- * Where the rest of the pending work is light, such a solve, or one of n < 16,
- * is done whole by the one-block or the cooperative kernel of btas_apsp
- * instead, launched in the step after the persistent kernel.
+ * Where the rest of the pending work is light, such a solve, one of n < 16, and
+ * one of n <= 640 (BTAS_SERVER_WHOLE_MAX_N at creation) while there are two of
+ * them at most, is done whole by the
+ * one-block or the cooperative kernel of btas_apsp instead, launched in the
+ * step after the persistent kernel.
  * BTAS_SERVER_NO_WHOLE=1 at creation turns both off.  Larger requests take a
  * lane of their own, through the single calls.  Results are bit-identical to btas_gemm /
  * btas_apsp.  Buffers must stay valid until the request is done.

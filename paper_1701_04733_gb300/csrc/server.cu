@@ -21,7 +21,8 @@
 //             sorted edge lists (relax.cuh) as tasks of the same launch; only
 //             one that the relaxation gives up goes on by squarings, or, with
 //             n <= 1792 and light other work, by the one-block or the
-//             cooperative kernel, launched after the persistent kernel;
+//             cooperative kernel, launched after the persistent kernel.  One
+//             or two small requests by themselves take those kernels at once;
 //   retire  - a product is finished after its step; an APSP solve after its
 //             last squaring or as soon as a squaring changed nothing (early
 //             exit, same result).  Its result is copied back on the copy
@@ -65,6 +66,14 @@ namespace {
 
 size_t a256(size_t v) { return (v + 255) & ~size_t(255); }
 long long r4(long long v) { return (v + 3) & ~3LL; }
+
+// Up to so many small APSP requests at once are solved whole and not by relaxation,
+// whose tasks leave most of the GPU idle then.  us from submission to result,
+// relaxation / whole: one of n = 16 85/73, 150 111/104, 300 157/117, 500 166/167, 600
+// 193/196, 700 214/236 (p = 0.1, w <= 100) and 92/77, 144/113, 225/127, 277/202, 333/268,
+// 334/326 (p = 0.5, w <= 10^6); two of n = 150 167/168 and 227/175, 500 270/285 and
+// 478/351, 700 341/404 and 586/578; three of n = 150 179/223 and 231/235.
+constexpr int kWholeCount = 2, kWholeMaxN = 640;  // BTAS_SERVER_WHOLE_MAX_N at creation: another size
 
 enum ReqState : int { kQueued = 0, kRunning = 1, kDone = 2, kFailed = 3 };
 
@@ -152,6 +161,7 @@ struct btas_server_t {
     int allow_u16 = 1;         // BTAS_SERVER_NO_U16=1 keeps every squaring in int32
     int allow_whole = 1;       // BTAS_SERVER_NO_WHOLE=1 runs every APSP squaring by squaring
     int allow_relax = 1;       // BTAS_SERVER_NO_RELAX=1: whole solves and squarings only
+    int whole_max_n = kWholeMaxN;
     double whole_below = 1.5e10;  // whole solves only when the other pending work is below this (terms)
     int64_t steps = 0;
     int64_t units = 0;
@@ -263,6 +273,12 @@ int launch_step(btas_server_t *sv, std::vector<Req *> &units) {
     }
     const double cap = sv->step_terms;
     const double small = 0.05 * cap;
+    auto relaxable = [&](const Req *r) {
+        return sv->allow_whole && sv->allow_relax && r->kind == 0 && r->s == 1 && r->tile_next == 0 && !r->no_relax &&
+               r->n >= 16 && r->n <= kRelaxBatchMaxN;
+    };
+    int relaxations = 0;
+    for (const Req *r : sv->active) relaxations += relaxable(r);
     for (Req *r : sv->active) {
         // an APSP request that fits the one-block or cooperative kernel is
         // solved whole, in one unit, instead of one squaring per step -- when
@@ -272,8 +288,7 @@ int launch_step(btas_server_t *sv, std::vector<Req *> &units) {
         r->whole = sv->allow_whole && r->kind == 0 && r->s == 1 && r->tile_next == 0 && r->n <= apsp_mid_max_n() &&
                    pending - r->unit_terms() < sv->whole_below && (r->n <= apsp_small_limit() || !bulk_busy);
         r->take = 0;
-        r->relax = sv->allow_whole && sv->allow_relax && r->kind == 0 && r->s == 1 && r->tile_next == 0 &&
-                   !r->no_relax && r->n >= 16 && r->n <= kRelaxBatchMaxN;
+        r->relax = relaxable(r) && !(r->whole && relaxations <= kWholeCount && r->n <= sv->whole_max_n);
         if (r->relax) {
             // its shared-memory work, as the terms a product computes meanwhile
             // (n = 1024: about 35 us of the whole GPU)
@@ -799,6 +814,7 @@ btas_status btas_server_create(btas_server_t **out, int64_t hbm_budget_bytes, in
     if (const char *e = getenv("BTAS_SERVER_NO_U16")) sv->allow_u16 = (*e && atoi(e) != 0) ? 0 : 1;
     if (const char *e = getenv("BTAS_SERVER_NO_WHOLE")) sv->allow_whole = (*e && atoi(e) != 0) ? 0 : 1;
     if (const char *e = getenv("BTAS_SERVER_NO_RELAX")) sv->allow_relax = (*e && atoi(e) != 0) ? 0 : 1;
+    if (const char *e = getenv("BTAS_SERVER_WHOLE_MAX_N")) sv->whole_max_n = *e ? atoi(e) : kWholeMaxN;
     if (const char *e = getenv("BTAS_SERVER_BULK_TERMS")) sv->bulk_terms = atof(e);
     sv->timeout_cycles = batch_timeout_cycles(sv->device);
     sv->flag_slots = 1 << 16;

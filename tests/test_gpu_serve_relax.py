@@ -61,8 +61,9 @@ def serve(btas, Ws, together):
     return [D.numpy() for _, D in bufs], states, stats["steps"]
 
 
-# one at a time: whole solves; together: a step takes a few tiles of one squaring
-MODES = {"alone": {}, "chunks": {"BTAS_SERVER_STEP_TERMS": "2e7"}}
+# one at a time: whole solves once the relaxation is given up; together: a step takes a few tiles of one squaring
+MODES = {"alone": {"BTAS_SERVER_WHOLE_MAX_N": "0"}, "chunks": {"BTAS_SERVER_STEP_TERMS": "2e7",
+                                                               "BTAS_SERVER_WHOLE_MAX_N": "0"}}
 
 
 @pytest.mark.parametrize("heavy", [False, True])
@@ -96,3 +97,29 @@ def test_whole_solves(btas, oracle_mod):
     for W, D in zip(Ws[:-2], outs):
         np.testing.assert_array_equal(D, oracle_mod.floyd_warshall(W))
     assert (outs[-1] == 77).all() and (outs[-2] == 77).all()
+
+
+@pytest.mark.parametrize("n", [16, 150, 300])
+def test_small_requests_alone_take_the_faster_kernels(btas, n):
+    """The fastest of 60 requests, one after another, against a server without relaxations; these took 1.15 to 1.35 times
+    as long."""
+    import time
+
+    import torch
+    W = torch.from_numpy(gen.random_graph(gen.BASE_SEED, 113 + n, n, 0.1 if n > 40 else 0.5, 1, 100)).pin_memory()
+    D = torch.empty_like(W).pin_memory()
+
+    def fastest():
+        srv, times = btas.Server(1 << 30), []
+        for _ in range(60):
+            t = time.perf_counter()
+            srv.submit_apsp(W, D)
+            srv.wait_all(60)
+            times.append(time.perf_counter() - t)
+        srv.close()
+        return min(times)
+
+    fastest()
+    with env(BTAS_SERVER_NO_RELAX="1"):
+        whole = min(fastest(), fastest())
+    assert min(fastest(), fastest()) < 1.1 * whole
