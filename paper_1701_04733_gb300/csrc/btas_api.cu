@@ -1479,14 +1479,15 @@ btas_status btas_apsp_paths(int64_t n, const int32_t *W, int32_t *D, int32_t *Ne
     void *lists = list_room ? reinterpret_cast<char *>(Ak) + ak_bytes : nullptr;
     bool sparse = false;
     if (lists) {
-        int host[3] = {0, 0, 0};
+        int host[4] = {0, 0, 0, 0};
         BTAS_CUDA(launch_edge_lists(W, (int)n, paths_key_max(), lists, dflags + 2 * S, st), "edge lists");
-        BTAS_CUDA(read_back(host, dflags + 2 * S, 12, st), "lists readback");
+        BTAS_CUDA(read_back(host, dflags + 2 * S, 16, st), "lists readback");
         if (host[0] != 0) return fail(BTAS_ERR_ARG, "btas_apsp_paths: %d entries outside the domain", host[0]);
         mval = host[1];
-        sparse = sparse_keys_pay(n, host[2]) && mval <= paths_key_max();
+        sparse = sparse_keys_pay(n, host[2], host[3]) && mval <= paths_key_max();
         if (sparse)
-            log_event("apsp_paths n=%lld: first squaring over edge lists (rows of up to %d edges)", (long long)n, host[2]);
+            log_event("apsp_paths n=%lld: first squaring over edge lists (%d edges, rows of up to %d)", (long long)n,
+                      host[3], host[2]);
     } else {
         int host[2] = {0, 0};
         BTAS_CUDA(launch_apsp_scan(W, n, dflags + 2 * S + 1, st), "domain scan");

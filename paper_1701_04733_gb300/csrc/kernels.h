@@ -198,16 +198,16 @@ size_t relax_workspace(long long n);
 int relax_max_n();
 cudaError_t launch_relax(const int *W, long long ldw, int n, int *D, long long ldd, void *ws, int *out,
                          cudaStream_t st);
-// The edge lists alone (ws: edge_lists_workspace(n) bytes), and in found (device, 3
+// The edge lists alone (ws: edge_lists_workspace(n) bytes), and in found (device, 4
 // ints, zero before): entries of W outside the domain, the largest weight, the most
-// edges of a row (INT_MAX if some list does not hold its row: it has more edges than
-// sparse_keys_pay accepts or one heavier than max_weight).  launch_sparse_keys then
-// writes the first squaring's keys (value << shift) | smallest minimising k, or INF,
-// to K (n x n, n <= 8192) from them; it needs every edge in the lists, and pays from
-// sparse_keys_pay on.
+// edges of a row (INT_MAX if some list does not hold its row: it has more than n / 6
+// or 512 edges or one heavier than max_weight) and the edges of all rows.
+// launch_sparse_keys then writes the first squaring's keys (value << shift) |
+// smallest minimising k, or INF, to K (n x n, n <= 8192) from them; it needs every
+// edge in the lists, and is the faster way where sparse_keys_pay says so.
 size_t edge_lists_workspace(long long n);
 cudaError_t launch_edge_lists(const int *W, int n, int max_weight, void *ws, int *found, cudaStream_t st);
-bool sparse_keys_pay(long long n, int most_edges);
+bool sparse_keys_pay(long long n, int most_edges, int edges);
 cudaError_t launch_sparse_keys(const int *W, int n, void *ws, int shift, int *K, cudaStream_t st);
 
 // ---- blocked Floyd-Warshall (fw.cu): phases 1 and 2 of pivot block kb

@@ -63,8 +63,8 @@ struct RelaxArgs {
     int *D;
     long long ldd;
     int *out;  // host-mapped words (see kernels.h)
-    int *found;  // optional: three words, zero before, to take entries outside the domain, the largest
-                 // weight and the most edges of a row (INT_MAX: some list does not hold its row); then no stats
+    int *found;  // optional: four words, zero before, to take entries outside the domain, the largest weight, the
+                 // most edges of a row (INT_MAX: some list does not hold its row) and all edges; then no stats
     int halves;  // 2: a second block takes half of each block's targets where 32 bits are needed from the start
 };
 
@@ -90,11 +90,13 @@ __global__ void __launch_bounds__(kListWarps * 32) relax_lists_kernel(const Rela
             st.far |= o.far;
             st.light += o.light;
             st.cut |= o.cut;
+            st.edges += o.edges;
         }
         if (a.found != nullptr) {
             if (st.bad) atomicAdd(a.found, st.bad);
             atomicMax(a.found + 1, st.maxw);
             atomicMax(a.found + 2, st.cut ? 0x7FFFFFFF : st.deg);
+            atomicAdd(a.found + 3, st.edges);
         } else {
             a.stats[blockIdx.x] = st;
         }
@@ -241,14 +243,17 @@ void place(void *ws, int n, int **ctl, RowStats **stats, Lists *lists) {
 
 size_t edge_lists_workspace(long long n) { return relax_workspace(n) + align256((size_t)n * 4); }
 
-// Most edges of a row with which the pairs of edges pay.  us per call, dense first
-// squaring / over the lists, all rows with n / 8, n / 7, n / 6 and n / 5 edges: n = 300
-// 284/270, 274/261, 278/270, 273/263; n = 600 410/385, 406/394, 410/403, 408/415; n =
+// The most edges that a row's list is kept for, and the most edges of all with
+// which the pairs of edges (all d^2 of a row, on average) pay.  us per call, dense
+// first squaring / over the lists, all rows with n / 8, n / 7, n / 6 and n / 5 edges: n =
+// 300 284/270, 274/261, 278/270, 273/263; n = 600 410/385, 406/394, 410/403, 408/415; n =
 // 1000 725/708, 726/721, 726/761, 725/801; n = 2048 3492/3465, 4049/4192, 3490/3866,
 // 3487/4252; n = 3000 10009/9987, 11671/12095, 10019/11165.
-static int sparse_row(long long n) { return (int)std::max(1LL, std::min<long long>(relax::kCap, n / (n < 800 ? 6 : 8))); }
+static int sparse_row(long long n) { return (int)std::max(1LL, std::min<long long>(relax::kCap, n / 6)); }
 
-bool sparse_keys_pay(long long n, int most_edges) { return most_edges <= sparse_row(n); }
+bool sparse_keys_pay(long long n, int most_edges, int edges) {
+    return most_edges <= sparse_row(n) && (n < 800 || 8LL * edges <= n * n);
+}
 
 // A row too full or too heavy decides against sparse_keys_pay, so its list is
 // not sorted or stored: with every list built a whole call on n = 519, p = 0.35

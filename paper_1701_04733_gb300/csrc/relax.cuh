@@ -66,6 +66,7 @@ struct RowStats {
     int far;    // 1: some row's lightest edge does not fit 16 bits
     float light;  // sum of the rows' lightest weights
     int cut;      // 1: some list holds less than its row
+    int edges;    // of all rows
 };
 
 // Clock cycles a block of 8 targets is worth: about twice what the slowest
@@ -327,6 +328,7 @@ __device__ __forceinline__ RowStats build_row(const int *W, long long ldw, int n
         st.minw = mn;
         st.deg = deg;
         st.cut = 1;
+        st.edges = deg;
         return st;
     }
     if (cnt > cap || (cnt < deg && cnt < 64)) {
@@ -352,6 +354,7 @@ __device__ __forceinline__ RowStats build_row(const int *W, long long ldw, int n
     st.far = deg > 0 && mn >= BTAS_INF_U16;
     st.light = deg > 0 ? (float)mn : 0.0f;
     st.cut = cnt < deg;
+    st.edges = deg;
     return st;
 }
 
