@@ -306,7 +306,7 @@ __device__ __noinline__ void relax_task(const BInst &I, int t, unsigned char *sm
     if (!wide) {
         relax::load_columns<true, R, 4>(W, I.lda, n, Y, j0);
         __syncthreads();
-        if (!relax::solve<true, 1, R, 4>(W, I.lda, n, I.rl, Y, minw, t0, give_up)) return;
+        if (!relax::solve<true, 1, R, 4>(W, I.lda, n, I.rl, Y, minw, maxw, t0, give_up)) return;
         wide = !relax::fits16<R, 4>(Y, n, maxw);
         if (!wide) relax::store_columns<true, R, 4>(D, I.ldc, n, Y, j0);
         else if (tid == 0) atomicOr(I.rstat + kRelaxWide, 1);
@@ -316,7 +316,7 @@ __device__ __noinline__ void relax_task(const BInst &I, int t, unsigned char *sm
             __syncthreads();
             relax::load_columns<false, R, 4>(W, I.lda, n, Y, j0 + h);
             __syncthreads();
-            if (!relax::solve<false, 1, R, 4>(W, I.lda, n, I.rl, Y, minw, t0, give_up)) return;
+            if (!relax::solve<false, 1, R, 4>(W, I.lda, n, I.rl, Y, minw, maxw, t0, give_up)) return;
             relax::store_columns<false, R, 4>(D, I.ldc, n, Y, j0 + h);
         }
     }

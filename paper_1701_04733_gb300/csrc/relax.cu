@@ -151,7 +151,7 @@ __global__ void __launch_bounds__(MAXT) relax_solve_kernel(const RelaxArgs a) {
             if (late) a.ctl[kAbort] = 1;
             return late;
         };
-        if (part == 0 && !wide && relax::solve<true, G, R, NV>(a.W, a.ldw, n, a.lists, Y, st.minw, t0, give_up)) {
+        if (part == 0 && !wide && relax::solve<true, G, R, NV>(a.W, a.ldw, n, a.lists, Y, st.minw, st.maxw, t0, give_up)) {
             wide = !relax::fits16<R, NV>(Y, n, st.maxw);
             if (!wide) relax::store_columns<true, R, NV>(a.D, a.ldd, n, Y, j0);
             else if (tid == 0) a.ctl[kWide] = 1;
@@ -163,7 +163,7 @@ __global__ void __launch_bounds__(MAXT) relax_solve_kernel(const RelaxArgs a) {
                 __syncthreads();
                 relax::load_columns<false, R, NV>(a.W, a.ldw, n, Y, j0 + h);
                 __syncthreads();
-                if (!relax::solve<false, G, R, NV>(a.W, a.ldw, n, a.lists, Y, st.minw, t0, give_up)) break;
+                if (!relax::solve<false, G, R, NV>(a.W, a.ldw, n, a.lists, Y, st.minw, st.maxw, t0, give_up)) break;
                 relax::store_columns<false, R, NV>(a.D, a.ldd, n, Y, j0 + h);
             }
         }

@@ -34,8 +34,10 @@ constexpr int kSample = 1024;      // entries the first guess of a long row's cu
 // - Distances are still missing after 8 sweeps (chains, rings, grids, lattices,
 //   and the sparsest random graphs).  They are found at an even pace or a growing
 //   one until all are, so the share found, or what the last 8 sweeps added to it,
-//   says what the solve will take.  From kSettle sweeps on it goes on while that
-//   is less than what solving otherwise is worth.
+//   says how long that still takes.  From kSettle sweeps on the solve goes on while
+//   that is less than what solving otherwise is worth, up to twice its worth; up to
+//   `cycles` in 16 bits that do not hold all weights, where a longer edge counts as
+//   missing.
 // - All are known by then and some still improve: nothing tells for how long,
 //   and `cycles` end it.
 struct Patience {
@@ -504,19 +506,27 @@ __device__ __forceinline__ void store_columns(int *D, long long ldd, int n, cons
     }
 }
 
-struct Looks {   // in shared memory, cleared by thread 0 before a solve's first sweep
-    int found;     // entries
-    bool finding;  // distances were missing after 8 sweeps
+struct Looks {  // in shared memory, set by thread 0 before a solve's first sweep
+    int found;    // entries
     float last_found, last_t;
 };
 
-// Whether the block's patience is at its end, asked after every 8 sweeps; valid in
-// thread 0.  t0, start: the clock when the solve and when the block began.
-// Called by the whole block, rarely.
+// Whether a tenth of the vertices still misses a path to some target; the same in every
+// thread.  Called by the whole block.
 template <bool U16, int R, int NV>
-__device__ __forceinline__ bool late(const Patience &p, const Vec<NV> *Y, int n, int sweeps, long long t0,
-                                  long long start, Looks &k) {
-    if (sweeps > 8 && !k.finding) return threadIdx.x == 0 && clock64() - start > (U16 ? 1 : 2) * p.cycles;
+__device__ __forceinline__ bool some_missing(const Vec<NV> *Y, int n) {
+    const int rows = n * R, looked = min(rows, (int)blockDim.x);
+    const int i = rows > looked ? (int)((long long)threadIdx.x * rows / looked) : threadIdx.x;
+    const bool missing = i < rows && top<U16, NV>(lds_relaxed(Y + i)) >= (U16 ? BTAS_INF_U16 : kInfI32);
+    return 10 * __syncthreads_count(missing) > looked;
+}
+
+// Whether the patience of a block with distances missing is at its end, asked after
+// every 8 sweeps from 16 on; valid in thread 0.  t0: the clock when the solve began.
+// Called by the whole block; random graphs do not get here, whose smallest batches would
+// pay for fetching these instructions (32 graphs of n = 128: 10 of 90 us).
+template <bool U16, int R, int NV>
+__device__ __forceinline__ bool late(const Patience &p, const Vec<NV> *Y, int n, int sweeps, long long t0, Looks &k) {
     int c = 0;
     for (int i = threadIdx.x; i < n * R; i += blockDim.x) {
         const Vec<NV> y = lds_relaxed(Y + i);
@@ -532,23 +542,21 @@ __device__ __forceinline__ bool late(const Patience &p, const Vec<NV> *Y, int n,
     if (threadIdx.x != 0) return false;
     const float found = (float)k.found / ((float)n * (float)targets<U16, R, NV>());
     k.found = 0;  // for the next look, some barriers from here
-    if (sweeps == 8) k.finding = p.by_share && found < 0.9f;
-    if (!k.finding) return clock64() - start > (U16 ? 1 : 2) * p.cycles;
     const float t = (float)(clock64() - t0), worth = (float)(U16 ? p.worth16 : p.worth32);
     const float more = (1.0f - found) * (t - k.last_t) / fmaxf(found - k.last_found, 1e-6f);
     k.last_found = found;
     k.last_t = t;
-    if (found >= 0.9f) return t > 1.5f * worth;  // near its end: worth a little more
-    return sweeps < kSettle ? t > worth : fminf(t / found, t + more) > worth;
+    if (found >= 0.9f) return t > 1.5f * worth;  // near its end
+    return sweeps < kSettle ? t > worth : t > 2.0f * worth || fminf(t / found - t, more) > worth;
 }
 
-// The same out of the sweeps' registers, for rows of 4 words (in line n = 1024 takes 1.3 %
-// longer and the batched launch loses 2 %; the smaller kernels lose as much to the
-// call).
+// The same out of the way of the sweeps' registers, for rows of 4 words.  Smaller rows
+// take it in line: a kernel without calls needs no stack, and small graphs show it (n =
+// 49 ... 304: 1 to 2 %).
 template <bool U16, int R, int NV>
 __device__ __noinline__ bool late_apart(const Patience &p, const Vec<NV> *Y, int n, int sweeps, long long t0,
-                                        long long start, Looks &k) {
-    return late<U16, R, NV>(p, Y, n, sweeps, t0, start, k);
+                                        Looks &k) {
+    return late<U16, R, NV>(p, Y, n, sweeps, t0, k);
 }
 
 // Sweeps over all vertices until Y is the closure's columns.  A sweep lowers
@@ -565,7 +573,7 @@ __device__ __noinline__ bool late_apart(const Patience &p, const Vec<NV> *Y, int
 // is at its end; returns false if it said so.  start: the clock when the block
 // began, earlier solves included.  Called by the whole block.
 template <bool U16, int G, int R, int NV, class GiveUp>
-__device__ __forceinline__ bool solve(const int *W, long long ldw, int n, const Lists &l, Vec<NV> *Y, int minw,
+__device__ __forceinline__ bool solve(const int *W, long long ldw, int n, const Lists &l, Vec<NV> *Y, int minw, int maxw,
                                       long long start, GiveUp give_up) {
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, nwarps = blockDim.x >> 5;
     constexpr int VW = 32 / (G * R);  // vertices of a warp
@@ -575,7 +583,11 @@ __device__ __forceinline__ bool solve(const int *W, long long ldw, int n, const 
     int sweeps = 0;
     const long long t0 = clock64();
     __shared__ Looks looks;
-    if (tid == 0) looks = Looks{0, false, 0.0f, 0.0f};
+    if (tid == 0) looks = Looks{0, 0.0f, 0.0f};
+    // the same in every thread: distances were missing after 8 sweeps, and the budget
+    // of cycles does not hold then, unless 16 bits are too few for some weight
+    bool finding = false;
+    const bool heavy = U16 && maxw >= BTAS_INF_U16;
     for (;;) {
         for (;;) {
             bool ch = false, cut = false;
@@ -637,9 +649,12 @@ __device__ __forceinline__ bool solve(const int *W, long long ldw, int n, const 
             }
             if (!__syncthreads_or(ch || cut)) break;
             if ((sweeps & 7) == 0) {
-                bool at_end;
-                if constexpr (NV == 4) at_end = late_apart<U16, R, NV>(l.patience, Y, n, sweeps, t0, start, looks);
-                else at_end = late<U16, R, NV>(l.patience, Y, n, sweeps, t0, start, looks);
+                if (sweeps == 8) finding = l.patience.by_share && some_missing<U16, R, NV>(Y, n);
+                bool at_end = (!finding || heavy) && clock64() - start > (U16 ? 1 : 2) * l.patience.cycles;
+                if (finding && sweeps > 8) {
+                    if constexpr (NV == 4) at_end |= late_apart<U16, R, NV>(l.patience, Y, n, sweeps, t0, looks);
+                    else at_end |= late<U16, R, NV>(l.patience, Y, n, sweeps, t0, looks);
+                }
                 if (__syncthreads_or(tid == 0 && give_up(at_end))) return false;
             }
         }
