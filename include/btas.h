@@ -239,11 +239,11 @@ btas_status btas_gemv(int semiring, int dtype, int trans, int64_t m, int64_t n, 
  * receives the number of products that changed d.  All products run in one
  * cooperative launch with one bounded grid barrier each (BTAS_ERR_TIMEOUT if
  * a wait expires; the first pass over W also checks the domain and builds
- * edge lists, up to n n bytes of scratch; later products relax the vertices
- * that the one before lowered), and the call
- * synchronises `stream` once.  Where a cooperative launch is refused (or
- * with BTAS_SSSP_NO_COOP=1 in the environment) it launches the products in
- * gated groups of 8 and synchronises once per group. */
+ * edge lists, 8 n min(1024, max(64, n / 8)) bytes of scratch; later products
+ * relax the vertices that the one before lowered), and the call synchronises
+ * `stream` once.  Where a cooperative launch is refused, the scratch cannot be
+ * had, or BTAS_SSSP_NO_COOP=1 is in the environment, it launches the products
+ * in gated groups of 8 and synchronises once per group. */
 btas_status btas_sssp(int64_t n, const int32_t *W, int64_t src, int32_t *dist, int *iterations, void *stream);
 
 /* ------------------------------------------------------------------------
@@ -283,19 +283,28 @@ btas_status btas_mul(int semiring, int dtype, int64_t n, const void *x, const vo
  *     the algorithm for non-negative edge weights).
  * D : n x n int32 output; D == W (in place) is allowed, any other overlap is
  *     not.
- * btas_apsp checks the domain on the device (one synchronisation of
- * `stream`; BTAS_ERR_ARG if violated).  It asks for the distances alone, and so
- * does btas_apsp_ex with flags == BTAS_APSP_EARLY_EXIT and no out-parameter: from
- * n = 49 up to 14400 such a call relaxes W's edges, sorted by weight, until
- * nothing changes, 8 targets per block (every block works on its own, so no
- * squaring is computed); blocks that run far longer than random graphs take
- * (paths of very many edges) give up.  The same D then comes from the squarings
- * below n = 2048 and from blocked Floyd-Warshall from there on, which also takes
- * n > 14400.  Scratch for the relaxation: about 8 n min(n, 512) bytes, and n * n
- * words more in place (D == W).  Other calls, and all of them while the
- * environment sets any BTAS_APSP_* or BTAS_MID_* switch (BTAS_APSP_NO_RELAX=1 does
- * nothing else), run the squarings, with the early exit and the exact
- * representation per squaring as btas_apsp_ex describes.
+ * btas_apsp checks the domain on the device (BTAS_ERR_ARG if violated).  It
+ * asks for the distances alone, and so does btas_apsp_ex with flags ==
+ * BTAS_APSP_EARLY_EXIT and no out-parameter: from n = 49 up to 14400 such a
+ * call relaxes W's edges, sorted by weight, until nothing changes, 2, 4 or 8
+ * targets per block (every block works on its own, so no squaring is
+ * computed).  A solve whose shortest paths have so many edges that the
+ * relaxation would take longer than what replaces it is given up; the same D
+ * then comes from the squarings below n = 2048 and from blocked
+ * Floyd-Warshall from there on, which also takes n > 14400.  Scratch for the
+ * relaxation: about 8 n min(n, 512) bytes, and n * n words more in place (D
+ * == W); where it cannot be had the call goes on as if given up.  Other calls,
+ * and all of them while the environment sets any BTAS_APSP_* or BTAS_MID_*
+ * switch (BTAS_APSP_NO_RELAX=1 does nothing else), run the squarings, with the
+ * early exit and the exact representation per squaring as btas_apsp_ex
+ * describes.
+ * The call waits until the outcome of the domain check is known, not until
+ * `stream` is idle: D is ready for later work on `stream`, and for anything
+ * else once `stream` has been synchronised.  (Floyd-Warshall and the tiled
+ * squarings leave work queued behind the check; the relaxation returns when
+ * its last block has reported to the host, a few microseconds before the
+ * stream is idle.  An asynchronous error of that work shows at the next
+ * synchronisation.)
  *
  * Execution of the squarings by size (same results and the same squarings
  * count in every regime; FORCE_U16 / FORCE_CARRIER always take the tiled path):
@@ -603,7 +612,9 @@ int btas_tune_entries(void);
  *                      one of BTAS_BATCH_TILE, _NO_U16, _NO_CERT, _CERT_MIN_N or
  *                      _NO_RELAX in the environment.
  *                      The domain (zero diagonal, weights in [0, 2^28] or
- *                      INF) is assumed, not checked.
+ *                      INF) is assumed, not checked: a W outside it gets
+ *                      whatever the squarings make of it.  The relaxation's
+ *                      lists lie in the space of the squarings' buffers.
  * btas_batch_add_gemm: C = A (x) B as btas_gemm (int32 or fp32, min-plus or
  *                      max-plus, optional BTAS_GEMM_TRANS_B; m, n, k >= 1).
  * btas_batch_launch  : enqueues the whole batch on `stream`.  The first

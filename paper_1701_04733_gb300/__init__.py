@@ -509,9 +509,10 @@ def sync_status(stream=None):
 
 
 def apsp(W, out=None, flags=APSP_EARLY_EXIT, stream=None, info=False):
-    """All-pairs shortest paths of the int32 adjacency matrix W by repeated
-    min-plus squaring (Sec. III).  out may be W (in place).  With info=True
-    returns (D, {"squarings": ..., "bound": ..., "path": ...})."""
+    """All-pairs shortest paths of the int32 adjacency matrix W.  out may be W
+    (in place).  A plain call relaxes W's edges (see btas_apsp in btas.h).  With
+    info=True, which returns (D, {"squarings": ..., "bound": ..., "path": ...}),
+    or other flags the same D comes from repeated min-plus squaring (Sec. III)."""
     torch = _torch()
     n = W.shape[0]
     if W.shape != (n, n) or not W.is_contiguous() or W.dtype != torch.int32:

@@ -189,10 +189,9 @@ cudaError_t launch_apsp_mid(const int *W, long long ldw, int n, int S, bool earl
 // relax_workspace(n) bytes, not initialised.  out: 4 host-mapped words, written
 // as the solve ends: [0] a RelaxOutcome, [1] entries of W outside the domain (D
 // is then not written), [2] most edges of a row, [3] whether 32 bits were
-// needed.  kRelaxGaveUp: some block ran longer than the budget that such
-// graphs are worth (paths of very many edges, or long rows of equal weights);
-// some columns of D may be written.  BTAS_RELAX_BUDGET=cycles overrides the
-// budget (tests).
+// needed.  kRelaxGaveUp: some block's patience came to its end (relax.cuh: paths of
+// very many edges, or long rows of equal weights); some columns of D may be
+// written.  BTAS_RELAX_BUDGET=cycles puts a budget in its place (tests).
 enum RelaxOutcome { kRelaxDone = 1, kRelaxBad = 2, kRelaxGaveUp = 3 };
 size_t relax_workspace(long long n);
 int relax_max_n();

@@ -6,6 +6,7 @@
 // over W's edges computes far fewer, and every block can solve a few targets by
 // itself, without a grid barrier: 16 bytes per vertex hold the distances to 8
 // targets in 16 bits (or 4 in 32), which fits shared memory up to n = 14400.
+// (Smaller graphs take 2 or 4 targets per block: launch_relax.)
 // One edge is then one 16-byte load and 4 DPX add-mins for 8 terms.
 //
 // What makes it short is the order of the edges.  Each row's list is sorted by
@@ -21,17 +22,17 @@
 // Sums of non-negative weights reach one fixpoint in any order, so the result is
 // that of the squarings bit for bit; only the number of squarings is not known.
 //
-// Measured (GB300, us per call with its synchronisation, before -> after):
-//   n = 128 (complete), 256 (p = 0.1):              60 -> 41, 60 -> 48
-//   n = 512, 1024 (p = 0.1, w <= 100):              98 -> 65, 288 -> 100
-//   n = 2048 (p = 0.1 / complete, w <= 10^6):       1416 -> 193 / 3279 -> 280
-//   n = 2999 (p = 0.5, w <= 10^6):                  10400 -> 555
-//   n = 4096 (p = 0.05, w <= 7 / p = 0.01, w <= 10^6): 6260 -> 610 / 16700 -> 1610
-//   n = 8192 (p = 0.01, w <= 1000 / complete, w <= 100): 93600 -> 3320 / 47000 -> 4020
-// The sweeps are bound by shared memory: ncu at n = 4096 (p = 0.01) has the
-// L1/shared pipe 92 % busy while SMs are active, 43 % of its cycles bank
-// conflicts of the random 16-byte rows (8 lanes on 8 bank groups).  Wider rows
-// conflict less but do not fit; ordering a chunk's 4 edges by bank gains 5 %.
+// Measured (GB300, us per call with its synchronisation, squarings -> relaxation):
+//   n = 128 (complete), 256 (p = 0.1):              51 -> 34, 59 -> 39
+//   n = 512, 1024 (p = 0.1, w <= 100):              94 -> 63, 290 -> 89
+//   n = 2048 (p = 0.1 / complete, w <= 10^6):       1668 -> 187 / 3278 -> 250
+//   n = 2999 (p = 0.5, w <= 10^6):                  11060 -> 570
+//   n = 4096 (p = 0.05, w <= 7 / p = 0.01, w <= 10^6): 5840 -> 608 / 16790 -> 1514
+//   n = 8192 (p = 0.01, w <= 1000 / complete, w <= 100): 93670 -> 3450 / 47010 -> 4045
+// The sweeps are bound by shared memory: ncu at n = 4096 (p = 0.05, w <= 7) has the L1
+// pipe 89 % busy while SMs are active, 35 % of its wavefronts bank conflicts of the
+// random 16-byte rows (8 lanes on 8 bank groups).  Wider rows conflict less but do not
+// fit; ordering a chunk's 4 edges by bank gains 5 %.
 // The last wave costs 15-30 % where n / 8 blocks are few per SM.
 #include <algorithm>
 #include <cstdlib>
@@ -336,7 +337,8 @@ cudaError_t launch_relax(const int *W, long long ldw, int n, int *D, long long l
     // = 8192: 3662 us against 3779), 512 and two blocks per SM between (n = 4096, p =
     // 0.01: 1060 us against 1118).  Rows of 16 or 32 targets, which pay in the batched
     // launch, lose more to their fewer blocks than they gain (n = 2048: 265 and 377 us
-    // against 249).
+    // against 249).  (These figures compare the shapes; the calls were 4 to 40 us longer
+    // then than above.)
     const int words = n <= 2 * sms ? 1 : n <= 4 * sms ? 2 : 4, lanes = words == 1 ? 2 : 1;
     const int maxt = (words == 4 && n <= 8 * sms) || n > kTwoBlocksMaxN ? 1024 : 512;
     void (*kern)(const RelaxArgs) = words == 1 ? relax_solve_kernel<2, 1, 512>
