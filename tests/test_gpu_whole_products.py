@@ -21,7 +21,7 @@ def btas():
 @pytest.mark.parametrize("dt", ["i32", "f32"])
 @pytest.mark.parametrize("m,n,k", SIZES)
 def test_choice_of_tiles(btas, dt, m, n, k):
-    """Each side is the fastest of 6 rounds of 10 calls; the model's own error over 46 shapes is 5 %, and the choice was
+    """Each side is the fastest of 6 rounds of 10 calls; the model's own error over 44 shapes is 5 %, and the choice was
     1.2 to 1.6 times the best at the first three sizes."""
     import torch
     if dt == "i32":
